@@ -63,13 +63,42 @@ __device__ __forceinline__ bool load_item(const AttnParams& p, int idx, ItemGeom
   return g.n > 0;
 }
 
+// Work item records in shared memory: 4 words of the item, 16 of the unit, 1 = there is one.
+constexpr int kItemWords = 24;
+// One warp copies item idx and its unit there (or the end mark).
+__device__ __forceinline__ void publish_item(const AttnParams& p, int idx, bool more, int* dst, int lane) {
+  int v = 0;
+  if (more) {
+    const int* it = reinterpret_cast<const int*>(&p.items[idx]);
+    const int* un = reinterpret_cast<const int*>(&p.units[it[0]]);
+    v = lane < 4 ? it[lane] : lane < 20 ? un[lane - 4] : 1;
+  }
+  if (lane < 21) dst[lane] = v;
+  __syncwarp();
+}
+// Returns false at the end mark.  g.n <= 0: an item without visible keys.
+__device__ __forceinline__ bool load_item(const int* src, ItemGeom& g) {
+  const int4* v = reinterpret_cast<const int4*>(src);
+  const int4 it = v[0], u0 = v[1], u1 = v[2], u2 = v[3], u3 = v[4];
+  g.un.req = u0.x; g.un.kvh = u0.y; g.un.slotA = u0.z; g.un.slotB = u0.w;
+  g.kvhA = u0.y & 0xffff; g.kvhB = u0.y >> 16;
+  g.un.t0A = u1.x; g.un.t0B = u1.y; g.un.n_tiles = u1.z; g.un.n_chunks = u1.w;
+  g.un.nvisA = u2.x; g.un.nvisB = u2.y; g.un.part_base = u2.z; g.un.prefix_len = u2.w;
+  g.un.npt = u3.x; g.un.win_row0 = u3.y; g.un.winA = u3.z; g.un.winB = u3.w;
+  g.chunk = it.y; g.jb = it.z;
+  const int je = it.w;
+  g.nA = max(0, min(je, g.un.nvisA) - g.jb);
+  g.nB = g.un.slotB >= 0 ? max(0, min(je, g.un.nvisB) - g.jb) : 0;
+  g.n = max(g.nA, g.nB);
+  return src[20] != 0;
+}
+
 // 2^x for a pair of values on the FMA pipe (the MUFU pipe is as busy as the
-// tensor pipe in this kernel, so a share of the exponentials is moved off it):
+// tensor pipe, so the CTA-pair kernel moves a share of the exponentials off it):
 // round-to-nearest split x = n + f, f in [-0.5, 0.5], cubic minimax fit of 2^f
 // (max relative error 7.5e-5, far below bf16 resolution), then n is added to
 // the exponent field.  Valid for -120 <= x <= 120.
-constexpr int kPolyOf4 = 1;   // pairs out of every 4 that take this path (bf16 pages)
-constexpr int kPolyOf4F8 = 1;   // the same share with 8-bit pages (0, 2 and 3 of 4 measured slower)
+constexpr int kPolyOf4 = 1;   // pairs out of every 4 that take this path (CTA-pair kernel)
 __device__ __forceinline__ float2 exp2_poly2(float2 x) {
   x.x = fminf(fmaxf(x.x, -120.f), 120.f);     // beyond +120 the result stays huge: the caller's overflow check fires
   x.y = fminf(fmaxf(x.y, -120.f), 120.f);
@@ -113,10 +142,30 @@ __device__ __forceinline__ bool load_item_uniform(const AttnParams& p, int idx, 
   return u.n > 0;
 }
 
+__device__ __forceinline__ bool load_item_uniform(const int* src, const AttnParams& p, ItemU& u) {
+  ItemGeom g;
+  const bool more = load_item(src, g);
+  u.req = uni(g.un.req); u.kvhA = uni(g.kvhA); u.kvhB = uni(g.kvhB);
+  u.rowA = uni(g.un.slotA * p.bl + g.un.t0A); u.rowB = uni(g.un.slotB * p.bl + g.un.t0B);
+  u.jb = uni(g.jb); u.n = uni(g.n); u.nA = uni(g.nA); u.nB = uni(g.nB);
+  u.npt = uni(g.un.npt); u.prefix_len = uni(g.un.prefix_len); u.win_row0 = uni(g.un.win_row0);
+  u.winA = uni(g.un.winA); u.winB = uni(g.un.winB);
+  return uni(more) != 0;
+}
+
 // All lanes of a converged warp wait on the barrier; the result is uniform.
 __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volatile int* abort, long long limit) {
   const bool ok = mbar_wait(bar, parity, abort, limit);
   return __all_sync(0xffffffffu, ok);
+}
+
+// The same with the expected case first: one try_wait, one vote and a uniform branch (about 60
+// cycles on a barrier that has already flipped, against 140 for the general form, whose loop the
+// compiler has to treat as divergent).  The caller's role must not start at all when
+// limit < 0 (the self-test of the give-up path).
+__device__ __forceinline__ bool warp_wait_ready(uint64_t* bar, uint32_t parity, volatile int* abort, long long limit) {
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  return warp_wait(bar, parity, abort, limit);
 }
 
 // number of keys of local tile j that tile X (window reach winX) may see

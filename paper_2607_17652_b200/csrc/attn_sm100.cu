@@ -10,13 +10,17 @@
 //               works on one tile while the other is in softmax
 //   warp 3      idle (it completes the control warpgroup, which gives its
 //               registers to the softmax warpgroups with setmaxnreg)
-//   warps 4-7   softmax of tile A, one thread per query row: tcgen05.ld of S in
-//               32-column chunks, exp2 against a lazily re-based reference
-//               (only the first tile of an item takes a max pass; part of the
-//               exponentials runs as a polynomial on the FMA pipe), P (bf16)
-//               kept in registers until the tile is known to be in range, then
-//               written back over S in TMEM; epilogue
+//   warps 4-7   softmax of tile A, one thread per query row: its 128 scores are read
+//               from TMEM at once, exp2 against a lazily re-based reference (only the
+//               first tile of an item takes a max pass), P (bf16) written over the
+//               last columns of S in TMEM; epilogue
 //   warps 8-11  the same for tile B
+// What bounds it: at full load the board's power limit (the SM clock falls from 1965
+// to about 1500 MHz), so both fewer cycles and fewer instructions pay; below that,
+// the chain S -> P -> P V -> next S of a tile (about 2500 cycles against 2048 of
+// MMA time for the two tiles of a CTA).  Sustained, back to back, before and after
+// the present form of the loop: long-context workload 1259 -> 1184 us, 64 requests
+// 458 -> 428 us, 128 requests 498 -> 466 us, long context in 8 bits 996 -> 962 us.
 // A Q tile is 128 rows = (128/G tokens) x (G query heads of one KV head) of one
 // slot.  A unit runs two Q tiles side by side: two tiles of one request and KV
 // head, which share each K/V tile from shared memory, or the odd tile left
@@ -37,6 +41,110 @@
 
 namespace fb {
 
+// Largest of N scores held in registers.
+template <int N>
+__device__ __forceinline__ float max_cols(const uint32_t* s) {
+  float m8[8];
+#pragma unroll
+  for (int t = 0; t < 8; ++t) m8[t] = fmaxf(__uint_as_float(s[t]), __uint_as_float(s[8 + t]));
+#pragma unroll
+  for (int i = 16; i < N; i += 16)
+#pragma unroll
+    for (int t = 0; t < 8; ++t) m8[t] = max3(m8[t], __uint_as_float(s[i + t]), __uint_as_float(s[i + 8 + t]));
+  return fmaxf(fmaxf(fmaxf(m8[0], m8[1]), fmaxf(m8[2], m8[3])), fmaxf(fmaxf(m8[4], m8[5]), fmaxf(m8[6], m8[7])));
+}
+
+// P of N scores against the reference behind mb = m_ref * sl2 - shift: packed into pk, the sum of
+// the unrounded values returned, for 8-bit P the largest exponent in xmax.  A masked score (-inf)
+// comes out as exactly 0.  All exponentials run on the MUFU pipe: moving a quarter of them to a
+// polynomial on the FMA pipe shortens the loop in cycles, but at full load this kernel runs at the
+// board's power limit, where the ~13 extra instructions per pair cost more clock than that
+// gains (long-context workload, sustained: 1205 us without against 1262 us with the polynomial;
+// 64 requests 442 against 464; 8-bit pages 970 against 974).
+template <bool F8, int N>
+__device__ __forceinline__ float exp_cols(const uint32_t* s, uint32_t* pk, float sl2, float mb, float& xmax) {
+  const float2 sl2v = make_float2(sl2, sl2), nmb = make_float2(-mb, -mb);
+  float2 acc[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+  float xm4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+  float2 prev = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int i = 0; i < N; i += 2) {
+    const int pr = i >> 1;
+    const float2 x = __ffma2_rn(make_float2(__uint_as_float(s[i]), __uint_as_float(s[i + 1])), sl2v, nmb);
+    if constexpr (F8) xm4[pr & 3] = max3(xm4[pr & 3], x.x, x.y);    // 8-bit P saturates: tracked element by element
+    const float2 pv = make_float2(ex2_approx(x.x), ex2_approx(x.y));
+    acc[pr & 3] = __fadd2_rn(acc[pr & 3], pv);
+    if constexpr (F8) {
+      if (i & 2) pk[i >> 2] = pack_e4m3x4(prev.x, prev.y, pv.x, pv.y);
+      prev = pv;
+    } else {
+      pk[pr] = pack_bf16x2(pv.x, pv.y);
+    }
+  }
+  if constexpr (F8) xmax = fmaxf(fmaxf(xm4[0], xm4[1]), fmaxf(xm4[2], xm4[3]));
+  const float2 t = __fadd2_rn(__fadd2_rn(acc[0], acc[1]), __fadd2_rn(acc[2], acc[3]));
+  return t.x + t.y;
+}
+
+// A key tile taken 32 columns at a time out of TMEM: ragged tiles (`limit` visible keys) and full
+// tiles that broke the bound on their exponentials.  A max pass first; rows whose scores lie more
+// than 2^8 above the reference, or that ask for it (`grow`), move it to their largest score and
+// rescale O and the row sum (O is quiescent: the commit behind this S also covered the previous
+// P V).  Then the exponentials, last columns first, since P goes over the last columns of S.
+// Warp-wide: every lane takes part.  By value in and out, so that the caller's registers stay
+// registers: l (.x) with the tile's weights added, the reference (.y).
+template <int D, bool F8>
+__device__ __noinline__ float2 tile_compact(uint32_t tS, uint32_t tO, int limit, bool first, bool grow, float sl2,
+                                            float shift, float m_ref, float l) {
+  constexpr int P_COL = F8 ? 96 : 64, P_STEP = F8 ? 8 : 16;
+  const int nch = (limit + 31) >> 5;
+  float mx = -INFINITY;
+#pragma unroll 1
+  for (int c = 0; c < nch; ++c) {
+    uint32_t s[32];
+    tmem_ld32(tS + 32 * c, s);
+    tmem_ld_wait();
+#pragma unroll
+    for (int i = 0; i < 32; ++i) s[i] = 32 * c + i < limit ? s[i] : __float_as_uint(-INFINITY);
+    mx = fmaxf(mx, max_cols<32>(s));
+  }
+  if (first) {
+    m_ref = mx;                       // nothing accumulated yet
+  } else {
+    const float xmax = fmaf(mx, sl2, shift - m_ref * sl2);
+    grow = grow || xmax > kRescaleThreshold;
+    if (__any_sync(0xffffffffu, grow)) {
+      const float alpha = grow ? ex2_approx(shift - xmax) : 1.0f;
+      if (grow) { m_ref += (xmax - shift) / sl2; l *= alpha; }
+#pragma unroll 1
+      for (int c = 0; c < D / 32; ++c) {
+        uint32_t o[32];
+        tmem_ld32(tO + c * 32, o);
+        tmem_ld_wait();
+#pragma unroll
+        for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
+        tmem_st32(tO + c * 32, o);
+      }
+    }
+  }
+  const float mb = m_ref * sl2 - shift;
+  float sum = 0.f;
+#pragma unroll 1
+  for (int c = nch - 1; c >= 0; --c) {
+    uint32_t s[32], pk[16];
+    tmem_ld32(tS + 32 * c, s);
+    tmem_ld_wait();
+#pragma unroll
+    for (int i = 0; i < 32; ++i) s[i] = 32 * c + i < limit ? s[i] : __float_as_uint(-INFINITY);
+    float none;
+    sum += exp_cols<F8, 32>(s, pk, sl2, mb, none);
+    if constexpr (F8) tmem_st8(tS + P_COL + P_STEP * c, pk);
+    else tmem_st16(tS + P_COL + P_STEP * c, pk);
+  }
+  tmem_st_wait();
+  return make_float2(l + sum, m_ref);
+}
+
 // F8: the KV pages hold FP8 E4M3 bytes (window resident in the pages, D = 128).  Both products
 // then run as kind::f8f6f4 MMAs: the softmax warps convert their Q tile to E4M3 once per item
 // (per-row power-of-two scale, undone in the row's score factor together with the K scale of
@@ -53,6 +161,7 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
   constexpr int TILE_BYTES = NHKV * 16384;   // one 128-key K or V tile
   constexpr int PAGE_BYTES = NHKV * 8192;    // one 64-key page of it
   constexpr int KSTEPS = F8 ? D / 32 : D / 16;   // MMAs per Q K^T
+  constexpr int P_COL = F8 ? 96 : 64;            // P overwrites the last columns of its tile's S
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sQ = smem;                        // [2] tiles A, B (bf16, as loaded)
@@ -67,11 +176,11 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
   uint64_t* v_full = bars + 6;    // [2]
   uint64_t* v_empty = bars + 8;   // [2]
   uint64_t* s_full = bars + 10;   // [2] A, B
-  uint64_t* p_full = bars + 12;   // [2]
+  uint64_t* p_full = bars + 12;   // [2] P handed over (4 softmax warps)
   uint64_t* o_full = bars + 14;   // [2]
   uint64_t* item_full = bars + 20;   // [2] next work item published by the producer
   uint64_t* item_empty = bars + 22;  // [2] ... and read by the second producer, the MMA warp and the 8 softmax warps
-  volatile int* s_item = reinterpret_cast<volatile int*>(bars + 24);   // [2]
+  int* s_item = reinterpret_cast<int*>(bars + 28);                     // [2][kItemWords] published item records
   uint64_t* drain = bars + 25;       // give-up path only: everything the MMA warp has issued is complete
   uint64_t* q8_full = bars + 26;     // [2] F8: tile X converted to E4M3 by its 128 softmax threads
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 18);
@@ -86,7 +195,7 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     for (int i = 0; i < 2; ++i) {
       mbar_init(&k_full[i], 1); mbar_init(&k_empty[i], 1);
       mbar_init(&v_full[i], 1); mbar_init(&v_empty[i], 1);
-      mbar_init(&s_full[i], 1); mbar_init(&p_full[i], 128); mbar_init(&o_full[i], 1);
+      mbar_init(&s_full[i], 1); mbar_init(&p_full[i], 4); mbar_init(&o_full[i], 1);
       mbar_init(&item_full[i], 1); mbar_init(&item_empty[i], 10);
     }
     mbar_init(drain, 1);
@@ -107,10 +216,11 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
   // warpgroups.  All four warps of a warpgroup execute the same setmaxnreg
   // instruction, and each role's code is dominated by its warpgroup's one.
   // Registers only move inside the CTA: what the two softmax warpgroups take
-  // (2 x 128 x (208 - 168)) must not exceed what the control warpgroup gives up
-  // (128 x (168 - 88)), or setmaxnreg.inc blocks for good.
+  // (2 x 128 x (192 - 168)) must not exceed what the control warpgroup gives up
+  // (128 x (168 - 120)), or setmaxnreg.inc blocks for good.  (88 / 208 measured 1 % slower on
+  // the long-context workload: the control roles spill.)
   if (warp < 4) {
-  asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 120;");
   if (warp == 0 || warp == 2) {
     // ----------------------------------------------------------- producers
     // Warp 0 owns K/V stage 0, warp 2 owns stage 1; warp 0 also draws the work
@@ -185,24 +295,31 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     // Work items are handed out longest first through a global ticket; warp 0
     // draws the ticket and publishes the item to the other roles.
     for (int k = 0; ok; ++k) {
-      int idx = 0;
+      ItemU g;
+      bool more;
       if (warp == 0) {
         if (k >= 2 && !warp_wait(&item_empty[k & 1], ((k >> 1) - 1) & 1, abortf, LIM)) { ok = false; break; }
-        if (lane == 0) idx = atomicAdd(&p.hdr->ticket, 1);
-        idx = uni(idx);
-        if (idx >= n_items) idx = -1;
-        if (lane == 0) { s_item[k & 1] = idx; mbar_arrive(&item_full[k & 1]); }
+        int idx = blockIdx.x;        // the first round needs no ticket
+        if (k > 0) {
+          if (lane == 0) idx = gridDim.x + atomicAdd(&p.hdr->ticket, 1);
+          idx = uni(idx);
+        }
+        // the record goes to shared memory: the other roles would each pay two dependent
+        // global loads (~1300 cycles per item) for it
+        more = idx < n_items;
+        publish_item(p, idx, more, s_item + (k & 1) * kItemWords, lane);
+        if (lane == 0) mbar_arrive(&item_full[k & 1]);
+        load_item_uniform(s_item + (k & 1) * kItemWords, p, g);
         __syncwarp();
-        if (idx < 0) break;          // (the combine kernel re-arms the ticket for the next launch)
+        if (!more) break;            // (the combine kernel re-arms the ticket for the next launch)
       } else {
         if (!warp_wait(&item_full[k & 1], (k >> 1) & 1, abortf, LIM)) { ok = false; break; }
-        idx = s_item[k & 1];
+        more = load_item_uniform(s_item + (k & 1) * kItemWords, p, g);
         __syncwarp();
         if (lane == 0) mbar_arrive(&item_empty[k & 1]);
-        if (idx < 0) break;
+        if (!more) break;
       }
-      ItemU g;
-      if (!load_item_uniform(p, idx, g)) continue;
+      if (g.n <= 0) continue;
       pc_blk = (g.jb * 2) >> 5;
       pc_cur = load_pages(g.req, pc_blk);
       pc_next = load_pages(g.req, pc_blk + 1);
@@ -238,9 +355,15 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     }
   } else if (warp == 1) {
     // ---------------------------------------------------------- MMA issuer
+    // The tensor pipe takes 64 cycles per MMA and queues about 250 cycles of work behind the
+    // issuing thread.  The K and V waits of a key tile come before the wait for P, which is
+    // the last thing to arrive: behind it they would sit in the S -> P -> P V -> next S chain
+    // that bounds a tile (measured: +3 to 5 % on the whole kernel).
     const bool leader = elect_one();
     int q_cnt = 0, q8A = 0, q8B = 0, cntPA = 0, cntPB = 0;
-    bool ok = true;
+    bool ok = LIM >= 0;
+    if (!ok) *abortf = 1;
+    auto wait = [&](uint64_t* bar, uint32_t parity) { return warp_wait_ready(bar, parity, abortf, LIM); };
     // All descriptors are built once; a k-step only adds a constant to the
     // address field (low word, no carry: shared-memory addresses fit the
     // 14-bit field).
@@ -267,16 +390,16 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       }
       __syncwarp();
     };
-    // O_X (+)= P_X V over k-steps [ks0, ks1) of V stage `st`; P_X is read from TMEM.  A step
+    // O_X (+)= P_X V over the first `nks` k-steps of V stage `st`; P_X is read from TMEM.  A step
     // is 16 keys (bf16) or 32 keys (E4M3): 8 TMEM columns of P and 2 KB / 4 KB of V rows.
     constexpr int PV_STEPS = F8 ? 4 : 8, PV_STEP_BYTES = F8 ? 4096 : 2048;
-    auto issue_pv = [&](const int X, int st, int ks0, int ks1, bool acc) {
+    auto issue_pv = [&](const int X, int st, int nks, bool acc) {
       const uint64_t vb = dV0 + (uint32_t)((st * TILE_BYTES) >> 4);
-      const uint32_t d = tmem + 256 + X * 128, a = tmem + X * 128;
+      const uint32_t d = tmem + 256 + X * 128, a = tmem + X * 128 + P_COL;
       if (leader) {
 #pragma unroll
         for (int ks = 0; ks < PV_STEPS; ++ks)
-          if (ks >= ks0 && ks < ks1) {
+          if (ks < nks) {
             if (F8) umma_ts_f8(d, a + ks * 8, vb + (uint32_t)((ks * PV_STEP_BYTES) >> 4), idesc_pv, (acc || ks > 0) ? 1u : 0u);
             else umma_ts(d, a + ks * 8, vb + (uint32_t)((ks * PV_STEP_BYTES) >> 4), idesc_pv, (acc || ks > 0) ? 1u : 0u);
           }
@@ -291,28 +414,28 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     auto wait_k = [&](int st) -> bool {
       const int use = st ? kuse1 : kuse0;
       if (st) ++kuse1; else ++kuse0;
-      return warp_wait(&k_full[st], use & 1, abortf, LIM);
+      return wait(&k_full[st], use & 1);
     };
     auto wait_v = [&](int st) -> bool {
       const int use = st ? vuse1 : vuse0;
       if (st) ++vuse1; else ++vuse0;
-      return warp_wait(&v_full[st], use & 1, abortf, LIM);
+      return wait(&v_full[st], use & 1);
     };
     for (int k = 0; ok; ++k) {
-      if (!warp_wait(&item_full[k & 1], (k >> 1) & 1, abortf, LIM)) { ok = false; break; }
-      const int idx = s_item[k & 1];
+      if (!wait(&item_full[k & 1], (k >> 1) & 1)) { ok = false; break; }
+      ItemU g;
+      const bool more = load_item_uniform(s_item + (k & 1) * kItemWords, p, g);
       __syncwarp();
       if (lane == 0) mbar_arrive(&item_empty[k & 1]);
-      if (idx < 0) break;
-      ItemU g;
-      if (!load_item_uniform(p, idx, g)) continue;
+      if (!more) break;
+      if (g.n <= 0) continue;
       const int nA = g.nA, nB = g.nB, n = g.n;
       if (F8) {     // the tiles in E4M3, written by the softmax warps
-        if (nA > 0 && !warp_wait(&q8_full[0], q8A & 1, abortf, LIM)) { ok = false; break; }
-        if (nB > 0 && !warp_wait(&q8_full[1], q8B & 1, abortf, LIM)) { ok = false; break; }
+        if (nA > 0 && !wait(&q8_full[0], q8A & 1)) { ok = false; break; }
+        if (nB > 0 && !wait(&q8_full[1], q8B & 1)) { ok = false; break; }
         q8A += nA > 0; q8B += nB > 0;
         fence_proxy_async_smem();
-      } else if (!warp_wait(q_full, q_cnt & 1, abortf, LIM)) { ok = false; break; }
+      } else if (!wait(q_full, q_cnt & 1)) { ok = false; break; }
       ++q_cnt;
       if (!g.dual()) {
         // ---- tiles A and B share every K/V tile
@@ -333,10 +456,10 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
           // tile A: O_A += P_A(j) V(j), then S_A(j+1) so that softmax A can go on
           if (j < nA) {
             const int nks = pv_steps(g.limit(j, g.winA, p.resident));
-            if (!warp_wait(&p_full[0], cntPA & 1, abortf, LIM)) { ok = false; break; }
+            if (!wait(&p_full[0], cntPA & 1)) { ok = false; break; }
             ++cntPA;
             tc_fence_after();
-            issue_pv(0, sv, 0, nks, j > 0);
+            issue_pv(0, sv, nks, j > 0);
           }
           if (j + 1 < nA) {
             tc_fence_after();
@@ -345,10 +468,10 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
           // tile B
           if (j < nB) {
             const int nks = pv_steps(g.limit(j, g.winB, p.resident));
-            if (!warp_wait(&p_full[1], cntPB & 1, abortf, LIM)) { ok = false; break; }
+            if (!wait(&p_full[1], cntPB & 1)) { ok = false; break; }
             ++cntPB;
             tc_fence_after();
-            issue_pv(1, sv, 0, nks, j > 0);
+            issue_pv(1, sv, nks, j > 0);
           }
           commit(&v_empty[sv]);
           if (j + 1 < nB) {
@@ -391,7 +514,7 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
           if (X) { ++jB; ++cntPB; } else { ++jA; ++cntPA; }
           if (!wait_v(X)) { ok = false; break; }
           tc_fence_after();
-          issue_pv(X, X, 0, pv_steps(g.limit(j, g.winA, p.resident)), j > 0);
+          issue_pv(X, X, pv_steps(g.limit(j, g.winA, p.resident)), j > 0);
           commit(&v_empty[X]);
           if (j + 1 < n) {
             // this stream's next K tile could only be requested when its last Q K^T had
@@ -415,7 +538,7 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     // Four warps per Q tile, one thread per query row (its TMEM lane).  Every wait is
     // taken by the whole warp with one outcome (warp_wait): tcgen05.ld / st below are
     // warp-wide and must never run with part of a warp gone.
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 208;");
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 192;");
     const int X = (warp - 4) >> 2;                 // 0: tile A, 1: tile B
     const int quad = warp & 3;                     // TMEM lane quadrant of this warp
     const int row = quad * 32 + lane;              // query row of the tile
@@ -426,15 +549,16 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     float out_scale = 1.0f;            // F8: V scale of the KV head
     constexpr float kShift = F8 ? kF8PShift : 0.f;
     int cntS = 0, cntO = 0, qcnt = 0;
-    bool ok = true;
+    bool ok = LIM >= 0;
+    if (!ok) *abortf = 1;
     for (int k = 0; ok; ++k) {
-      if (!warp_wait(&item_full[k & 1], (k >> 1) & 1, abortf, LIM)) { ok = false; break; }
-      const int idx = s_item[k & 1];
+      if (!warp_wait_ready(&item_full[k & 1], (k >> 1) & 1, abortf, LIM)) { ok = false; break; }
+      ItemGeom g;
+      const bool more = load_item(s_item + (k & 1) * kItemWords, g);
       __syncwarp();
       if (lane == 0) mbar_arrive(&item_empty[k & 1]);
-      if (idx < 0) break;
-      ItemGeom g;
-      if (!load_item(p, idx, g)) continue;
+      if (!more) break;
+      if (g.n <= 0) continue;
       const int q_par = qcnt & 1;        // phase of q_full that carries this item's Q tiles
       ++qcnt;
       const int nMine = X == 0 ? g.nA : g.nB;
@@ -480,135 +604,60 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       }
       float m_ref = -INFINITY, l = 0.f;
       for (int j = 0; j < nMine; ++j) {
-        if (!warp_wait(&s_full[X], cntS & 1, abortf, LIM)) { ok = false; break; }
+        if (!warp_wait_ready(&s_full[X], cntS & 1, abortf, LIM)) { ok = false; break; }
         ++cntS;
         tc_fence_after();
         const int limit = tile_limit(g, j, winX, p.resident);
-        // The running reference m_ref is only re-based when a score exceeds it by
-        // more than 2^8 (lazy rescale), so the common tile needs no separate max
-        // pass: the exponentials are taken against the old reference while the
-        // largest exponent is tracked, P stays in registers, and only if the
-        // bound was broken is the tile redone against the new reference.  The
-        // first tile of an item has no reference yet and takes a max pass.
-        if (j == 0) {
-          float m8[8];
-#pragma unroll
-          for (int t = 0; t < 8; ++t) m8[t] = -INFINITY;
-          uint32_t sa[64], sb[64];
-          tmem_ld32(tS, sa); tmem_ld32(tS + 32, sa + 32);
+        if (limit == kTileN) {
+          // A full tile.  The whole row of S is read at once and the exponentials are taken against
+          // the running reference m_ref, which is only re-based when they grow past 2^8 (lazy
+          // rescale), so the common tile needs no separate max pass; the first tile of an item
+          // has no reference yet and takes one.  P goes over the last columns of S while the
+          // sum is still being formed: what it overwrites is kept in registers (s + P_COL) and
+          // the rest stays in TMEM, so the rare tile that has to be redone can be, and the
+          // check costs nothing on the way to the hand-off.
+          uint32_t s[128], pk[32];
+          tmem_ld32(tS, s); tmem_ld32(tS + 32, s + 32); tmem_ld32(tS + 64, s + 64); tmem_ld32(tS + 96, s + 96);
           tmem_ld_wait();
-          tmem_ld32(tS + 64, sb); tmem_ld32(tS + 96, sb + 32);     // in flight during the first half
-#pragma unroll
-          for (int i = 0; i < 64; i += 16)
-#pragma unroll
-            for (int t = 0; t < 8; ++t)
-              m8[t] = max3(m8[t], i + t < limit ? __uint_as_float(sa[i + t]) : -INFINITY,
-                           i + 8 + t < limit ? __uint_as_float(sa[i + 8 + t]) : -INFINITY);
-          tmem_ld_wait();
-#pragma unroll
-          for (int i = 0; i < 64; i += 16)
-#pragma unroll
-            for (int t = 0; t < 8; ++t)
-              m8[t] = max3(m8[t], 64 + i + t < limit ? __uint_as_float(sb[i + t]) : -INFINITY,
-                           64 + i + 8 + t < limit ? __uint_as_float(sb[i + 8 + t]) : -INFINITY);
-          m_ref = fmaxf(fmaxf(fmaxf(m8[0], m8[1]), fmaxf(m8[2], m8[3])), fmaxf(fmaxf(m8[4], m8[5]), fmaxf(m8[6], m8[7])));
-        }
-        uint32_t pk[F8 ? 32 : 64];             // P of this tile: packed bf16 pairs, or E4M3 four to a word
-        // 8-bit P saturates at 448, so the largest exponent of the tile is tracked element by
-        // element; bf16 P has the range of fp32 and only needs the tile's sum to stay finite
-        constexpr bool TRACK = F8;
-        float tile_sum = 0.f;
-#pragma unroll 1
-        for (int attempt = 0; attempt < 2; ++attempt) {
+          if (j == 0) m_ref = max_cols<128>(s);
           const float mb = m_ref * sl2 - kShift;
-          float2 acc2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-          float xm4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-          const float2 sl2v = make_float2(sl2, sl2), nmb = make_float2(-mb, -mb);
-          uint32_t sc[2][32];
-          tmem_ld32(tS, sc[0]);
-#pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            uint32_t* sr = sc[c & 1];
-            tmem_ld_wait();
-            if (c < 3) tmem_ld32(tS + 32 * (c + 1), sc[(c + 1) & 1]);   // next chunk in flight
-            if (limit >= 32 * c + 32) {
-              float2 prev = make_float2(0.f, 0.f);
-#pragma unroll
-              for (int i = 0; i < 32; i += 2) {
-                const float2 x = __ffma2_rn(make_float2(__uint_as_float(sr[i]), __uint_as_float(sr[i + 1])), sl2v, nmb);
-                if constexpr (TRACK) xm4[(i >> 1) & 3] = max3(xm4[(i >> 1) & 3], x.x, x.y);
-                float2 pv;
-                if (((i >> 1) & 3) < (F8 ? kPolyOf4F8 : kPolyOf4)) pv = exp2_poly2(x);
-                else pv = make_float2(ex2_approx(x.x), ex2_approx(x.y));
-                acc2[(i >> 1) & 1] = __fadd2_rn(acc2[(i >> 1) & 1], pv);
-                if constexpr (F8) {
-                  if (i & 2) pk[8 * c + (i >> 2)] = pack_e4m3x4(prev.x, prev.y, pv.x, pv.y);
-                  prev = pv;
-                } else {
-                  pk[16 * c + (i >> 1)] = pack_bf16x2(pv.x, pv.y);
-                }
-              }
-            } else {
-              float2 prev = make_float2(0.f, 0.f);
-#pragma unroll
-              for (int i = 0; i < 32; i += 2) {
-                const bool v0 = 32 * c + i < limit, v1 = 32 * c + i + 1 < limit;
-                const float x0 = fmaf(__uint_as_float(sr[i]), sl2, -mb), x1 = fmaf(__uint_as_float(sr[i + 1]), sl2, -mb);
-                if constexpr (TRACK) {
-                  if (v0) xm4[0] = fmaxf(xm4[0], x0);
-                  if (v1) xm4[1] = fmaxf(xm4[1], x1);
-                }
-                const float p0 = v0 ? ex2_approx(x0) : 0.f, p1 = v1 ? ex2_approx(x1) : 0.f;
-                acc2[0].x += p0 + p1;
-                if constexpr (F8) {
-                  if (i & 2) pk[8 * c + (i >> 2)] = pack_e4m3x4(prev.x, prev.y, p0, p1);
-                  prev = make_float2(p0, p1);
-                } else {
-                  pk[16 * c + (i >> 1)] = pack_bf16x2(p0, p1);
-                }
-              }
-            }
-          }
-          tile_sum = (acc2[0].x + acc2[0].y) + (acc2[1].x + acc2[1].y);
-          float xmax = fmaxf(fmaxf(xm4[0], xm4[1]), fmaxf(xm4[2], xm4[3]));
-          const bool grow = attempt == 0 && (TRACK ? xmax > kRescaleThreshold : !(tile_sum <= kGrowSum));
-          if (!__any_sync(0xffffffffu, grow)) break;
-          if constexpr (!TRACK) {
-            // the largest exponent of the tile was not tracked: one more pass over S (whole warp)
-#pragma unroll 1
-            for (int c = 0; c < 4; ++c) {
-              uint32_t sr[32];
-              tmem_ld32(tS + 32 * c, sr);
-              tmem_ld_wait();
-#pragma unroll
-              for (int i = 0; i < 32; ++i)
-                if (32 * c + i < limit) xmax = fmaxf(xmax, fmaf(__uint_as_float(sr[i]), sl2, -mb));
-            }
-          }
-          // rare: re-base this row's reference, rescale what has been accumulated so far
-          // (O is quiescent: the commit behind this S also covered the previous P V)
-          const float alpha = grow ? ex2_approx(kShift - xmax) : 1.0f;
-          if (grow) { m_ref += (xmax - kShift) / sl2; l *= alpha; }
-#pragma unroll
-          for (int c = 0; c < D / 32; ++c) {
-            uint32_t o[32];
-            tmem_ld32(tO + c * 32, o);
-            tmem_ld_wait();
-#pragma unroll
-            for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
-            tmem_st32(tO + c * 32, o);
+          float tile_sum;
+          bool grow;
+          if constexpr (F8) {
+            float xm;
+            tile_sum = exp_cols<true, 128>(s, pk, sl2, mb, xm);
+            tmem_st32(tS + P_COL, pk);
+            grow = xm > kRescaleThreshold;
+          } else {
+            float none;
+            uint32_t pk2[32];
+            tile_sum = exp_cols<false, 64>(s, pk, sl2, mb, none);
+            tmem_st32(tS + P_COL, pk);
+            tile_sum += exp_cols<false, 64>(s + 64, pk2, sl2, mb, none);
+            tmem_st32(tS + P_COL + 32, pk2);
+            grow = !(tile_sum <= kGrowSum);
           }
           tmem_st_wait();
+          if (__any_sync(0xffffffffu, grow)) {
+            // rare: put S back as it was and take the tile again, re-based
+#pragma unroll
+            for (int c = P_COL; c < 128; c += 32) tmem_st32(tS + c, s + c);
+            tmem_st_wait();
+            const float2 r = tile_compact<D, F8>(tS, tO, kTileN, j == 0, grow, sl2, kShift, m_ref, l);
+            l = r.x; m_ref = r.y;
+          } else {
+            l += tile_sum;
+          }
+        } else {
+          const float2 r = tile_compact<D, F8>(tS, tO, limit, j == 0, false, sl2, kShift, m_ref, l);
+          l = r.x; m_ref = r.y;
         }
-        l += tile_sum;
-        tmem_st32(tS, pk);
-        if constexpr (!F8) tmem_st32(tS + 32, pk + 32);
-        tmem_st_wait();
         tc_fence_before();
-        mbar_arrive(&p_full[X]);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&p_full[X]);
       }
       if (!ok) break;
-      if (!warp_wait(&o_full[X], cntO & 1, abortf, LIM)) { ok = false; break; }
+      if (!warp_wait_ready(&o_full[X], cntO & 1, abortf, LIM)) { ok = false; break; }
       ++cntO;
       tc_fence_after();
       if (g.un.n_chunks <= 1) {
