@@ -1,13 +1,12 @@
 // fb_t2t_step: the token-to-token step over the logits (Sec. 2.1, Eq. 1; the
 // counts of Eq. 2).
 //
-// Kernel 1 (bandwidth-bound): one CTA (128 threads, eight 16-byte loads in
-// flight each: the best of the shapes tried) per live row, or a cluster of two
-// CTAs per row when the batch has few rows, streams the row's bf16
-// logits once with 16-byte loads and keeps, per thread, a running
-// (max, first index of the max, sum of exp relative to that max); a
-// warp-shuffle + shared-memory reduction merges them with the lowest-index
-// rule.  Output: top-1 token and its softmax probability 1 / sum exp(z - max).
+// Kernel 1 (bandwidth-bound): one CTA per live row, or a cluster of up to eight CTAs per
+// row when the batch has few rows, streams the row's bf16 logits once with 16-byte loads
+// (the next batch of loads in flight while the current one is absorbed) and keeps, per
+// thread, a running (max, first index of the max, sum of exp relative to that max); a
+// warp-shuffle + shared-memory reduction merges them with the lowest-index rule.
+// Output: top-1 token and its softmax probability 1 / sum exp(z - max).
 // Kernel 2 (tiny): one warp per slot applies Eq. 1 to the slot's bl positions,
 // updates the tokens in place and produces the per-block counts.
 #include <cfloat>
@@ -18,8 +17,7 @@
 
 namespace fb {
 
-constexpr int kRowThreads = 128;
-constexpr int kRowUnroll = 8;   // 16-byte loads in flight per thread
+constexpr int kRowUnroll = 4;   // 16-byte loads per thread and batch, two batches in flight
 constexpr float kLog2e = 1.4426950408889634f;
 
 __device__ __forceinline__ uint4 ld_stream16(const uint4* p) {
@@ -74,7 +72,44 @@ __device__ __forceinline__ void absorb8(RowAcc& a, const uint4 v, int base) {
   a.s += acc;
 }
 
-__global__ void __launch_bounds__(kRowThreads)
+__device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b) {
+  uint32_t r;
+  asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  return r;
+}
+
+// Two 16-byte pieces at once (`base` < `base2`: their first vocabulary indices): the maximum of the
+// 16 logits on the packed values, the exponentials with packed fp32 arithmetic into two sums.
+__device__ __forceinline__ void absorb16(RowAcc& a, float2& s2, const uint4 v, const uint4 w, int base, int base2) {
+  const uint32_t q[8] = {v.x, v.y, v.z, v.w, w.x, w.y, w.z, w.w};
+  const uint32_t mm = max_bf16x2(max_bf16x2(max_bf16x2(q[0], q[1]), max_bf16x2(q[2], q[3])),
+                                 max_bf16x2(max_bf16x2(q[4], q[5]), max_bf16x2(q[6], q[7])));
+  const float cm = fmaxf(bf16_lo(mm), bf16_hi(mm));
+  if (cm > a.m) {                       // rare after the first few pieces
+    const float f = a.m == -INFINITY ? 0.f : fast_ex2((a.m - cm) * kLog2e);
+    s2.x *= f; s2.y *= f;
+    a.m = cm;
+#pragma unroll
+    for (int i = 7; i >= 0; --i) {
+      const int at = (i < 4 ? base : base2) + 2 * (i & 3);
+      if (bf16_hi(q[i]) == cm) a.idx = at + 1;
+      if (bf16_lo(q[i]) == cm) a.idx = at;
+    }
+  }
+  if (a.m == -INFINITY) return;          // nothing but -inf so far: contributes 0
+  const float mb = -a.m * kLog2e;
+  const float2 mb2 = make_float2(mb, mb), l2 = make_float2(kLog2e, kLog2e);
+  float2 t = make_float2(0.f, 0.f);      // a sum of its own first: short chains of roundings
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const float2 x = __ffma2_rn(make_float2(bf16_lo(q[i]), bf16_hi(q[i])), l2, mb2);
+    t = __fadd2_rn(t, make_float2(fast_ex2(x.x), fast_ex2(x.y)));
+  }
+  s2 = __fadd2_rn(s2, t);
+}
+
+template <int T>
+__global__ void __launch_bounds__(T)
 t2t_rows_kernel(const uint4* __restrict__ logits, const int32_t* __restrict__ n_live, int bl, int nvec,
                 int32_t* __restrict__ argmax, float* __restrict__ conf, int32_t* __restrict__ status) {
   pdl_wait();
@@ -89,19 +124,42 @@ t2t_rows_kernel(const uint4* __restrict__ logits, const int32_t* __restrict__ n_
     if (tid == 0 && rank == 0) { argmax[row] = -1; conf[row] = 0.f; }
     return;
   }
+  constexpr int U = kRowUnroll, kStep = U * T;
   const int seg = (nvec + cl - 1) / cl;
-  const int vend = min(nvec, (rank + 1) * seg);
+  const int vbeg = min(nvec, rank * seg), vend = min(nvec, vbeg + seg);
   const uint4* p = logits + (size_t)row * nvec;
   RowAcc a{-INFINITY, 0.f, 0x7fffffff};
-  int i = rank * seg + tid;
-  for (; i + (kRowUnroll - 1) * kRowThreads < vend; i += kRowUnroll * kRowThreads) {
-    uint4 v[kRowUnroll];
+  float2 s2 = make_float2(0.f, 0.f);
+  const int full = (vend - vbeg) / kStep;         // whole batches
+  uint4 v[2][U];
+  if (full > 0) {
 #pragma unroll
-    for (int u = 0; u < kRowUnroll; ++u) v[u] = ld_stream16(p + i + u * kRowThreads);
-#pragma unroll
-    for (int u = 0; u < kRowUnroll; ++u) absorb8(a, v[u], (i + u * kRowThreads) * 8);
+    for (int u = 0; u < U; ++u) v[0][u] = ld_stream16(p + vbeg + tid + u * T);
   }
-  for (; i < vend; i += kRowThreads) absorb8(a, ld_stream16(p + i), i * 8);
+  int k = 0;
+  for (; k + 2 <= full; k += 2) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      if (k + h + 1 < full) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) v[h ^ 1][u] = ld_stream16(p + vbeg + (k + h + 1) * kStep + tid + u * T);
+      }
+#pragma unroll
+      for (int u = 0; u < U; u += 2) {
+        const int i = vbeg + (k + h) * kStep + tid + u * T;
+        absorb16(a, s2, v[h][u], v[h][u + 1], i * 8, (i + T) * 8);
+      }
+    }
+  }
+  if (k < full) {
+#pragma unroll
+    for (int u = 0; u < U; u += 2) {
+      const int i = vbeg + k * kStep + tid + u * T;
+      absorb16(a, s2, v[0][u], v[0][u + 1], i * 8, (i + T) * 8);
+    }
+  }
+  a.s = s2.x + s2.y;
+  for (int i = vbeg + full * kStep + tid; i < vend; i += T) absorb8(a, ld_stream16(p + i), i * 8);
   // warp reduce
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -111,7 +169,7 @@ t2t_rows_kernel(const uint4* __restrict__ logits, const int32_t* __restrict__ n_
     b.idx = __shfl_xor_sync(0xffffffffu, a.idx, o);
     merge(a, b);
   }
-  __shared__ RowAcc sh[kRowThreads / 32];
+  __shared__ RowAcc sh[T / 32];
   if ((tid & 31) == 0) sh[tid >> 5] = a;
   __syncthreads();
   RowAcc b{-INFINITY, 0.f, 0x7fffffff};
@@ -127,7 +185,7 @@ t2t_rows_kernel(const uint4* __restrict__ logits, const int32_t* __restrict__ n_
     }
   };
   if (tid < 32) {
-    if (tid < kRowThreads / 32) b = sh[tid];
+    if (tid < T / 32) b = sh[tid];
     warp_merge(16);
   }
   if (cl > 1) {                          // uniform over the cluster
@@ -232,19 +290,46 @@ __global__ void __launch_bounds__(128) t2t_update_kernel(const UpdParams p) {
   }
 }
 
+// Threads that share a row (in CTAs of up to 512, a cluster of up to eight).  A pass is fastest
+// with about 1,000 threads an SM: fewer do not cover the load latency, more only add merging.
+// That is about 180,000 threads over the slot capacity (live rows are typically two thirds of
+// it), rounded to a power of two, and no more threads than the row has pairs of pieces.
+// Measured, V = 151,552, call time in us (live rows of capacity: 128x1 / 256x1 / 512x1 / 512x2 /
+// 512x4 threads x CTAs per row; in front the former 128 threads, a pair of CTAs below 2048 rows):
+//     64 of    64:  30.4 |  27.0   21.4   17.8   13.5    9.9
+//     96 of   128:  33.8 |  47.9   31.8   19.0   13.0   14.1
+//    640 of  1024:  47.3 |  60.7   43.0   42.5   51.3   68.7
+//   3072 of  4608:   160 |   155    159    170    212    307
+//   5120 of  8192:   259 |   252    262    279    351    511
+struct RowShape { int threads, ctas; };
+static RowShape row_shape(int rows, int nvec) {
+  const int floor_ = rows < 2048 ? 256 : 128;
+  int w = 128;
+  while (w < 4096 && (long long)w * 1448 / 1024 * rows < 180000) w *= 2;   // nearest power of two (in the log)
+  w = w < floor_ ? floor_ : w;
+  while (w > 128 && 2 * w > nvec) w /= 2;
+  RowShape s;
+  s.threads = w < 512 ? w : 512;
+  s.ctas = w / s.threads;
+  return s;
+}
+
 int launch_t2t(fb_ctx* ctx, const fb_pack* pk, const void* logits, const fb_state* st, int32_t* argmax,
                float* conf, uint8_t* action, int32_t* slot_stats, int32_t* status, cudaStream_t stream) {
   const fb_config& c = ctx->cfg;
   const int max_slots = c.max_requests * c.wmax;
   const int rows = max_slots * c.block_len;
-  // few rows: a pair of CTAs per row (measured on 1024 rows of 151,936 logits: 42 us against
-  // 50 us for one CTA per row, 45 us for four, 50 us for eight; on 8192 rows a pair loses 6 %)
-  const int cl = rows >= 2048 ? 1 : 2;
-  if (int e = cuda_err(ctx, launch_pdl_cluster(t2t_rows_kernel, rows * cl, kRowThreads, 0, stream, cl,
-                                               static_cast<const uint4*>(logits), pk->n_live, c.block_len,
-                                               c.vocab / 8, argmax, conf, status),
-                       "t2t_rows_kernel launch"))
-    return e;
+  const RowShape shape = row_shape(rows, c.vocab / 8);
+  const int T = shape.threads, cl = shape.ctas;
+  auto launch = [&](auto kernel, int threads) {
+    return cuda_err(ctx, launch_pdl_cluster(kernel, rows * cl, threads, 0, stream, cl,
+                                            static_cast<const uint4*>(logits), pk->n_live, c.block_len,
+                                            c.vocab / 8, argmax, conf, status),
+                    "t2t_rows_kernel launch");
+  };
+  const int e = T == 128 ? launch(t2t_rows_kernel<128>, 128) : T == 256 ? launch(t2t_rows_kernel<256>, 256)
+                                                                        : launch(t2t_rows_kernel<512>, 512);
+  if (e) return e;
   return launch_t2t_update(ctx, pk, st, argmax, conf, action, slot_stats, stream);
 }
 
