@@ -1,9 +1,11 @@
-"""ctypes binding of libflowblock.so: argument marshalling only.
+"""Binding of libflowblock.so: argument marshalling only.
 
 Every step of the hot path runs inside the CUDA library; this module turns
 torch tensors into raw device pointers and calls the C entry points of the
-same name.  There is no CPU fallback: if the library has not been built the
-import of :func:`lib` raises.
+same name.  The calls of a decode step go through the small C module _marshal
+(a step of one request is bound by the host, and ctypes structures took about
+10 us a call); set-up and host-buffer calls go through ctypes.  There is no
+CPU fallback: if the library has not been built :func:`lib` raises.
 """
 from __future__ import annotations
 
@@ -76,12 +78,18 @@ class fb_device_bufs(C.Structure):
         "step_counters", "status", "ws")]
 
 
+# the calls that _marshal makes, in the order of its bind()
+_FAST = ("fb_pack_wavefronts", "fb_wavefront_attn", "fb_t2t_step", "fb_gate_commit", "fb_scatter_window_kv",
+         "fb_scatter_window_kv_fp8", "fb_wavefront_attn_fp8", "fb_embed_gather", "fb_lm_head_t2t",
+         "fb_wavefront_attn_static")
+
 _lib = None
+_m = None
 
 
 def lib() -> C.CDLL:
     """The loaded CUDA library.  Raises if it is missing (no fallback)."""
-    global _lib
+    global _lib, _m
     if _lib is None:
         if not os.path.exists(LIB_PATH):
             raise RuntimeError(
@@ -125,7 +133,9 @@ def lib() -> C.CDLL:
             if n not in ("fb_last_error", "fb_workspace_bytes",
                          "fb_lm_head_workspace_bytes"):
                 getattr(l, n).restype = I
-        _lib = l
+        from . import _marshal
+        _marshal.bind(*(C.cast(getattr(l, n), P).value for n in _FAST))
+        _lib, _m = l, _marshal
     return _lib
 
 
@@ -143,8 +153,16 @@ def _ptr(t) -> int | None:
     return t.data_ptr()
 
 
+# the current stream of the current device as a raw handle, without building a
+# torch.cuda.Stream object where torch offers that
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_raw_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream(stream) -> int:
     if stream is None:
+        if _raw_stream is not None and _raw_device is not None:
+            return _raw_stream(_raw_device())
         stream = torch.cuda.current_stream()
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
@@ -158,6 +176,7 @@ class Context:
         rc = lib().fb_create(C.byref(self.cfg), C.byref(self._h))
         if rc != FB_OK:
             raise FlowBlockError(rc, lib().fb_last_error(None).decode())
+        self._hv = self._h.value
         if tuning:
             self.set_tuning(**tuning)
 
@@ -182,6 +201,7 @@ class Context:
             if self._h:
                 lib().fb_destroy(self._h)
                 self._h = C.c_void_p()
+                self._hv = None
         except Exception:
             pass
 
@@ -261,59 +281,51 @@ def alloc_workspace(ctx: Context, device) -> torch.Tensor:
 # ----------------------------------------------------------------- the calls
 def fb_pack_wavefronts(ctx: Context, st: DeviceState, pk: PackBuffers, ws,
                        status, stream=None):
-    s, p = st.c(), pk.c()
-    ctx.check(lib().fb_pack_wavefronts(ctx.handle, C.byref(s), C.byref(p),
-                                       _ptr(ws), _ptr(status), _stream(stream)))
+    rc = _m.pack(ctx._hv, st, pk, ws, status, _stream(stream))
+    if rc:
+        ctx.check(rc)
 
 
 def fb_wavefront_attn(ctx: Context, pk: PackBuffers, q, k_win, v_win, k_pool,
                       v_pool, page_table, out, ws, status, stream=None):
-    p = pk.c()
-    ctx.check(lib().fb_wavefront_attn(
-        ctx.handle, C.byref(p), _ptr(q), _ptr(k_win), _ptr(v_win),
-        _ptr(k_pool), _ptr(v_pool), _ptr(page_table), _ptr(out), _ptr(ws),
-        _ptr(status), _stream(stream)))
+    rc = _m.attn(ctx._hv, pk, q, k_win, v_win, k_pool, v_pool, page_table, out, ws, status, _stream(stream))
+    if rc:
+        ctx.check(rc)
 
 
 def fb_scatter_window_kv(ctx: Context, pk: PackBuffers, page_table, k_new, v_new,
                          k_pool, v_pool, status, rope_base: float = 0.0,
                          stream=None):
     """Eq. 6 as data movement (contexts with window_in_pages=1)."""
-    p = pk.c()
-    ctx.check(lib().fb_scatter_window_kv(
-        ctx.handle, C.byref(p), _ptr(page_table), _ptr(k_new), _ptr(v_new),
-        _ptr(k_pool), _ptr(v_pool), C.c_float(rope_base), _ptr(status),
-        _stream(stream)))
+    rc = _m.scatter(ctx._hv, pk, page_table, k_new, v_new, k_pool, v_pool, rope_base, status, _stream(stream))
+    if rc:
+        ctx.check(rc)
 
 
 def fb_scatter_window_kv_fp8(ctx: Context, pk: PackBuffers, page_table, k_new, v_new,
                              k_pool8, v_pool8, k_scale, v_scale, status,
                              rope_base: float = 0.0, stream=None):
     """Eq. 6 into 8-bit (E4M3) pages with per-KV-head scales."""
-    p = pk.c()
-    ctx.check(lib().fb_scatter_window_kv_fp8(
-        ctx.handle, C.byref(p), _ptr(page_table), _ptr(k_new), _ptr(v_new),
-        _ptr(k_pool8), _ptr(v_pool8), _ptr(k_scale), _ptr(v_scale),
-        C.c_float(rope_base), _ptr(status), _stream(stream)))
+    rc = _m.scatter_fp8(ctx._hv, pk, page_table, k_new, v_new, k_pool8, v_pool8, k_scale, v_scale, rope_base, status,
+                        _stream(stream))
+    if rc:
+        ctx.check(rc)
 
 
 def fb_wavefront_attn_fp8(ctx: Context, pk: PackBuffers, q, k_pool8, v_pool8,
                           k_scale, v_scale, page_table, out, ws, status,
                           stream=None):
     """Attention over 8-bit (E4M3) pages, window resident in the pages."""
-    p = pk.c()
-    ctx.check(lib().fb_wavefront_attn_fp8(
-        ctx.handle, C.byref(p), _ptr(q), _ptr(k_pool8), _ptr(v_pool8),
-        _ptr(k_scale), _ptr(v_scale), _ptr(page_table), _ptr(out), _ptr(ws),
-        _ptr(status), _stream(stream)))
+    rc = _m.attn_fp8(ctx._hv, pk, q, k_pool8, v_pool8, k_scale, v_scale, page_table, out, ws, status, _stream(stream))
+    if rc:
+        ctx.check(rc)
 
 
 def fb_embed_gather(ctx: Context, pk: PackBuffers, table, x, status, stream=None):
     """x[i] = table[qtok[i]] for the rows of live slots (Eq. 4 feeding the model)."""
-    p = pk.c()
-    ctx.check(lib().fb_embed_gather(
-        ctx.handle, C.byref(p), _ptr(table), int(table.shape[0]),
-        int(table.shape[1]), _ptr(x), _ptr(status), _stream(stream)))
+    rc = _m.embed(ctx._hv, pk, table, int(table.shape[0]), int(table.shape[1]), x, status, _stream(stream))
+    if rc:
+        ctx.check(rc)
 
 
 def fb_wavefront_attn_static(ctx: Context, st: DeviceState, pk: PackBuffers, q,
@@ -321,39 +333,34 @@ def fb_wavefront_attn_static(ctx: Context, st: DeviceState, pk: PackBuffers, q,
                              stream=None):
     """Attention for callers that cannot allocate: no workspace argument, the
     scratch is an array inside the library (see the header for its limits)."""
-    s, p = st.c(), pk.c()
-    ctx.check(lib().fb_wavefront_attn_static(
-        ctx.handle, C.byref(s), C.byref(p), _ptr(q), _ptr(k_win), _ptr(v_win),
-        _ptr(k_pool), _ptr(v_pool), _ptr(out), _ptr(status), _stream(stream)))
+    rc = _m.attn_static(ctx._hv, st, pk, q, k_win, v_win, k_pool, v_pool, out, status, _stream(stream))
+    if rc:
+        ctx.check(rc)
 
 
 def fb_t2t_step(ctx: Context, pk: PackBuffers, logits, st: DeviceState, argmax,
                 conf, action, slot_stats, status, stream=None):
-    s, p = st.c(), pk.c()
-    ctx.check(lib().fb_t2t_step(
-        ctx.handle, C.byref(p), _ptr(logits), C.byref(s), _ptr(argmax),
-        _ptr(conf), _ptr(action), _ptr(slot_stats), _ptr(status),
-        _stream(stream)))
+    rc = _m.t2t(ctx._hv, pk, logits, st, argmax, conf, action, slot_stats, status, _stream(stream))
+    if rc:
+        ctx.check(rc)
 
 
 def fb_lm_head_t2t(ctx: Context, pk: PackBuffers, x, w, st: DeviceState, argmax,
                    conf, action, slot_stats, ws, status, stream=None):
     """fb_t2t_step with the LM head fused in front (logits never written)."""
-    s, p = st.c(), pk.c()
-    ctx.check(lib().fb_lm_head_t2t(
-        ctx.handle, C.byref(p), _ptr(x), _ptr(w), int(x.shape[1]), C.byref(s),
-        _ptr(argmax), _ptr(conf), _ptr(action), _ptr(slot_stats), _ptr(ws),
-        _ptr(status), _stream(stream)))
+    rc = _m.lm_head(ctx._hv, pk, x, w, int(x.shape[1]), st, argmax, conf, action, slot_stats, ws, status,
+                    _stream(stream))
+    if rc:
+        ctx.check(rc)
 
 
 def fb_gate_commit(ctx: Context, pk: PackBuffers, slot_stats, st: DeviceState,
                    k_win, v_win, k_pool, v_pool, n_committed, spawned,
                    step_counters, status, stream=None):
-    s, p = st.c(), pk.c()
-    ctx.check(lib().fb_gate_commit(
-        ctx.handle, C.byref(p), _ptr(slot_stats), C.byref(s), _ptr(k_win),
-        _ptr(v_win), _ptr(k_pool), _ptr(v_pool), _ptr(n_committed),
-        _ptr(spawned), _ptr(step_counters), _ptr(status), _stream(stream)))
+    rc = _m.gate(ctx._hv, pk, slot_stats, st, k_win, v_win, k_pool, v_pool, n_committed, spawned, step_counters, status,
+                 _stream(stream))
+    if rc:
+        ctx.check(rc)
 
 
 def fb_step_host(ctx: Context, st: DeviceState, pk: PackBuffers, dev: dict,

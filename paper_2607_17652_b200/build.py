@@ -1,4 +1,5 @@
-"""Builds libflowblock.so (sm_100a) in-tree with nvcc.
+"""Builds libflowblock.so (sm_100a) in-tree with nvcc, and the binding's
+marshalling module (csrc/marshal.c) with the C compiler.
 
 ``python -m paper_2607_17652_b200.build`` or :func:`build`.  Cross-compiles
 without a GPU.  Objects are rebuilt only when a source or header is newer.
@@ -8,12 +9,14 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 ROOT = os.path.dirname(HERE)
 LIB = os.path.join(HERE, "libflowblock.so")
+MARSHAL = os.path.join(HERE, "_marshal.so")
 SOURCES = ["api.cu", "pack.cu", "t2t.cu", "gate_commit.cu", "attn_sm100.cu", "scatter.cu", "lm_head.cu",
            "attn_static.cu", "attn_pair_sm100.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo",
@@ -50,7 +53,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         if verbose or r.returncode:
             sys.stderr.write(" ".join(cmd) + "\n" + r.stdout + r.stderr)
         if r.returncode:
-            raise RuntimeError("nvcc failed for " + cmd[-3])
+            raise RuntimeError("the compiler failed for " + cmd[-3])
         return r.stderr
 
     with ThreadPoolExecutor(max_workers=4) as ex:
@@ -58,6 +61,11 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if jobs or not os.path.exists(LIB) or force:
         run([_nvcc(), "-shared", "-o", LIB, *objs, "-gencode",
              "arch=compute_100a,code=sm_100a"])
+    src = os.path.join(CSRC, "marshal.c")
+    if force or not os.path.exists(MARSHAL) or \
+            os.path.getmtime(MARSHAL) < max(os.path.getmtime(src), hdr_time):
+        run([os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-Wall",
+             "-I", sysconfig.get_paths()["include"], src, "-o", MARSHAL])
     if logs:
         with open(os.path.join(HERE, "build", "ptxas.log"), "w") as f:
             f.write("\n".join(logs))

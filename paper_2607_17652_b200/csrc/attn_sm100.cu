@@ -795,10 +795,13 @@ int ensure_device(fb_ctx* ctx) {
   // forget the cached tensor maps
   ctx->dev_ready = false;
   for (auto& mp : ctx->map_ptrs) mp = nullptr;
-  cudaDeviceProp prop;
-  if (int e = cuda_err(ctx, cudaGetDeviceProperties(&prop, dev), "cudaGetDeviceProperties")) return e;
-  if (prop.major != 10) return set_err(ctx, FB_ERR_UNSUPPORTED, "the attention kernel needs an sm_100 device");
-  ctx->num_sms = prop.multiProcessorCount;
+  // (two attributes, not cudaGetDeviceProperties, which takes milliseconds: this is on the path of
+  // a new context's first step)
+  int major = 0, sms = 0;
+  if (int e = cuda_err(ctx, cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev), "cudaDeviceGetAttribute")) return e;
+  if (int e = cuda_err(ctx, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "cudaDeviceGetAttribute")) return e;
+  if (major != 10) return set_err(ctx, FB_ERR_UNSUPPORTED, "the attention kernel needs an sm_100 device");
+  ctx->num_sms = sms;
   void* fn = nullptr;
   cudaDriverEntryPointQueryResult q;
   if (int e = cuda_err(ctx, cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &q),
