@@ -175,6 +175,13 @@ __device__ __forceinline__ int tile_limit(const ItemGeom& g, int j, int winX, in
                                 : winX - (gj - g.un.npt) * kTileN;
   return min(lim, kTileN);
 }
+// Unnormalised O of a split piece in the workspace: `tile` = 2 * piece + Q tile, 8 columns (32 bytes)
+// of a row together and the 128 rows of a tile side by side, so that a warp whose lanes hold
+// successive rows stores and loads whole kilobytes (a row-major layout took 6000 cycles a piece).
+template <int D>
+__device__ __forceinline__ float* part_o_at(float* base, size_t tile, int row, int col8) {
+  return base + ((tile * (D / 8) + col8) * kTileM + row) * 8;
+}
 __device__ __forceinline__ int round16(int x) { return (x + 15) & ~15; }
 
 void fill_attn_params(fb_ctx* ctx, AttnParams& p, const int32_t* page_table, void* out, void* ws, int32_t* status,

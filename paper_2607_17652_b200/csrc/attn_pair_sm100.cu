@@ -510,17 +510,15 @@ wavefront_attn_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid
             }
           }
         } else {
-          const size_t prow = ((size_t)(me.part_base + g.chunk) * 2 + X) * kTileM + row;
-          p.part_ml[prow * 2 + 0] = m_ref * sl2;
-          p.part_ml[prow * 2 + 1] = l;
-          uint4* dst = reinterpret_cast<uint4*>(p.part_o + prow * D);
+          const size_t tile = (size_t)(me.part_base + g.chunk) * 2 + X;
+          reinterpret_cast<float2*>(p.part_ml)[tile * kTileM + row] = make_float2(m_ref * sl2, l);
 #pragma unroll
           for (int c = 0; c < D / 32; ++c) {
             uint32_t o[32];
             tmem_ld32(tO + c * 32, o);
             tmem_ld_wait();
 #pragma unroll
-            for (int i = 0; i < 4; ++i) st_global_v8(dst + c * 8 + 2 * i, o + 8 * i);
+            for (int i = 0; i < 4; ++i) st_global_v8(part_o_at<D>(p.part_o, tile, row, 4 * c + i), o + 8 * i);
           }
         }
       }

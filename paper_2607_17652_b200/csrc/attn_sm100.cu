@@ -681,17 +681,17 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
           }
         }
       } else {
-        const size_t prow = ((size_t)(g.un.part_base + g.chunk) * 2 + X) * kTileM + row;
-        p.part_ml[prow * 2 + 0] = m_ref * sl2 - kShift;     // the reference the exponentials were taken against
-        p.part_ml[prow * 2 + 1] = l / out_scale;            // (the merge divides by the sum: the V scale goes in here)
-        uint4* dst = reinterpret_cast<uint4*>(p.part_o + prow * D);
+        const size_t tile = (size_t)(g.un.part_base + g.chunk) * 2 + X;
+        // the reference the exponentials were taken against, and the sum (the merge divides by
+        // it: the V scale goes in here)
+        reinterpret_cast<float2*>(p.part_ml)[tile * kTileM + row] = make_float2(m_ref * sl2 - kShift, l / out_scale);
 #pragma unroll
         for (int c = 0; c < D / 32; ++c) {
           uint32_t o[32];
           tmem_ld32(tO + c * 32, o);
           tmem_ld_wait();
 #pragma unroll
-          for (int i = 0; i < 4; ++i) st_global_v8(dst + c * 8 + 2 * i, o + 8 * i);
+          for (int i = 0; i < 4; ++i) st_global_v8(part_o_at<D>(p.part_o, tile, row, 4 * c + i), o + 8 * i);
         }
       }
       tc_fence_before();
@@ -718,71 +718,95 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
   if (warp == 1) { tc_fence_after(); tmem_dealloc(tmem, 512); }
 }
 
-// Merge of the split-KV partials, chunks in index order.  A unit is cut into
-// 32 pieces of 8 of its 256 rows; the CTAs of a fixed-size grid loop over
-// the pieces (nothing to do, and an immediate return, when no unit was split).
-// A warp takes one row at a time and keeps the loads of four chunks in flight.
-constexpr int kCombineSplit = 32;        // pieces of 8 rows: one row per warp, no serial row loop
-constexpr int kCombineCtasPerSm = 8;
+// Merge of the split-KV partials (deterministic: a fixed order of additions).  A warp takes 8
+// columns of 32 / W rows; its lanes are W groups that share the pieces of a row (group g takes
+// pieces g, g + W, ...), so that up to 4 W pieces are in flight together and every access is a run
+// of at least 256 bytes.  Each lane carries a running maximum along, the groups meet by shuffles.
+// A CTA keeps its rows and columns and goes over every G-th unit, picking the split ones 32 at a
+// time; it returns at once when no unit was split.
+// Bound by latency (a round of loads takes 2 to 3 us under this load), so W grows with the longest
+// split of the batch, up to the point where the CTAs no longer run together: attention call in us
+// with W = 1 / 2 / 4: one request of 3,000 tokens (6 pieces a unit) 20.9 / 19.3 / 20.1, 28,000
+// tokens (12 pieces) 84 / 76 / 65, 8 requests (3 pieces, 40 units) 23.6 / 26.9 / 29; with a warp
+// per row over a row-major layout these took 23.1, 97 and 26.4.
+constexpr int kCombineThreads = 256, kCombineCtasPerSm = 8, kCombineDepth = 4, kCombineMostCtas = 1024, kCombineMaxWays = 4;
 template <int D>
-__global__ void __launch_bounds__(256) attn_combine_kernel(const AttnParams p) {
+__global__ void __launch_bounds__(kCombineThreads, 3) attn_combine_kernel(const AttnParams p) {
   pdl_wait();
   // The attention kernel is complete: re-arm its work ticket, so that the same work list can be
   // run again (also after a launch that gave up on a bounded wait half way through its items).
   if (blockIdx.x == 0 && threadIdx.x == 0) p.hdr->ticket = 0;
-  if (p.hdr->n_parts == 0) return;
-  const int n_pieces = p.hdr->n_units * kCombineSplit;
+  const int n_parts = p.hdr->n_parts, n_units = p.hdr->n_units, longest = p.hdr->max_chunks;
+  if (n_parts == 0) return;
+  int W = 1;
+  while (W < kCombineMaxWays && W * kCombineDepth < longest && 2 * W * n_units * (D / 8) <= kCombineMostCtas) W *= 2;
+  const int per_unit = W * (D / 8), G = gridDim.x / per_unit;           // (the grid is a multiple of 4 D / 8)
+  const int sub = blockIdx.x % per_unit, cols = sub % (D / 8);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  constexpr int PER = D / 32;
-  for (int piece = blockIdx.x; piece < n_pieces; piece += gridDim.x) {
-  const AttnUnit un = p.units[piece / kCombineSplit];
-  if (un.n_chunks <= 1) continue;
-  const int row0 = (piece % kCombineSplit) * (2 * kTileM / kCombineSplit);
-  for (int rr = row0 + warp; rr < row0 + 2 * kTileM / kCombineSplit; rr += 8) {
-    const int X = rr / kTileM, row = rr % kTileM;
-    const int slot = X == 0 ? un.slotA : un.slotB;
-    if (slot < 0) continue;
-    const int nvis = X == 0 ? un.nvisA : un.nvisB, t0 = X == 0 ? un.t0A : un.t0B;
-    int nc = 0;                               // chunks that hold keys visible to this tile
-    while (nc < un.n_chunks && (int)((long long)nc * un.n_tiles / un.n_chunks) < nvis) ++nc;
-    const size_t prow0 = ((size_t)un.part_base * 2 + X) * kTileM + row;   // chunk c: + c * 2 * kTileM
-    float M = -INFINITY;
-    for (int c = lane; c < nc; c += 32) M = fmaxf(M, p.part_ml[(prow0 + (size_t)c * 2 * kTileM) * 2]);
+  const int rpw = 32 / W, way = lane / rpw;                             // rows per warp, this lane's group
+  const int first_row = ((sub / (D / 8)) * 8 + warp) * rpw;             // of the unit's 256
+  const int X = first_row >= kTileM, row = first_row % kTileM + lane % rpw;
+  for (int u0 = blockIdx.x / per_unit; u0 < n_units; u0 += 32 * G) {
+    const int mine = u0 + lane * G;
+    unsigned todo = __ballot_sync(0xffffffffu, mine < n_units && p.units[mine].n_chunks > 1);
+    for (; todo; todo &= todo - 1) {
+      const AttnUnit un = p.units[u0 + (__ffs(todo) - 1) * G];
+      const int slot = X == 0 ? un.slotA : un.slotB;
+      if (slot < 0) continue;                                           // (uniform: X is the warp's)
+      const int nvis = X == 0 ? un.nvisA : un.nvisB, t0 = X == 0 ? un.t0A : un.t0B;
+      // chunks that hold keys visible to this tile: those that start before tile nvis
+      const int nc = min(un.n_chunks, (int)(((long long)nvis * un.n_chunks + un.n_tiles - 1) / un.n_tiles));
+      const size_t tile0 = (size_t)un.part_base * 2 + X;              // chunk c: + 2 c
+      const float2* ml = reinterpret_cast<const float2*>(p.part_ml) + tile0 * kTileM + row;
+      float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+      float M = -INFINITY, L = 0.f;
+      for (int c0 = way; c0 < nc; c0 += kCombineDepth * W) {
+        float2 w[kCombineDepth];
+        float v[kCombineDepth][8];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
-    float acc[PER];
+        for (int k = 0; k < kCombineDepth; ++k) {
+          const int c = c0 + k * W;
+          w[k] = make_float2(-INFINITY, 0.f);
 #pragma unroll
-    for (int i = 0; i < PER; ++i) acc[i] = 0.f;
-    float L = 0.f;
-    for (int c0 = 0; c0 < nc; c0 += 4) {
-      float w[4], lv[4], v[4][PER];
+          for (int i = 0; i < 8; ++i) v[k][i] = 0.f;
+          if (c < nc) {
+            ld_global_v8(v[k], part_o_at<D>(p.part_o, tile0 + 2 * c, row, cols));
+            w[k] = ml[(size_t)c * 2 * kTileM];
+          }
+        }
+        float m = M;
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int c = min(c0 + k, nc - 1);
-        const size_t prow = prow0 + (size_t)c * 2 * kTileM;
-        w[k] = p.part_ml[prow * 2];
-        lv[k] = p.part_ml[prow * 2 + 1];
-        const float* src = p.part_o + prow * D + lane * PER;
+        for (int k = 0; k < kCombineDepth; ++k) m = fmaxf(m, w[k].x);
+        const float f = M == -INFINITY ? 0.f : ex2_approx(M - m);
+        M = m;
+        L *= f;
 #pragma unroll
-        for (int i = 0; i < PER; ++i) v[k][i] = src[i];
+        for (int i = 0; i < 8; ++i) acc[i] *= f;
+#pragma unroll
+        for (int k = 0; k < kCombineDepth; ++k) {
+          const float wk = ex2_approx(w[k].x - M);                      // a piece that is not there: 2^-inf = 0
+          L += wk * w[k].y;
+#pragma unroll
+          for (int i = 0; i < 8; ++i) acc[i] += wk * v[k][i];
+        }
       }
+      for (int o = rpw; o < 32; o <<= 1) {
+        const float m2 = __shfl_xor_sync(0xffffffffu, M, o), m = fmaxf(M, m2);   // group 0 holds piece 0: finite in pairs with it
+        const float f = M == -INFINITY ? 0.f : ex2_approx(M - m), f2 = m2 == -INFINITY ? 0.f : ex2_approx(m2 - m);
+        M = m;
+        L = L * f + __shfl_xor_sync(0xffffffffu, L, o) * f2;
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        if (c0 + k >= nc) break;
-        const float wk = ex2_approx(w[k] - M);
-        L += wk * lv[k];
-#pragma unroll
-        for (int i = 0; i < PER; ++i) acc[i] += wk * v[k][i];
+        for (int i = 0; i < 8; ++i) acc[i] = acc[i] * f + __shfl_xor_sync(0xffffffffu, acc[i], o) * f2;
+      }
+      if (way == 0) {
+        const float inv = 1.0f / L;
+        const int grow_ = slot * p.bl + t0 + row / p.group;
+        const int head = (X == 0 ? (un.kvh & 0xffff) : (un.kvh >> 16)) * p.group + row % p.group;
+        *reinterpret_cast<uint4*>(p.out + ((size_t)grow_ * p.n_q_heads + head) * D + cols * 8) =
+            make_uint4(pack_bf16x2(acc[0] * inv, acc[1] * inv), pack_bf16x2(acc[2] * inv, acc[3] * inv),
+                       pack_bf16x2(acc[4] * inv, acc[5] * inv), pack_bf16x2(acc[6] * inv, acc[7] * inv));
       }
     }
-    const float inv = 1.0f / L;
-    const int grow_ = slot * p.bl + t0 + row / p.group;
-    const int head = (X == 0 ? (un.kvh & 0xffff) : (un.kvh >> 16)) * p.group + row % p.group;
-    __nv_bfloat16* dst = p.out + ((size_t)grow_ * p.n_q_heads + head) * D + lane * PER;
-#pragma unroll
-    for (int i = 0; i < PER; i += 2)
-      *reinterpret_cast<uint32_t*>(dst + i) = pack_bf16x2(acc[i] * inv, acc[i + 1] * inv);
-  }
   }
 }
 
@@ -860,10 +884,13 @@ void fill_attn_params(fb_ctx* ctx, AttnParams& p, const int32_t* page_table, voi
 }
 
 int launch_attn_combine(fb_ctx* ctx, const AttnParams& p, int list, cudaStream_t stream) {
-  const int grid = min(max(ctx->ws.l[list].max_units, 1) * kCombineSplit, kCombineCtasPerSm * ctx->num_sms);
+  const int per_unit = kCombineMaxWays * ctx->cfg.head_dim / 8;
+  const int groups = max(1, min(ctx->ws.l[list].max_units, kCombineCtasPerSm * ctx->num_sms / per_unit));
   if (ctx->cfg.head_dim == 64)
-    return cuda_err(ctx, launch_pdl(attn_combine_kernel<64>, grid, 256, 0, stream, p), "attn_combine_kernel launch");
-  return cuda_err(ctx, launch_pdl(attn_combine_kernel<128>, grid, 256, 0, stream, p), "attn_combine_kernel launch");
+    return cuda_err(ctx, launch_pdl(attn_combine_kernel<64>, groups * per_unit, kCombineThreads, 0, stream, p),
+                    "attn_combine_kernel launch");
+  return cuda_err(ctx, launch_pdl(attn_combine_kernel<128>, groups * per_unit, kCombineThreads, 0, stream, p),
+                  "attn_combine_kernel launch");
 }
 
 static int encode_q(fb_ctx* ctx, const void* q) {

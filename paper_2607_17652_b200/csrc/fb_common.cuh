@@ -36,7 +36,8 @@ struct __align__(16) AttnItem {
 struct SchedHeader {
   int32_t n_items, n_units, chunk_tiles, n_parts;
   int32_t total_tiles;
-  int32_t ticket, done;                // dynamic item hand-out of the attention kernel
+  int32_t ticket;                      // dynamic item hand-out of the attention kernel
+  int32_t max_chunks;                  // pieces of the most finely split unit
   int32_t pad[9];
 };
 

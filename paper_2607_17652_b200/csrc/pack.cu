@@ -122,7 +122,7 @@ __device__ void build_sched(const PackParams& p, const int list) {
   const int max_items = p.max_items[list], max_units = p.max_units[list], max_parts = p.max_parts[list];
   __shared__ int sh_scan[kPackThreads / 32 + 1];
   __shared__ int bins[kCostBins];
-  __shared__ int sh_total, sh_units;
+  __shared__ int sh_total, sh_units, sh_chunks;
   __shared__ SplitRule sh_rule;
   const int tid = threadIdx.x;
   // bad states are reported once, by the gather blocks (null status here)
@@ -133,7 +133,7 @@ __device__ void build_sched(const PackParams& p, const int list) {
     mine += g.nunits * g.nt;
     mine_units += g.nt ? g.nunits : 0;
   }
-  if (tid == 0) { sh_total = 0; sh_units = 0; }
+  if (tid == 0) { sh_total = 0; sh_units = 0; sh_chunks = 0; }
   for (int i = tid; i < kCostBins; i += kPackThreads) bins[i] = 0;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -163,6 +163,7 @@ __device__ void build_sched(const PackParams& p, const int list) {
     const int wbase = work_run + block_excl_scan(nunits * g.nt, &tw, sh_scan);
     work_run += tw;
     const ReqSplit rs = req_split(rule, wbase, nunits, g.nt);
+    if (nunits) atomicMax(&sh_chunks, max(rs.ufine > 0 ? rs.nch_c : 0, rs.ufine < nunits ? rs.nch_f : 0));
     const int urel = block_excl_scan(nunits, &tu, sh_scan);
     const int pbase = part_run + block_excl_scan(rs.parts(nunits), &tp, sh_scan);
     block_excl_scan(rs.items(nunits), &ti, sh_scan);
@@ -241,7 +242,7 @@ __device__ void build_sched(const PackParams& p, const int list) {
       hdr->chunk_tiles = rule.ct;
       hdr->n_parts = mult * part_run;
       hdr->total_tiles = sh_total;
-      hdr->ticket = 0; hdr->done = 0;
+      hdr->ticket = 0; hdr->max_chunks = sh_chunks;
       if (total_items > max_items || mult * unit_run > max_units || mult * part_run > max_parts)
         atomicOr(p.status, FB_ST_BAD_STATE);
     }
