@@ -172,11 +172,13 @@ const char* fb_last_error(const fb_ctx* ctx); /* ctx may be NULL */
  * split-KV merge.  The paper has no counterpart (it states no kernel design).
  * 0 in a field selects the default. */
 typedef struct {
-  int32_t attn_target_items;     /* work items the key-axis split aims for
-                                    (default 2 x 148: two per SM); 1 = never
-                                    split, large = split down to the minimum  */
+  int32_t attn_target_items;     /* work items the key-axis split aims for; 1 =
+                                    never split, large = split down to the
+                                    minimum.  Default: the split with the least
+                                    estimated time for the batch at hand      */
   int32_t attn_min_chunk_tiles;  /* shortest key range of a split piece, in
-                                    128-key tiles (default 4)                 */
+                                    128-key tiles (default 4 with a target, 2
+                                    without)                                  */
   int32_t attn_pair;             /* 1: four Q tiles of one request and KV head
                                     at a time run on a pair of CTAs that share
                                     every K/V tile (tcgen05 cta_group::2; bf16

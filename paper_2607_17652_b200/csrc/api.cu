@@ -23,10 +23,18 @@ int fail(fb_ctx* ctx, int code, const std::string& msg) {
 
 namespace fb {
 
-WsLayout make_ws_layout(const fb_config& c, int tiles_per_slot, int target_items, int min_chunk_tiles, int pair_on) {
+WsLayout make_ws_layout(const fb_ctx* ctx) {
+  const fb_config& c = ctx->cfg;
+  const int target_items = ctx->target_items, pair_on = ctx->pair_on;
   WsLayout w{};
-  const long long qtiles = (long long)c.max_requests * c.wmax * tiles_per_slot;
-  const long long max_tiles = ((long long)c.max_pages_per_req * kPage + kTileN - 1) / kTileN + 2;
+  const long long qtiles = (long long)c.max_requests * c.wmax * ctx->tiles_per_slot;
+  // key tiles of a request whose page-table row covers its prefix and window
+  long long max_tiles = 0;
+  for (int k = 1; k <= c.wmax; ++k) {
+    const long long window = (long long)k * c.block_len, prefix = (long long)c.max_pages_per_req * kPage - window;
+    const long long n = (prefix > 0 ? (prefix + kTileN - 1) / kTileN : 0) + (window + kTileN - 1) / kTileN;
+    max_tiles = n > max_tiles ? n : max_tiles;
+  }
   size_t off = 0;
   for (int l = 0; l < 2; ++l) {
     WsList& x = w.l[l];
@@ -39,7 +47,8 @@ WsLayout make_ws_layout(const fb_config& c, int tiles_per_slot, int target_items
     // split pieces: the bound that split_rule derives (per scheduling unit; list 1 has two records
     // per unit), and never more than every unit cut into pieces of the minimum length (a unit spans
     // at most the keys its page-table row can address)
-    const long long every = units * ((max_tiles + min_chunk_tiles - 1) / min_chunk_tiles);
+    const int min_chunk = l == 0 && ctx->auto_min_chunk < ctx->min_chunk_tiles ? ctx->auto_min_chunk : ctx->min_chunk_tiles;
+    const long long every = max_tiles > min_chunk ? units * ((max_tiles + min_chunk - 1) / min_chunk) : 0;
     const long long by_target = mult * ((long long)kPartsPerTarget * target + 8);
     x.max_units = (int)units;
     x.max_parts = units ? (int)(by_target < every ? by_target : every) : 0;
@@ -128,9 +137,11 @@ int fb_create(const fb_config* cfg, fb_ctx** out) {
   ctx->target_items = fb::kDefaultTargetItems;
   ctx->min_chunk_tiles = fb::kDefaultMinChunkTiles;
   ctx->wait_cycles = fb::kDefaultWaitCycles;
+  ctx->auto_split = 1;
+  ctx->auto_min_chunk = fb::kAutoMinChunkTiles;
   ctx->pair_on = 0;                      // the CTA-pair kernel is opt-in (fb_tuning.attn_pair)
   ctx->sm_scale = c.sm_scale > 0.f ? c.sm_scale : 1.0f / sqrtf((float)c.head_dim);
-  ctx->ws = fb::make_ws_layout(c, ctx->tiles_per_slot, ctx->target_items, ctx->min_chunk_tiles, ctx->pair_on);
+  ctx->ws = fb::make_ws_layout(ctx);
   *out = ctx;
   return FB_OK;
 }
@@ -143,9 +154,11 @@ int fb_set_tuning(fb_ctx* ctx, const fb_tuning* t) {
     return fail(ctx, FB_ERR_INVALID_ARG, "a tuning value is out of range");
   ctx->target_items = t->attn_target_items ? t->attn_target_items : fb::kDefaultTargetItems;
   ctx->min_chunk_tiles = t->attn_min_chunk_tiles ? t->attn_min_chunk_tiles : fb::kDefaultMinChunkTiles;
+  ctx->auto_split = t->attn_target_items == 0;
+  ctx->auto_min_chunk = t->attn_min_chunk_tiles ? t->attn_min_chunk_tiles : fb::kAutoMinChunkTiles;
   ctx->wait_cycles = t->wait_cycles ? (long long)t->wait_cycles : fb::kDefaultWaitCycles;
   ctx->pair_on = ctx->cfg.head_dim == 128 && !ctx->cfg.kv_fp8 && t->attn_pair;
-  ctx->ws = fb::make_ws_layout(ctx->cfg, ctx->tiles_per_slot, ctx->target_items, ctx->min_chunk_tiles, ctx->pair_on);
+  ctx->ws = fb::make_ws_layout(ctx);
   return FB_OK;
 }
 
@@ -168,14 +181,32 @@ int fb_attn_plan_host(const fb_ctx* ctx, const int32_t* h_prefix_len, const int3
     const int target = list == 0 ? ctx->target_items : (ctx->target_items > 1 ? ctx->target_items / 2 : 1);
     const int mult = list + 1;
     long long total = 0, units = 0;
+    int longest = 0;
     for (int r = 0; r < n; ++r) {
       const fb::ReqGeom g = fb::req_geom_of(h_live_blocks[r], h_prefix_len[r], ctx->tiles_per_slot, c.block_len,
                                             c.n_kv_heads, c.window_in_pages, list, ctx->pair_on);
       total += (long long)g.nunits * g.nt;
       units += g.nt ? g.nunits : 0;
+      longest = g.nt > longest ? g.nt : longest;
     }
     if (total > 0x7fffffffll) return fail(nullptr, FB_ERR_UNSUPPORTED, "fb_attn_plan_host: work list too long");
-    const fb::SplitRule rule = fb::split_rule((int)total, (int)units, target, ctx->min_chunk_tiles);
+    fb::SplitRule rule = fb::split_rule((int)total, (int)units, target, ctx->min_chunk_tiles);
+    if (list == 0 && ctx->auto_split) {
+      long long best = -1;
+      int ct = longest > 0 ? longest : 1;
+      for (int i = 0; i < fb::kSplitCandidates; ++i) {
+        const int cand = fb::split_candidate(i, longest);
+        if (i > 0 && cand < ctx->auto_min_chunk) continue;
+        fb::SplitStat st{};
+        for (int r = 0; r < n; ++r)
+          fb::split_stat_add(st, fb::req_geom_of(h_live_blocks[r], h_prefix_len[r], ctx->tiles_per_slot, c.block_len,
+                                                 c.n_kv_heads, c.window_in_pages, list, ctx->pair_on),
+                             c.n_kv_heads, cand > 0 ? cand : 1);
+        const long long e = fb::split_estimate(st, ctx->ws.l[0].max_parts);
+        if (e >= 0 && (best < 0 || e < best)) { best = e; ct = cand > 0 ? cand : 1; }
+      }
+      rule = fb::split_auto((int)total, (int)units, ct);
+    }
     long long wbase = 0, items = 0, parts = 0;
     for (int r = 0; r < n; ++r) {
       const fb::ReqGeom g = fb::req_geom_of(h_live_blocks[r], h_prefix_len[r], ctx->tiles_per_slot, c.block_len,

@@ -311,7 +311,7 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
         if (lane == 0) mbar_arrive(&item_full[k & 1]);
         load_item_uniform(s_item + (k & 1) * kItemWords, p, g);
         __syncwarp();
-        if (!more) break;            // (the combine kernel re-arms the ticket for the next launch)
+        if (!more) break;
       } else {
         if (!warp_wait(&item_full[k & 1], (k >> 1) & 1, abortf, LIM)) { ok = false; break; }
         more = load_item_uniform(s_item + (k & 1) * kItemWords, p, g);
@@ -700,6 +700,9 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
   // ---------------------------------------------------------------- teardown
   tc_fence_before();
   __syncthreads();
+  // Last one out re-arms the work ticket, so that the same work list can be run again (also after
+  // a launch that gave up half way through its items).  This thread drew this CTA's tickets.
+  if (tid == 0 && atomicAdd(&p.hdr->done, 1) == (int)gridDim.x - 1) { p.hdr->ticket = 0; p.hdr->done = 0; }
   if (*abortf) {
     // A bounded wait gave up.  Nothing may still be running on this CTA's shared memory or
     // TMEM when they are handed on: (1) the MMA warp commits everything it has issued to a
@@ -733,8 +736,7 @@ constexpr int kCombineThreads = 256, kCombineCtasPerSm = 8, kCombineDepth = 4, k
 template <int D>
 __global__ void __launch_bounds__(kCombineThreads, 3) attn_combine_kernel(const AttnParams p) {
   pdl_wait();
-  // The attention kernel is complete: re-arm its work ticket, so that the same work list can be
-  // run again (also after a launch that gave up on a bounded wait half way through its items).
+  // (the CTA-pair kernel's list: its ticket is re-armed here, for a further run of the same list)
   if (blockIdx.x == 0 && threadIdx.x == 0) p.hdr->ticket = 0;
   const int n_parts = p.hdr->n_parts, n_units = p.hdr->n_units, longest = p.hdr->max_chunks;
   if (n_parts == 0) return;
@@ -884,6 +886,7 @@ void fill_attn_params(fb_ctx* ctx, AttnParams& p, const int32_t* page_table, voi
 }
 
 int launch_attn_combine(fb_ctx* ctx, const AttnParams& p, int list, cudaStream_t stream) {
+  if (list == 0 && ctx->ws.l[0].max_parts == 0) return FB_OK;      // this context never splits a key range
   const int per_unit = kCombineMaxWays * ctx->cfg.head_dim / 8;
   const int groups = max(1, min(ctx->ws.l[list].max_units, kCombineCtasPerSm * ctx->num_sms / per_unit));
   if (ctx->cfg.head_dim == 64)

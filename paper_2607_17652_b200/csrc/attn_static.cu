@@ -42,7 +42,7 @@ fb::WsLayout unsplit_layout(const fb_ctx* c) {
   fb::WsList& x = w.l[0];
   x.max_units = (int)((qtiles + c->cfg.max_requests + 1) / 2) * c->cfg.n_kv_heads;
   x.max_items = x.max_units + 8;
-  x.max_parts = 2;        // never used: no unit is split
+  x.max_parts = 0;        // no unit is split
   size_t off = 0;
   x.header = off;  off = align_up(off + sizeof(fb::SchedHeader), 256);
   x.items = off;   off = align_up(off + (size_t)x.max_items * sizeof(fb::AttnItem), 256);
@@ -112,6 +112,7 @@ extern "C" int fb_wavefront_attn_static(fb_ctx* ctx, const fb_state* st, const f
     sh->sm_scale = ctx->sm_scale;
     sh->target_items = 1;                 // chunk length = all tiles: nothing is split
     sh->min_chunk_tiles = 1 << 20;
+    sh->auto_split = 0;
     sh->pair_on = 0;                      // one work list, one kernel
     sh->ws = lay;
   }

@@ -14,8 +14,10 @@ namespace fb {
 constexpr int kTileM = 128;      // query rows per Q tile (tokens x group heads)
 constexpr int kTileN = 128;      // keys per K/V tile (two 64-token pages)
 constexpr int kPage = 64;
+constexpr int kSms = 148;
 constexpr int kDefaultMinChunkTiles = 4;
-constexpr int kDefaultTargetItems = 2 * 148;   // about two work items per SM before key ranges are split
+constexpr int kAutoMinChunkTiles = 2;          // the same where the split is chosen by estimate (no target given)
+constexpr int kDefaultTargetItems = 2 * kSms;  // about two work items per SM before key ranges are split
 
 // One unit = two Q tiles of one request that run side by side in a CTA: either
 // two different tiles under one KV head (they share every K/V tile), or one
@@ -36,9 +38,9 @@ struct __align__(16) AttnItem {
 struct SchedHeader {
   int32_t n_items, n_units, chunk_tiles, n_parts;
   int32_t total_tiles;
-  int32_t ticket;                      // dynamic item hand-out of the attention kernel
+  int32_t ticket, done;                // dynamic item hand-out of the attention kernel; CTAs that have left it
   int32_t max_chunks;                  // pieces of the most finely split unit
-  int32_t pad[9];
+  int32_t pad[8];
 };
 
 // The workspace holds two work lists: list 0 for the one-CTA kernel, list 1 ("quads": four Q
@@ -122,6 +124,57 @@ __host__ __device__ inline SplitRule split_rule(int total, int units, int target
   s.fine_from = on ? total - (int)((long long)kFillerPercent * total / 100) : 0x7fffffff;
   return s;
 }
+// Without a target from the caller the chunk length is chosen by estimate, for the whole batch: of
+// 32 lengths from the longest key range down to 1/48 of it, the one with the least
+//   makespan = max(W / SMs, longest item, waves * W / items) + merge,
+// W the work of all items.  A batch of equal items that just misses whole waves pays for the last
+// one in full; from three waves on handing out longest first fills half of that in.  The costs
+// are measured (ns): a key tile of a pair, of two K/V streams; what an item costs beside its
+// tiles, whole or as a piece; the merge, once and per piece.  Against always aiming at two items
+// an SM: 28,000-token request 72 -> 64 us, 24 requests of 700 to 5,000 tokens 161 -> 151 (not split
+// at all), 8 requests 24.6 (the same split).
+// With two units an SM and more, and items so long that half of one outweighs their cost twice,
+// the last 15 % of the work are cut into filler pieces as above (16 long contexts: 1064 -> 1030).
+constexpr int kTileNs = 1600, kTileDualNs = 2200, kItemNs = 4000, kPieceNs = 4500, kMergeNs = 5000, kMergePieceNs = 26;
+constexpr int kSplitCandidates = 32;
+// candidate i: the longest range (`longest` key tiles) divided by 1, 1.25, ... 48
+__host__ __device__ inline int split_candidate(int i, int longest) {
+  const int q[kSplitCandidates] = {4, 5, 6, 7, 8, 9, 10, 11, 12, 14, 16, 18, 20, 22, 24, 26, 28, 32, 36, 40, 44, 48, 56,
+                                   64, 72, 80, 96, 112, 128, 144, 160, 192};     // quarters
+  return (int)((4ll * longest + q[i] - 1) / q[i]);
+}
+struct SplitStat { long long work; int items, parts, longest; };
+__host__ __device__ inline void split_stat_add(SplitStat& s, const ReqGeom& g, int n_kv_heads, int ct) {
+  if (g.nt <= 0) return;
+  const int nch = (g.nt + ct - 1) / ct, len = (g.nt + nch - 1) / nch, fixed = nch > 1 ? kPieceNs : kItemNs;
+  const int pairs = g.nfull * n_kv_heads, duals = g.nunits - pairs;
+  s.work += (long long)g.nt * (pairs * kTileNs + duals * kTileDualNs) + (long long)g.nunits * nch * fixed;
+  s.items += g.nunits * nch;
+  s.parts += nch > 1 ? g.nunits * nch : 0;
+  const int item = len * (duals > 0 ? kTileDualNs : kTileNs) + fixed;
+  s.longest = item > s.longest ? item : s.longest;
+}
+// -1: not allowed (more pieces than the workspace holds)
+__host__ __device__ inline long long split_estimate(const SplitStat& s, int max_parts) {
+  if (s.parts > max_parts) return -1;
+  const long long even = s.work / kSms, waves = (s.items + kSms - 1) / kSms;
+  const long long over = s.items > 0 ? waves * s.work / s.items - even : 0;
+  long long e = even + (waves >= 3 ? over / 2 : over);
+  e = e < s.longest ? s.longest : e;
+  return e + (s.parts ? kMergeNs + (long long)kMergePieceNs * s.parts : 0);
+}
+// The chosen candidate's chunk length, or the filler rule where it pays.
+__host__ __device__ inline SplitRule split_auto(int total, int units, int ct) {
+  SplitRule s = split_rule(total, units, kDefaultTargetItems, kDefaultMinChunkTiles);
+  if (s.fine_from != 0x7fffffff && units >= kDefaultTargetItems) {
+    const long long half_item = (long long)total / units * kTileNs / 2;
+    const long long pieces = (long long)kFillerPercent * total / 100 / s.fine_ct;
+    if (half_item > 2 * (pieces * kPieceNs / kSms + kMergeNs + kMergePieceNs * pieces)) return s;
+  }
+  s.ct = ct; s.fine_ct = ct; s.fine_from = 0x7fffffff;
+  return s;
+}
+
 // One request under the rule: its first `ufine` units take chunks of ct, the others (work
 // offset >= fine_from) chunks of fine_ct.  wbase = work offset of the request's first unit.
 struct ReqSplit {
@@ -158,6 +211,8 @@ struct fb_ctx {
   int tokens_per_tile;  // 128 / G
   int target_items;       // list 0; list 1 aims for target_items / 2 (half as many executors)
   int min_chunk_tiles;
+  int auto_split;         // no target given: the split is chosen by estimate (list 0)
+  int auto_min_chunk;
   int pair_on;            // quads go to the CTA-pair kernel (bf16 pages, head_dim 128)
   long long wait_cycles;  // limit of every bounded device-side wait, in SM clock cycles
   float sm_scale;
@@ -242,7 +297,7 @@ int launch_gate(fb_ctx*, const fb_pack*, const int32_t* slot_stats, const fb_sta
 
 constexpr long long kDefaultWaitCycles = 2000000000LL;   // about a second at the SM clock
 
-fb::WsLayout make_ws_layout(const fb_config& c, int tiles_per_slot, int target_items, int min_chunk_tiles, int pair_on);
+fb::WsLayout make_ws_layout(const fb_ctx* ctx);
 int launch_attn_pair(fb_ctx*, const int32_t* page_table, void* out, void* ws, int32_t* status, cudaStream_t);
 int attn_pair_device_setup(fb_ctx*);
 int check_state(fb_ctx* ctx, const fb_state* st);   // every member non-null, else FB_ERR_INVALID_ARG

@@ -25,6 +25,7 @@ struct PackParams {
   int32_t pair_on;
   int32_t max_requests, wmax, bl, max_slots, max_blocks, mask_id, n_kv_heads;
   int32_t tiles_per_slot, tokens_per_tile, min_chunk_tiles;
+  int32_t auto_split, auto_min_chunk;
   int32_t resident;   // window K/V live in the pages: key tiles follow absolute positions
   int32_t n_gather_blocks;
 };
@@ -122,28 +123,53 @@ __device__ void build_sched(const PackParams& p, const int list) {
   const int max_items = p.max_items[list], max_units = p.max_units[list], max_parts = p.max_parts[list];
   __shared__ int sh_scan[kPackThreads / 32 + 1];
   __shared__ int bins[kCostBins];
-  __shared__ int sh_total, sh_units, sh_chunks;
+  __shared__ int sh_total, sh_units, sh_chunks, sh_longest;
+  __shared__ unsigned long long sh_best;
   __shared__ SplitRule sh_rule;
   const int tid = threadIdx.x;
   // bad states are reported once, by the gather blocks (null status here)
   // phase 1: total key-tile work -> chunk length
-  int mine = 0, mine_units = 0;
+  int mine = 0, mine_units = 0, mine_longest = 0;
   for (int r = tid; r < p.max_requests; r += kPackThreads) {
     ReqGeom g = req_geom(p, r, nullptr, list);
     mine += g.nunits * g.nt;
     mine_units += g.nt ? g.nunits : 0;
+    mine_longest = max(mine_longest, g.nt);
   }
-  if (tid == 0) { sh_total = 0; sh_units = 0; sh_chunks = 0; }
+  if (tid == 0) { sh_total = 0; sh_units = 0; sh_chunks = 0; sh_longest = 0; sh_best = ~0ull; }
   for (int i = tid; i < kCostBins; i += kPackThreads) bins[i] = 0;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     mine += __shfl_xor_sync(0xffffffffu, mine, o);
     mine_units += __shfl_xor_sync(0xffffffffu, mine_units, o);
+    mine_longest = max(mine_longest, __shfl_xor_sync(0xffffffffu, mine_longest, o));
   }
   __syncthreads();
-  if ((tid & 31) == 0) { atomicAdd(&sh_total, mine); atomicAdd(&sh_units, mine_units); }
+  if ((tid & 31) == 0) { atomicAdd(&sh_total, mine); atomicAdd(&sh_units, mine_units); atomicMax(&sh_longest, mine_longest); }
   __syncthreads();
-  if (tid == 0) sh_rule = split_rule(sh_total, sh_units, p.target_items[list], p.min_chunk_tiles);
+  if (list == 0 && p.auto_split) {
+    // one warp per candidate chunk length; the least (estimate, candidate) wins
+    static_assert(kPackThreads / 32 == kSplitCandidates, "one warp per candidate");
+    const int cand = tid >> 5, ct = max(split_candidate(cand, sh_longest), 1);
+    if (cand == 0 || ct >= p.auto_min_chunk) {
+      SplitStat st{};
+      for (int r = tid & 31; r < p.max_requests; r += 32) split_stat_add(st, req_geom(p, r, nullptr, list), p.n_kv_heads, ct);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        st.work += __shfl_xor_sync(0xffffffffu, st.work, o);
+        st.items += __shfl_xor_sync(0xffffffffu, st.items, o);
+        st.parts += __shfl_xor_sync(0xffffffffu, st.parts, o);
+        st.longest = max(st.longest, __shfl_xor_sync(0xffffffffu, st.longest, o));
+      }
+      const long long e = split_estimate(st, max_parts);
+      if ((tid & 31) == 0 && e >= 0) atomicMin(&sh_best, ((unsigned long long)e << 8) | (unsigned)cand);
+    }
+    __syncthreads();
+    if (tid == 0)
+      sh_rule = split_auto(sh_total, sh_units, max(split_candidate((int)(sh_best & 0xff) % kSplitCandidates, sh_longest), 1));
+  } else if (tid == 0) {
+    sh_rule = split_rule(sh_total, sh_units, p.target_items[list], p.min_chunk_tiles);
+  }
   __syncthreads();
   const SplitRule rule = sh_rule;
   // phase 2 + 3: per-request bases (chunked scan), then one thread per unit of the chunk's
@@ -242,7 +268,7 @@ __device__ void build_sched(const PackParams& p, const int list) {
       hdr->chunk_tiles = rule.ct;
       hdr->n_parts = mult * part_run;
       hdr->total_tiles = sh_total;
-      hdr->ticket = 0; hdr->max_chunks = sh_chunks;
+      hdr->ticket = 0; hdr->done = 0; hdr->max_chunks = sh_chunks;
       if (total_items > max_items || mult * unit_run > max_units || mult * part_run > max_parts)
         atomicOr(p.status, FB_ST_BAD_STATE);
     }
@@ -345,6 +371,7 @@ int launch_pack(fb_ctx* ctx, const fb_state* st, const fb_pack* out, void* ws, i
   p.n_kv_heads = c.n_kv_heads; p.tiles_per_slot = ctx->tiles_per_slot;
   p.tokens_per_tile = ctx->tokens_per_tile;
   p.min_chunk_tiles = ctx->min_chunk_tiles;
+  p.auto_split = ctx->auto_split; p.auto_min_chunk = ctx->auto_min_chunk;
   p.resident = ctx->cfg.window_in_pages;
   p.n_gather_blocks = (p.max_slots + kSlotsPerBlock - 1) / kSlotsPerBlock;
   // one more block per work list in use (the CTA-pair kernel's list only when that kernel is on)

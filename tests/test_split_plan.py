@@ -1,0 +1,69 @@
+"""The split of the key axis that is chosen by estimate: the device builds the list that the host
+mirror of the arithmetic announces, whatever the batch (few or many units, short or long, with
+leftover tiles, more requests than one pass of the scheduler block), and the attention over
+it agrees with the unsplit one."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2607_17652_b200 import binding as B
+from paper_2607_17652_b200 import synth
+
+DEV = "cuda:0"
+
+
+def _cfg(**over):
+    return dict(dict(max_requests=64, wmax=4, block_len=32, n_q_heads=32, n_kv_heads=8, head_dim=128, page_size=64,
+                     num_pages=64 * 520, max_pages_per_req=520, vocab=1024, mask_id=1023, eos_id=1022, max_blocks=32,
+                     s_pe=1, tau_mask=0.9, tau_edit=0.95, theta_spawn=0.5, sm_scale=0.0), **over)
+
+
+def test_estimated_split_fits_and_leaves_nothing_out():
+    rg = np.random.default_rng(11)
+    ctx = B.Context(**_cfg())
+    for _ in range(400):
+        n = int(rg.integers(1, 65))
+        P = rg.integers(0, int(2 ** rg.uniform(5, 15)), size=n)
+        w = rg.integers(0, 5, size=n)
+        pl = ctx.attn_plan(P, w)
+        assert pl["parts"] <= pl["max_parts"] and pl["units"] <= pl["max_units"] and pl["items"] <= pl["max_items"], pl
+        assert pl["items"] >= pl["units"]
+    # 160 long units for 148 SMs: the second wave would run nearly empty, pieces fill it
+    assert ctx.attn_plan([16000] * 10, [4] * 10)["parts"] > 0
+    # three full waves of short items: nothing to gain
+    assert ctx.attn_plan([300] * 28, [4] * 28)["parts"] == 0
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n_requests,prefix,w,resident", [
+    (1, (64, 64), (2, 2), 0), (1, (3001, 3001), (1, 1), 1), (2, (9000, 12000), (3, 3), 0), (9, (100, 2500), (1, 4), 1),
+    (20, (1500, 4000), (1, 3), 0), (60, (100, 900), (1, 4), 0), (1100, (1, 200), (1, 1), 0)])
+def test_device_builds_the_announced_list(n_requests, prefix, w, resident):
+    wl = synth.tiny_workload(n_requests=n_requests, wmax=4, w_lo=w[0], w_hi=w[1], prefix_lo=prefix[0],
+                             prefix_hi=prefix[1], head_dim=128, n_q_heads=12, n_kv_heads=3)
+    stc = synth.make_structure(wl)
+    tokens = synth.make_tokens(stc)
+    q, kw, vw, kp, vp = (t.to(DEV) for t in synth.make_attn_inputs(stc))
+    if resident:
+        kw = vw = None
+    outs = []
+    for tuning in (None, dict(attn_target_items=1)):
+        ctx = B.Context(tuning=tuning, **synth.config_dict(stc, window_in_pages=resident))
+        st = B.DeviceState.from_numpy(DEV, stc.active, stc.prefix_len, stc.L, stc.R, tokens,
+                                      np.zeros((wl.n_requests, wl.wmax), np.uint8), stc.page_table)
+        pk = B.PackBuffers.alloc(ctx, DEV)
+        sb = B.StepBuffers(ctx, DEV)
+        B.fb_pack_wavefronts(ctx, st, pk, sb.ws, sb.status)
+        for _ in range(2):                        # the work ticket is re-armed by the launch itself
+            sb.out.fill_(7.0)
+            B.fb_wavefront_attn(ctx, pk, q, kw, vw, kp, vp, st.page_table, sb.out, sb.ws, sb.status)
+        torch.cuda.synchronize()
+        assert int(sb.status.item()) == 0
+        hdr = sb.ws[:64].cpu().numpy().view(np.int32)          # n_items, n_units, chunk length, n_parts
+        plan = ctx.attn_plan(stc.prefix_len, stc.R - stc.L)
+        assert (int(hdr[1]), int(hdr[0]), int(hdr[3])) == (plan["units"], plan["items"], plan["parts"])
+        outs.append(sb.out.float())
+    # two schedules of the same sums: the weights are rounded to bf16 against different references
+    # (2^-9 each) and the output once more
+    err = float((outs[0] - outs[1]).norm() / outs[1].norm())
+    assert err <= 4 * 2 ** -9, err
