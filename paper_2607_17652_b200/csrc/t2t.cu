@@ -229,13 +229,16 @@ __global__ void __launch_bounds__(128) t2t_update_kernel(const UpdParams p) {
   const int slot = blockIdx.x * 4 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (slot >= p.max_slots) return;
-  if (slot >= *p.n_live) {
+  // what does not depend on another load, together (the first 32 positions of the block)
+  const int n_live = *p.n_live, r = p.slot_req[slot], s0 = p.slot_s[slot];
+  const int xh0 = lane < p.bl ? p.argmax[slot * p.bl + lane] : 0;
+  const float pr0 = lane < p.bl ? p.conf[slot * p.bl + lane] : 0.f;
+  if (slot >= n_live) {
     for (int t = lane; t < p.bl; t += 32) p.action[slot * p.bl + t] = 0;
     if (lane < FB_SLOT_STATS) p.slot_stats[slot * FB_SLOT_STATS + lane] = 0;
     return;
   }
-  const int r = p.slot_req[slot];
-  const int g = p.L[r] + p.slot_s[slot];
+  const int g = p.L[r] + s0;
   int32_t* tok = p.tokens + (size_t)r * p.max_blocks * p.bl + (size_t)g * p.bl;
   int m0 = 0, rdy = 0, m2t = 0, t2t = 0, m1 = 0, eos = 0;
   float bestp = -1.f;                               // most confident mask this lane left in place
@@ -243,8 +246,8 @@ __global__ void __launch_bounds__(128) t2t_update_kernel(const UpdParams p) {
   for (int t = lane; t < p.bl; t += 32) {
     const int i = slot * p.bl + t;
     int x = tok[t];
-    const int xh = p.argmax[i];
-    const float pr = p.conf[i];
+    const int xh = t == lane ? xh0 : p.argmax[i];
+    const float pr = t == lane ? pr0 : p.conf[i];
     uint8_t act = FB_ACT_NONE;
     if (x == p.mask_id) {                         // Gamma of Eq. 1: strict >
       m0++;
@@ -272,7 +275,7 @@ __global__ void __launch_bounds__(128) t2t_update_kernel(const UpdParams p) {
   }
   // forced progress: the oldest block went in with masks and Eq. 1 revealed none -> its most
   // confident masked position (lowest position on ties) is revealed
-  if (p.force_progress && p.slot_s[slot] == 0 && m0 > 0 && m2t == 0) {
+  if (p.force_progress && s0 == 0 && m0 > 0 && m2t == 0) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       const float op = __shfl_xor_sync(0xffffffffu, bestp, o);
