@@ -192,9 +192,10 @@ int fb_attn_plan_host(const fb_ctx* ctx, const int32_t* h_prefix_len, const int3
     if (total > 0x7fffffffll) return fail(nullptr, FB_ERR_UNSUPPORTED, "fb_attn_plan_host: work list too long");
     fb::SplitRule rule = fb::split_rule((int)total, (int)units, target, ctx->min_chunk_tiles);
     if (list == 0 && ctx->auto_split) {
-      long long best = -1;
+      float best = -1.f;
       int ct = longest > 0 ? longest : 1;
-      for (int i = 0; i < fb::kSplitCandidates; ++i) {
+      const bool estimate = fb::split_worth_estimating((int)total, (int)units, longest);
+      for (int i = 0; i < (estimate ? fb::kSplitCandidates : 0); ++i) {
         const int cand = fb::split_candidate(i, longest);
         if (i > 0 && cand < ctx->auto_min_chunk) continue;
         fb::SplitStat st{};
@@ -202,8 +203,8 @@ int fb_attn_plan_host(const fb_ctx* ctx, const int32_t* h_prefix_len, const int3
           fb::split_stat_add(st, fb::req_geom_of(h_live_blocks[r], h_prefix_len[r], ctx->tiles_per_slot, c.block_len,
                                                  c.n_kv_heads, c.window_in_pages, list, ctx->pair_on),
                              c.n_kv_heads, cand > 0 ? cand : 1);
-        const long long e = fb::split_estimate(st, ctx->ws.l[0].max_parts);
-        if (e >= 0 && (best < 0 || e < best)) { best = e; ct = cand > 0 ? cand : 1; }
+        const float e = fb::split_estimate(st, ctx->ws.l[0].max_parts);
+        if (e >= 0.f && (best < 0.f || e < best)) { best = e; ct = cand > 0 ? cand : 1; }
       }
       rule = fb::split_auto((int)total, (int)units, ct);
     }

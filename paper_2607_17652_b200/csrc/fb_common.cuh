@@ -129,47 +129,58 @@ __host__ __device__ inline SplitRule split_rule(int total, int units, int target
 //   makespan = max(W / SMs, longest item, waves * W / items) + merge,
 // W the work of all items.  A batch of equal items that just misses whole waves pays for the last
 // one in full; from three waves on handing out longest first fills half of that in.  The costs
-// are measured (ns): a key tile of a pair, of two K/V streams; what an item costs beside its
-// tiles, whole or as a piece; the merge, once and per piece.  Against always aiming at two items
+// are measured (in units of 100 ns; the merge per piece in ns): a key tile of a pair, of two K/V
+// streams; what an item costs beside its tiles, whole or as a piece; the merge.  Against always aiming at two items
 // an SM: 28,000-token request 72 -> 64 us, 24 requests of 700 to 5,000 tokens 161 -> 151 (not split
 // at all), 8 requests 24.6 (the same split).
+// With four whole items an SM and more, none longer than half of an SM's share, the estimate is skipped
+// (longest items first leave nothing to gain that a split would not cost): the pack kernel takes
+// 2 to 3 us less on 64 and 128 requests.
 // With two units an SM and more, and items so long that half of one outweighs their cost twice,
 // the last 15 % of the work are cut into filler pieces as above (16 long contexts: 1064 -> 1030).
-constexpr int kTileNs = 1600, kTileDualNs = 2200, kItemNs = 4000, kPieceNs = 4500, kMergeNs = 5000, kMergePieceNs = 26;
+constexpr int kTileCost = 16, kTileDualCost = 22, kItemCost = 40, kPieceCost = 45, kMergeCost = 50, kMergePieceNs = 26;
 constexpr int kSplitCandidates = 32;
-// candidate i: the longest range (`longest` key tiles) divided by 1, 1.25, ... 48
+// Candidate i: the longest range (`longest` key tiles) divided by 1, 1.25, 1.5, 1.75, 2, 2.25, 2.5,
+// 2.75, 3, 3.5, 4, 4.5, 5, 5.5, 6, 6.5, 7, 8, 9, 10, 11, 12, 14, 16, 18, 20, 24, 28, 32, 36, 40, 48
+// (quarters, a byte each).
 __host__ __device__ inline int split_candidate(int i, int longest) {
-  const int q[kSplitCandidates] = {4, 5, 6, 7, 8, 9, 10, 11, 12, 14, 16, 18, 20, 22, 24, 26, 28, 32, 36, 40, 44, 48, 56,
-                                   64, 72, 80, 96, 112, 128, 144, 160, 192};     // quarters
-  return (int)((4ll * longest + q[i] - 1) / q[i]);
+  const unsigned long long w = i < 8 ? 795458214266537220ull : i < 16 ? 1880277119885381132ull : i < 24 ? 4627501583333335068ull : 13880252932871442504ull;
+  const unsigned q = (unsigned)(w >> (8 * (i & 7))) & 0xffu;
+  return (int)((4u * (unsigned)longest + q - 1u) / q);
 }
-struct SplitStat { long long work; int items, parts, longest; };
+struct SplitStat { unsigned work; int items, parts, longest; };
 __host__ __device__ inline void split_stat_add(SplitStat& s, const ReqGeom& g, int n_kv_heads, int ct) {
   if (g.nt <= 0) return;
-  const int nch = (g.nt + ct - 1) / ct, len = (g.nt + nch - 1) / nch, fixed = nch > 1 ? kPieceNs : kItemNs;
+  const int nch = (g.nt + ct - 1) / ct, len = (g.nt + nch - 1) / nch, fixed = nch > 1 ? kPieceCost : kItemCost;
   const int pairs = g.nfull * n_kv_heads, duals = g.nunits - pairs;
-  s.work += (long long)g.nt * (pairs * kTileNs + duals * kTileDualNs) + (long long)g.nunits * nch * fixed;
+  s.work += (unsigned)g.nt * (unsigned)(pairs * kTileCost + duals * kTileDualCost) + (unsigned)(g.nunits * nch * fixed);
   s.items += g.nunits * nch;
   s.parts += nch > 1 ? g.nunits * nch : 0;
-  const int item = len * (duals > 0 ? kTileDualNs : kTileNs) + fixed;
+  const int item = len * (duals > 0 ? kTileDualCost : kTileCost) + fixed;
   s.longest = item > s.longest ? item : s.longest;
 }
-// -1: not allowed (more pieces than the workspace holds)
-__host__ __device__ inline long long split_estimate(const SplitStat& s, int max_parts) {
-  if (s.parts > max_parts) return -1;
-  const long long even = s.work / kSms, waves = (s.items + kSms - 1) / kSms;
-  const long long over = s.items > 0 ? waves * s.work / s.items - even : 0;
-  long long e = even + (waves >= 3 ? over / 2 : over);
-  e = e < s.longest ? s.longest : e;
-  return e + (s.parts ? kMergeNs + (long long)kMergePieceNs * s.parts : 0);
+// As a float whose operations round alike on the host and on the device (no product that
+// feeds a sum is inexact).  Negative: not allowed (more pieces than the workspace holds).
+__host__ __device__ inline float split_estimate(const SplitStat& s, int max_parts) {
+  if (s.parts > max_parts || s.items <= 0) return -1.f;
+  const float work = (float)s.work, even = work / (float)kSms;
+  const int waves = (s.items + kSms - 1) / kSms;
+  const float over = work / (float)s.items * (float)waves;
+  float e = waves >= 3 ? 0.5f * (even + over) : (over > even ? over : even);
+  e = e < (float)s.longest ? (float)s.longest : e;
+  return s.parts ? e + (float)(kMergeCost + kMergePieceNs * s.parts / 100) : e;
+}
+__host__ __device__ inline bool split_worth_estimating(int total, int units, int longest) {
+  return units < 4 * kSms || longest > total / (2 * kSms);
 }
 // The chosen candidate's chunk length, or the filler rule where it pays.
 __host__ __device__ inline SplitRule split_auto(int total, int units, int ct) {
-  SplitRule s = split_rule(total, units, kDefaultTargetItems, kDefaultMinChunkTiles);
-  if (s.fine_from != 0x7fffffff && units >= kDefaultTargetItems) {
-    const long long half_item = (long long)total / units * kTileNs / 2;
-    const long long pieces = (long long)kFillerPercent * total / 100 / s.fine_ct;
-    if (half_item > 2 * (pieces * kPieceNs / kSms + kMergeNs + kMergePieceNs * pieces)) return s;
+  SplitRule s;
+  if (units >= kDefaultTargetItems) {
+    s = split_rule(total, units, kDefaultTargetItems, kDefaultMinChunkTiles);
+    const int pieces = total / 100 * kFillerPercent / s.fine_ct;
+    if (s.fine_from != 0x7fffffff &&
+        total / units * (kTileCost / 4) > pieces * kPieceCost / kSms + pieces * kMergePieceNs / 100 + kMergeCost) return s;
   }
   s.ct = ct; s.fine_ct = ct; s.fine_from = 0x7fffffff;
   return s;

@@ -10,9 +10,13 @@
 
 namespace fb {
 
-constexpr int kPackThreads = 1024;
+// Threads per block: bound by latency (dependent loads, block barriers), so small batches take
+// small blocks: call in us with 256 / 512 / 1024 threads, 1 request 5.5 / 6.0 / 7.0, 8 requests 5.9 /
+// 6.6 / 7.6, 24 requests 8.6 / 8.0 / 8.9, 128 requests 19.0 / 16.9 / 17.2.
+constexpr int kPackThreads = 512, kPackThreadsSmall = 256, kPackSmallRequests = 8;
 constexpr int kSlotsPerBlock = 32;
 constexpr int kCostBins = 1024;
+constexpr int kUnitInfo = 1024;       // units whose geometry stays in shared memory between the two passes over items
 
 struct PackParams {
   const int32_t *active, *prefix_len, *L, *R, *tokens;
@@ -30,10 +34,10 @@ struct PackParams {
   int32_t n_gather_blocks;
 };
 
-// live-block count of request r, sanitised to [0, wmax]
+// live-block count of request r, sanitised to [0, wmax]; the loads do not wait for one another
 __device__ __forceinline__ int live_blocks(const PackParams& p, int r, int32_t* status) {
-  if (p.active[r] != 1) return 0;
-  const int L = p.L[r], R = p.R[r];
+  const int active = p.active[r], L = p.L[r], R = p.R[r];
+  if (active != 1) return 0;
   int w = R - L;
   if (L < 0 || R > p.max_blocks || w < 0 || w > p.wmax) {
     if (status) atomicOr(status, FB_ST_BAD_STATE);
@@ -43,32 +47,38 @@ __device__ __forceinline__ int live_blocks(const PackParams& p, int r, int32_t* 
   return w;
 }
 
-// exclusive block scan of one value per thread; returns the exclusive prefix,
-// *total = block sum.  All threads must call.
-__device__ __forceinline__ int block_excl_scan(int v, int* total, int* sh /*[kPackThreads/32 + 1]*/) {
+// Exclusive block scan of N values per thread: excl = prefix, tot = block sum.  All threads must
+// call; `sh` [N * T / 32] must not be in use by an earlier scan (one barrier inside).
+template <int T, int N>
+__device__ __forceinline__ void block_excl_scan(const int (&v)[N], int (&excl)[N], int (&tot)[N], int* sh) {
+  constexpr int NW = T / 32;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int x = v;
+  int x[N];
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    int y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
-  __syncthreads();
-  if (lane == 31) sh[warp] = x;
-  __syncthreads();
-  if (warp == 0) {
-    int w = lane < kPackThreads / 32 ? sh[lane] : 0;
+  for (int n = 0; n < N; ++n) x[n] = v[n];
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      int y = __shfl_up_sync(0xffffffffu, w, o);
+  for (int o = 1; o < 32; o <<= 1)
+#pragma unroll
+    for (int n = 0; n < N; ++n) {
+      const int y = __shfl_up_sync(0xffffffffu, x[n], o);
+      if (lane >= o) x[n] += y;
+    }
+  if (lane == 31)
+#pragma unroll
+    for (int n = 0; n < N; ++n) sh[n * NW + warp] = x[n];
+  __syncthreads();
+#pragma unroll
+  for (int n = 0; n < N; ++n) {
+    int w = lane < NW ? sh[n * NW + lane] : 0;       // every warp scans the warp sums
+#pragma unroll
+    for (int o = 1; o < NW; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, w, o);
       if (lane >= o) w += y;
     }
-    if (lane < kPackThreads / 32) sh[lane] = w;   // inclusive warp sums
+    tot[n] = __shfl_sync(0xffffffffu, w, NW - 1);
+    const int before = __shfl_sync(0xffffffffu, w, warp == 0 ? 0 : warp - 1);
+    excl[n] = x[n] - v[n] + (warp == 0 ? 0 : before);
   }
-  __syncthreads();
-  const int base = warp == 0 ? 0 : sh[warp - 1];
-  *total = sh[kPackThreads / 32 - 1];
-  return base + x - v;
 }
 
 // Sort key of a work item: its key-tile iterations; an iteration with two Q
@@ -81,9 +91,10 @@ __device__ __forceinline__ int item_cost(int nA, int nB) {
 __device__ __forceinline__ ReqGeom geom_of(const PackParams& p, int w, int prefix_len, int list) {
   return req_geom_of(w, prefix_len, p.tiles_per_slot, p.bl, p.n_kv_heads, p.resident, list, p.pair_on);
 }
-__device__ __forceinline__ ReqGeom req_geom(const PackParams& p, int r, int32_t* status, int list) {
-  const int w = live_blocks(p, r, status);
-  return geom_of(p, w, w ? p.prefix_len[r] : 0, list);
+__device__ __forceinline__ ReqGeom req_geom(const PackParams& p, int r, int list) {
+  const int P = p.prefix_len[r];
+  const int w = live_blocks(p, r, nullptr);      // (bad states are reported once, by the gather blocks)
+  return geom_of(p, w, w ? P : 0, list);
 }
 
 // unit record of two Q tiles qa, qb (absolute tile indices of the request; qb < 0: none) under
@@ -115,29 +126,38 @@ __device__ __forceinline__ AttnUnit make_unit(const PackParams& p, const ReqGeom
 // `list` 0: pairs of tiles and leftover tiles, one record per scheduling unit.  `list` 1: quads,
 // two records per scheduling unit (2u for the first CTA of the pair, 2u + 1 for the second), both
 // cut into the same chunks; an item names record 2u.
+template <int T>
 __device__ void build_sched(const PackParams& p, const int list) {
   const int mult = list + 1;            // unit records (and partial-result ranges) per scheduling unit
   SchedHeader* const hdr = p.hdr[list];
   AttnItem* const items = p.items[list];
   AttnUnit* const units = p.units[list];
   const int max_items = p.max_items[list], max_units = p.max_units[list], max_parts = p.max_parts[list];
-  __shared__ int sh_scan[kPackThreads / 32 + 1];
+  __shared__ int sh_scan[3 * T / 32], sh_scan2[T / 32], sh_scan3[T / 32];
   __shared__ int bins[kCostBins];
   __shared__ int sh_total, sh_units, sh_chunks, sh_longest;
-  __shared__ unsigned long long sh_best;
+  __shared__ SplitStat sh_stat[kSplitCandidates];
+  static_assert(kSplitCandidates == 32, "one lane per candidate");
   __shared__ SplitRule sh_rule;
+  __shared__ int s_ub[T + 1], s_pb[T], s_first[T], s_wb[T], s_w[T], s_P[T];
+  __shared__ int4 s_info[kUnitInfo];
   const int tid = threadIdx.x;
-  // bad states are reported once, by the gather blocks (null status here)
-  // phase 1: total key-tile work -> chunk length
+  if (tid == 0) { sh_total = 0; sh_units = 0; sh_chunks = 0; sh_longest = 0; }
+  if (tid < kSplitCandidates) sh_stat[tid] = SplitStat{};
+  for (int i = tid; i < kCostBins; i += T) bins[i] = 0;
+  // phase 1: total key-tile work, longest key range -> chunk length.  The requests' geometry is
+  // loaded once where one pass over the requests holds all of them.
+  const bool one_pass = p.max_requests <= T;
+  ReqGeom g0{};
   int mine = 0, mine_units = 0, mine_longest = 0;
-  for (int r = tid; r < p.max_requests; r += kPackThreads) {
-    ReqGeom g = req_geom(p, r, nullptr, list);
+  for (int r = tid; r < p.max_requests; r += T) {
+    const ReqGeom g = req_geom(p, r, list);
     mine += g.nunits * g.nt;
     mine_units += g.nt ? g.nunits : 0;
     mine_longest = max(mine_longest, g.nt);
+    g0 = g;
   }
-  if (tid == 0) { sh_total = 0; sh_units = 0; sh_chunks = 0; sh_longest = 0; sh_best = ~0ull; }
-  for (int i = tid; i < kCostBins; i += kPackThreads) bins[i] = 0;
+  s_w[tid] = g0.w; s_P[tid] = g0.P;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     mine += __shfl_xor_sync(0xffffffffu, mine, o);
@@ -145,62 +165,72 @@ __device__ void build_sched(const PackParams& p, const int list) {
     mine_longest = max(mine_longest, __shfl_xor_sync(0xffffffffu, mine_longest, o));
   }
   __syncthreads();
-  if ((tid & 31) == 0) { atomicAdd(&sh_total, mine); atomicAdd(&sh_units, mine_units); atomicMax(&sh_longest, mine_longest); }
+  if ((tid & 31) == 0 && mine_units) {
+    atomicAdd(&sh_total, mine); atomicAdd(&sh_units, mine_units); atomicMax(&sh_longest, mine_longest);
+  }
   __syncthreads();
-  if (list == 0 && p.auto_split) {
-    // one warp per candidate chunk length; the least (estimate, candidate) wins
-    static_assert(kPackThreads / 32 == kSplitCandidates, "one warp per candidate");
-    const int cand = tid >> 5, ct = max(split_candidate(cand, sh_longest), 1);
-    if (cand == 0 || ct >= p.auto_min_chunk) {
-      SplitStat st{};
-      for (int r = tid & 31; r < p.max_requests; r += 32) split_stat_add(st, req_geom(p, r, nullptr, list), p.n_kv_heads, ct);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        st.work += __shfl_xor_sync(0xffffffffu, st.work, o);
-        st.items += __shfl_xor_sync(0xffffffffu, st.items, o);
-        st.parts += __shfl_xor_sync(0xffffffffu, st.parts, o);
-        st.longest = max(st.longest, __shfl_xor_sync(0xffffffffu, st.longest, o));
-      }
-      const long long e = split_estimate(st, max_parts);
-      if ((tid & 31) == 0 && e >= 0) atomicMin(&sh_best, ((unsigned long long)e << 8) | (unsigned)cand);
+  if (list == 0 && p.auto_split && !split_worth_estimating(sh_total, sh_units, sh_longest)) {
+    if (tid == 0) sh_rule = split_auto(sh_total, sh_units, max(sh_longest, 1));
+  } else if (list == 0 && p.auto_split) {
+    // every lane a candidate chunk length, the requests dealt to the warps; then the least
+    // (estimate, candidate) wins
+    const int lane = tid & 31, ct = max(split_candidate(lane, sh_longest), 1);
+    SplitStat st{};
+    for (int r = tid >> 5; r < p.max_requests; r += T / 32)
+      split_stat_add(st, one_pass ? geom_of(p, s_w[r], s_P[r], list) : req_geom(p, r, list), p.n_kv_heads, ct);
+    if (st.items) {
+      atomicAdd(&sh_stat[lane].work, st.work); atomicAdd(&sh_stat[lane].items, st.items);
+      atomicAdd(&sh_stat[lane].parts, st.parts); atomicMax(&sh_stat[lane].longest, st.longest);
     }
     __syncthreads();
-    if (tid == 0)
-      sh_rule = split_auto(sh_total, sh_units, max(split_candidate((int)(sh_best & 0xff) % kSplitCandidates, sh_longest), 1));
+    if (tid < 32) {
+      const float e = lane > 0 && ct < p.auto_min_chunk ? -1.f : split_estimate(sh_stat[lane], max_parts);
+      // (non-negative floats order like their bits; nothing to do at all: candidate 0)
+      unsigned best = e >= 0.f ? __float_as_uint(e) : 0xffffffffu;
+      int at = lane;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const unsigned b2 = __shfl_xor_sync(0xffffffffu, best, o);
+        const int a2 = __shfl_xor_sync(0xffffffffu, at, o);
+        if (b2 < best || (b2 == best && a2 < at)) { best = b2; at = a2; }
+      }
+      const int chosen = __shfl_sync(0xffffffffu, ct, at);
+      if (lane == 0) sh_rule = split_auto(sh_total, sh_units, chosen);
+    }
   } else if (tid == 0) {
     sh_rule = split_rule(sh_total, sh_units, p.target_items[list], p.min_chunk_tiles);
   }
   __syncthreads();
   const SplitRule rule = sh_rule;
-  // phase 2 + 3: per-request bases (chunked scan), then one thread per unit of the chunk's
-  // requests: unit record, cost histogram of its items
-  __shared__ int s_ub[kPackThreads + 1], s_pb[kPackThreads], s_first[kPackThreads], s_wb[kPackThreads],
-      s_w[kPackThreads], s_P[kPackThreads];
-  int unit_run = 0, part_run = 0, item_run = 0, slot_run = 0, work_run = 0;
-  for (int r0 = 0; r0 < p.max_requests; r0 += kPackThreads) {
+  // phase 2 + 3: per-request bases (scan over up to T requests at a time), then the units of
+  // these requests: unit record, cost histogram of its items.  A unit cut into many pieces is
+  // given to several threads.
+  int unit_run = 0, part_run = 0, slot_run = 0, work_run = 0, lanes = 1;
+  for (int r0 = 0; r0 < p.max_requests; r0 += T) {
     const int r = r0 + tid;
     ReqGeom g{};
-    int nunits = 0;
-    if (r < p.max_requests) {
-      g = req_geom(p, r, nullptr, list);
-      nunits = g.nt ? g.nunits : 0;
-    }
-    int tu, tp, ti, ts, tw;
-    const int wbase = work_run + block_excl_scan(nunits * g.nt, &tw, sh_scan);
-    work_run += tw;
+    if (one_pass) g = g0;
+    else if (r < p.max_requests) g = req_geom(p, r, list);
+    const int nunits = g.nt ? g.nunits : 0;
+    int pre[3], tot[3];
+    block_excl_scan<T, 3>({nunits * g.nt, nunits, g.w}, pre, tot, sh_scan);
+    const int wbase = work_run + pre[0];
     const ReqSplit rs = req_split(rule, wbase, nunits, g.nt);
     if (nunits) atomicMax(&sh_chunks, max(rs.ufine > 0 ? rs.nch_c : 0, rs.ufine < nunits ? rs.nch_f : 0));
-    const int urel = block_excl_scan(nunits, &tu, sh_scan);
-    const int pbase = part_run + block_excl_scan(rs.parts(nunits), &tp, sh_scan);
-    block_excl_scan(rs.items(nunits), &ti, sh_scan);
-    const int first0 = slot_run + block_excl_scan(g.w, &ts, sh_scan);  // first slot of the request
-    s_ub[tid] = urel; s_pb[tid] = pbase; s_first[tid] = first0; s_wb[tid] = wbase; s_w[tid] = g.w; s_P[tid] = g.P;
-    if (tid == 0) s_ub[kPackThreads] = tu;
+    int ppre[1], ptot[1];
+    block_excl_scan<T, 1>({rs.parts(nunits)}, ppre, ptot, sh_scan2);
+    const int tu = tot[1];
+    s_ub[tid] = pre[1]; s_pb[tid] = part_run + ppre[0]; s_first[tid] = slot_run + pre[2]; s_wb[tid] = wbase;
+    if (!one_pass) { s_w[tid] = g.w; s_P[tid] = g.P; }
+    if (tid == 0) s_ub[T] = tu;
     __syncthreads();
-    for (int i = tid; i < tu; i += kPackThreads) {
+    lanes = 1;
+    while (lanes < 32 && lanes < sh_chunks && 2 * lanes * tu <= T) lanes *= 2;
+    for (int j = tid; j < tu * lanes; j += T) {
+      const int i = j / lanes, c0 = j % lanes;
       // the request of unit i: the last k with s_ub[k] <= i (requests without units share
       // their successor's base and are skipped by "last")
-      int lo = 0, hi = kPackThreads - 1;
+      int lo = 0, hi = min(T, p.max_requests - r0) - 1;
       while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
         if (s_ub[mid] <= i) lo = mid; else hi = mid - 1;
@@ -237,29 +267,31 @@ __device__ void build_sched(const PackParams& p, const int list) {
       for (int rr = 0; rr < mult; ++rr) {
         un[rr].n_chunks = nch;
         un[rr].part_base = nc > 1 ? pb + rr * nc : -1;
-        units[mult * u + rr] = un[rr];
+        if (c0 == 0) units[mult * u + rr] = un[rr];
         nvA = max(nvA, un[rr].nvisA); nvB = max(nvB, un[rr].nvisB);
       }
-      for (int c = 0; c < nch; ++c) {
+      if (c0 == 0 && u < kUnitInfo) s_info[u] = make_int4(nvA, nvB, q.nt, nch);
+      for (int c = c0; c < nch; c += lanes) {
         const int jb = c * q.nt / nc, je = (c + 1) * q.nt / nc;
         int cost = item_cost(max(0, min(je, nvA) - jb), max(0, min(je, nvB) - jb));
         atomicAdd(&bins[min(cost, kCostBins - 1)], 1);
       }
     }
-    unit_run += tu; part_run += tp; item_run += ti; slot_run += ts;
-    __syncthreads();                      // the chunk's tables are overwritten next
+    unit_run += tu; part_run += ptot[0]; slot_run += tot[2]; work_run += tot[0];
+    __syncthreads();                      // the tables are overwritten next
   }
-  __syncthreads();
   // descending exclusive offsets over the cost bins: thread t owns the bins
   // kCostBins-1-kBinsPer*t and below (largest cost first)
   {
-    constexpr int kBinsPer = kCostBins / kPackThreads;
-    static_assert(kBinsPer * kPackThreads == kCostBins && kBinsPer >= 1, "whole bins per thread");
+    constexpr int kBinsPer = kCostBins / T;
+    static_assert(kBinsPer * T == kCostBins && kBinsPer >= 1, "whole bins per thread");
     int c[kBinsPer], sum = 0;
 #pragma unroll
     for (int j = 0; j < kBinsPer; ++j) { c[j] = bins[kCostBins - 1 - (kBinsPer * tid + j)]; sum += c[j]; }
-    int total_items;
-    int base = block_excl_scan(sum, &total_items, sh_scan);
+    int bpre[1], btot[1];
+    block_excl_scan<T, 1>({sum}, bpre, btot, sh_scan3);
+    int base = bpre[0];
+    const int total_items = btot[0];
 #pragma unroll
     for (int j = 0; j < kBinsPer; ++j) { bins[kCostBins - 1 - (kBinsPer * tid + j)] = base; base += c[j]; }
     if (tid == 0) {
@@ -275,13 +307,22 @@ __device__ void build_sched(const PackParams& p, const int list) {
   }
   __syncthreads();
   // phase 4: scatter items, longest first
-  for (int u = tid; u < min(unit_run, max_units / mult); u += kPackThreads) {
-    const AttnUnit un = units[mult * u];
-    int nvA = un.nvisA, nvB = un.nvisB;
-    if (mult == 2) { const AttnUnit u1 = units[2 * u + 1]; nvA = max(nvA, u1.nvisA); nvB = max(nvB, u1.nvisB); }
-    const int nch = un.n_chunks;
-    for (int c = 0; c < nch; ++c) {
-      const int jb = c * un.n_tiles / nch, je = (c + 1) * un.n_tiles / nch;
+  const int n_sched = min(unit_run, max_units / mult);
+  lanes = 1;
+  while (lanes < 32 && lanes < sh_chunks && 2 * lanes * n_sched <= T) lanes *= 2;
+  for (int j = tid; j < n_sched * lanes; j += T) {
+    const int u = j / lanes;
+    int nvA, nvB, nt, nch;
+    if (u < kUnitInfo) {
+      const int4 f = s_info[u];
+      nvA = f.x; nvB = f.y; nt = f.z; nch = f.w;
+    } else {
+      const AttnUnit un = units[mult * u];
+      nvA = un.nvisA; nvB = un.nvisB; nt = un.n_tiles; nch = un.n_chunks;
+      if (mult == 2) { const AttnUnit u1 = units[2 * u + 1]; nvA = max(nvA, u1.nvisA); nvB = max(nvB, u1.nvisB); }
+    }
+    for (int c = j % lanes; c < nch; c += lanes) {
+      const int jb = c * nt / nch, je = (c + 1) * nt / nch;
       int cost = item_cost(max(0, min(je, nvA) - jb), max(0, min(je, nvB) - jb));
       const int at = atomicAdd(&bins[min(cost, kCostBins - 1)], 1);
       if (at < max_items) {
@@ -292,22 +333,25 @@ __device__ void build_sched(const PackParams& p, const int list) {
   }
 }
 
-__global__ void __launch_bounds__(kPackThreads) pack_kernel(const PackParams p) {
+template <int T>
+__global__ void __launch_bounds__(T) pack_kernel(const PackParams p) {
   pdl_wait();
-  if ((int)blockIdx.x >= p.n_gather_blocks) { build_sched(p, (int)blockIdx.x - p.n_gather_blocks); return; }
-  __shared__ int sh_scan[kPackThreads / 32 + 1];
+  if ((int)blockIdx.x >= p.n_gather_blocks) { build_sched<T>(p, (int)blockIdx.x - p.n_gather_blocks); return; }
+  __shared__ int sh_scan[T / 32];
   __shared__ int s_req[kSlotsPerBlock], s_idx[kSlotsPerBlock], s_w[kSlotsPerBlock];
   const int tid = threadIdx.x;
   const int slot0 = blockIdx.x * kSlotsPerBlock;
   if (tid < kSlotsPerBlock) s_req[tid] = -1;
   __syncthreads();
   int run = 0;
-  for (int r0 = 0; r0 < p.max_requests; r0 += kPackThreads) {
+  for (int r0 = 0; r0 < p.max_requests; r0 += T) {
     const int r = r0 + tid;
     const int w = r < p.max_requests ? live_blocks(p, r, p.status) : 0;
-    int tot;
-    const int begin = run + block_excl_scan(w, &tot, sh_scan);
-    run += tot;
+    int pre[1], tot[1];
+    if (r0) __syncthreads();              // the scan's scratch of the previous round has been read
+    block_excl_scan<T, 1>({w}, pre, tot, sh_scan);
+    const int begin = run + pre[0];
+    run += tot[0];
     if (r < p.max_requests) {
       if (blockIdx.x == 0) p.req_slot_begin[r] = begin;
       for (int s = 0; s < w; ++s) {
@@ -321,7 +365,7 @@ __global__ void __launch_bounds__(kPackThreads) pack_kernel(const PackParams p) 
   if (blockIdx.x == 0 && tid == 0) { p.req_slot_begin[p.max_requests] = run; *p.n_live = run; }
   __syncthreads();
   // all slots of this block at once: one thread per (slot, token)
-  for (int i = tid; i < kSlotsPerBlock * p.bl; i += kPackThreads) {
+  for (int i = tid; i < kSlotsPerBlock * p.bl; i += T) {
     const int k = i / p.bl, t = i % p.bl;
     const int slot = slot0 + k;
     if (slot >= p.max_slots) break;
@@ -375,7 +419,10 @@ int launch_pack(fb_ctx* ctx, const fb_state* st, const fb_pack* out, void* ws, i
   p.resident = ctx->cfg.window_in_pages;
   p.n_gather_blocks = (p.max_slots + kSlotsPerBlock - 1) / kSlotsPerBlock;
   // one more block per work list in use (the CTA-pair kernel's list only when that kernel is on)
-  return cuda_err(ctx, launch_pdl(pack_kernel, p.n_gather_blocks + 1 + (p.pair_on ? 1 : 0), kPackThreads, 0, stream, p),
+  const int grid = p.n_gather_blocks + 1 + (p.pair_on ? 1 : 0);
+  return cuda_err(ctx, p.max_requests <= kPackSmallRequests
+                           ? launch_pdl(pack_kernel<kPackThreadsSmall>, grid, kPackThreadsSmall, 0, stream, p)
+                           : launch_pdl(pack_kernel<kPackThreads>, grid, kPackThreads, 0, stream, p),
                   "pack_kernel launch");
 }
 
