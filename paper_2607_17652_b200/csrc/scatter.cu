@@ -5,11 +5,16 @@
 // (all KV heads), optionally with the rotary embedding applied to the keys.
 // HBM-bound: 2 x rows x Hkv x d x 2 bytes read and as many written.
 //
-// One to four CTAs per slot (the slot's tokens are dealt among them).  For a (token, head) the head_dim elements are contiguous
-// in the source (slot-order rows) and in the destination (pool row of that
-// position), so a thread moves 16-byte pieces: with the rotary embedding a
-// thread owns the two pieces that hold elements i and i + d/2 of eight pairs,
-// and the rotation angles come from a per-slot table in shared memory.
+// Several CTAs per slot, the slot's tokens dealt among them so that a thread has one work item
+// (launch_scatter).  For a (token, head) the head_dim elements are contiguous in the source
+// (slot-order rows) and in the destination (pool row of that position), so a thread moves 16-byte
+// pieces: with the rotary embedding it owns the two pieces that hold elements i and i + d/2 of
+// eight pairs, and the rotation angles come from a table in shared memory, built while the
+// loads of the item are in flight.
+// Small batches are bound by the chain of dependent loads, large ones by bandwidth and by the
+// table's arithmetic.  Call in us, former form (256 threads, four CTAs a slot, loads behind the
+// table) -> this one: 1 request 4.8 -> 2.5, 8 requests 4.3 -> 3.9, 128 requests 18.6 -> 14.5
+// (84 MB: 5.8 TB/s), 64 requests into 8-bit pages 14.3 -> 11.9, 16 long contexts 20.8 -> 8.4.
 #include <cuda_fp8.h>
 
 #include <cmath>
@@ -18,7 +23,7 @@
 
 namespace fb {
 
-constexpr int kScatterThreads = 256;
+constexpr int kScatterThreads = 128;
 
 struct ScatterParams {
   const int32_t* n_live; const int32_t* slot_req; const int32_t* slot_pos0;
@@ -58,8 +63,8 @@ template <bool F8>
 __global__ void __launch_bounds__(kScatterThreads) scatter_window_kv_kernel(const ScatterParams p) {
   pdl_wait();
   const int slot = blockIdx.x;
-  if (slot >= *p.n_live) return;
-  const int r = p.slot_req[slot], pos0 = p.slot_pos0[slot];
+  const int n_live = *p.n_live, r = p.slot_req[slot], pos0 = p.slot_pos0[slot];      // (together: one latency)
+  if (slot >= n_live) return;
   const int vph = p.head_dim / 8;                    // 16-byte pieces per (token, head)
   const int vpt = p.n_kv_heads * vph;                // ... per token
   const bool rope = p.rope_base > 0.f;
@@ -71,61 +76,64 @@ __global__ void __launch_bounds__(kScatterThreads) scatter_window_kv_kernel(cons
   const int half = p.head_dim / 2;
   // work item = (token, head, piece); with the rotary embedding only the lower half of the
   // pieces is enumerated and each item also handles its partner piece + d/16
-  const int per_head = rope ? vph / 2 : vph;
+  const int per_head = rope ? vph / 2 : vph, partner = rope ? vph / 2 : 0;
   // the slot's tokens are dealt to the gridDim.y CTAs of the slot (each builds the table of its
   // own tokens only)
   const int tpc = (p.bl + (int)gridDim.y - 1) / (int)gridDim.y;
   const int tbeg = (int)blockIdx.y * tpc, tend = min(p.bl, tbeg + tpc);
-  for (int t0 = tbeg; t0 < tend; t0 += kTokBatch) {
-  const int nt = min(kTokBatch, tend - t0);
-  if (rope) {
-    __syncthreads();                                 // the previous batch has been read
-    for (int i = threadIdx.x; i < nt * half; i += kScatterThreads) {
-      const int t = i / half, k = i % half;
-      // angle in fp64, reduced to [-pi, pi] there; sine and cosine of the remainder in fp32
-      const double ang = (double)(pos0 + t0 + t) * p.inv_freq[k];
-      const double red = fma(-rint(ang * 0.15915494309189535), 6.283185307179586, ang);
-      float sf, cf;
-      sincosf((float)red, &sf, &cf);
-      cs[i] = make_float2(cf, sf);
-    }
-    __syncthreads();
-  }
   const int nh = p.n_kv_heads;
-  const int total = nt * nh * per_head;
-  for (int i = threadIdx.x; i < total; i += kScatterThreads) {
-    const int tb = i / (nh * per_head), rem = i % (nh * per_head);
-    const int t = t0 + tb;
-    const int h = rem / per_head, v = rem % per_head;
-    const int pos = pos0 + t, pidx = pos / kPage;
-    if (pidx >= p.max_pages_per_req) { atomicOr(p.status, FB_ST_BAD_PAGE); continue; }
-    const int page = p.page_table[(size_t)r * p.max_pages_per_req + pidx];
-    if (page < 0 || page >= p.num_pages) { atomicOr(p.status, FB_ST_BAD_PAGE); continue; }
-    const size_t src = (size_t)(slot * p.bl + t) * vpt + h * vph + v;
-    const size_t dst = (((size_t)page * p.n_kv_heads + h) * kPage + pos % kPage) * vph + v;
-    [[maybe_unused]] uint2* k8 = reinterpret_cast<uint2*>(p.k_pool);
-    [[maybe_unused]] uint2* v8 = reinterpret_cast<uint2*>(p.v_pool);
-    [[maybe_unused]] float ksc = 1.f, vsc = 1.f;
-    if constexpr (F8) { ksc = p.k_scale[h]; vsc = p.v_scale[h]; }
-    if (!rope) {
-      if constexpr (F8) {
-        k8[dst] = quant8(p.k_new[src], ksc);
-        v8[dst] = quant8(p.v_new[src], vsc);
-      } else {
-        p.k_pool[dst] = p.k_new[src];
-        p.v_pool[dst] = p.v_new[src];
+  for (int t0 = tbeg; t0 < tend; t0 += kTokBatch) {
+    const int nt = min(kTokBatch, tend - t0), total = nt * nh * per_head;
+    for (int i = threadIdx.x; i < (total + kScatterThreads - 1) / kScatterThreads * kScatterThreads; i += kScatterThreads) {
+      // the loads first: source rows and page id do not depend on the table
+      const int tb = i / (nh * per_head), rem = i % (nh * per_head), h = rem / per_head, v = rem % per_head;
+      const int pos = pos0 + t0 + tb;
+      uint4 ka, kb, va, vb;
+      int page = -1;
+      if (i < total) {
+        const size_t src = (size_t)(slot * p.bl + t0 + tb) * vpt + h * vph + v;
+        if (pos / kPage < p.max_pages_per_req) page = p.page_table[(size_t)r * p.max_pages_per_req + pos / kPage];
+        ka = p.k_new[src]; va = p.v_new[src];
+        if (rope) { kb = p.k_new[src + partner]; vb = p.v_new[src + partner]; }
       }
-      continue;
-    }
-    const uint4 a = p.k_new[src], b = p.k_new[src + vph / 2];      // elements i0.. and i0 + d/2..
-    float c[8], s[8];
+      if (rope && i < kScatterThreads) {             // (uniform: the first pass of the batch)
+        if (t0 != tbeg) __syncthreads();             // the previous batch has been read
+        for (int e = threadIdx.x; e < nt * half; e += kScatterThreads) {
+          const int t = e / half, k = e % half;
+          // angle in fp64, reduced to [-pi, pi] there; sine and cosine of the remainder in fp32
+          const double ang = (double)(pos0 + t0 + t) * p.inv_freq[k];
+          const double red = fma(-rint(ang * 0.15915494309189535), 6.283185307179586, ang);
+          float sf, cf;
+          sincosf((float)red, &sf, &cf);
+          cs[e] = make_float2(cf, sf);
+        }
+        __syncthreads();
+      }
+      if (i >= total) continue;
+      if (page < 0 || page >= p.num_pages) { atomicOr(p.status, FB_ST_BAD_PAGE); continue; }
+      const size_t dst = (((size_t)page * p.n_kv_heads + h) * kPage + pos % kPage) * vph + v;
+      [[maybe_unused]] uint2* k8 = reinterpret_cast<uint2*>(p.k_pool);
+      [[maybe_unused]] uint2* v8 = reinterpret_cast<uint2*>(p.v_pool);
+      [[maybe_unused]] float ksc = 1.f, vsc = 1.f;
+      if constexpr (F8) {
+        ksc = p.k_scale[h]; vsc = p.v_scale[h];
+        v8[dst] = quant8(va, vsc);
+        if (rope) v8[dst + partner] = quant8(vb, vsc);
+        else k8[dst] = quant8(ka, ksc);
+      } else {
+        p.v_pool[dst] = va;
+        if (rope) p.v_pool[dst + partner] = vb;
+        else p.k_pool[dst] = ka;
+      }
+      if (!rope) continue;
+      float c[8], s[8];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const float2 a2 = cs[tb * half + v * 8 + k];
-      c[k] = a2.x; s[k] = a2.y;
-    }
-    const uint32_t aw[4] = {a.x, a.y, a.z, a.w}, bw[4] = {b.x, b.y, b.z, b.w};
-    if constexpr (F8) {
+      for (int k = 0; k < 8; ++k) {
+        const float2 a2 = cs[tb * half + v * 8 + k];
+        c[k] = a2.x; s[k] = a2.y;
+      }
+      // elements i0.. (ka) and i0 + d/2.. (kb) of the head
+      const uint32_t aw[4] = {ka.x, ka.y, ka.z, ka.w}, bw[4] = {kb.x, kb.y, kb.z, kb.w};
       float lo[8], hi[8];
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
@@ -133,24 +141,14 @@ __global__ void __launch_bounds__(kScatterThreads) scatter_window_kv_kernel(cons
         lo[2 * k] = x0 * c[2 * k] - y0 * s[2 * k]; lo[2 * k + 1] = x1 * c[2 * k + 1] - y1 * s[2 * k + 1];
         hi[2 * k] = y0 * c[2 * k] + x0 * s[2 * k]; hi[2 * k + 1] = y1 * c[2 * k + 1] + x1 * s[2 * k + 1];
       }
-      k8[dst] = make_uint2(e4m3x4(lo[0], lo[1], lo[2], lo[3], ksc), e4m3x4(lo[4], lo[5], lo[6], lo[7], ksc));
-      k8[dst + vph / 2] = make_uint2(e4m3x4(hi[0], hi[1], hi[2], hi[3], ksc), e4m3x4(hi[4], hi[5], hi[6], hi[7], ksc));
-      v8[dst] = quant8(p.v_new[src], vsc);
-      v8[dst + vph / 2] = quant8(p.v_new[src + vph / 2], vsc);
-    } else {
-      uint32_t lo[4], hi[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const float x0 = bf16_lo(aw[k]), x1 = bf16_hi(aw[k]), y0 = bf16_lo(bw[k]), y1 = bf16_hi(bw[k]);
-        lo[k] = to_bf16x2(x0 * c[2 * k] - y0 * s[2 * k], x1 * c[2 * k + 1] - y1 * s[2 * k + 1]);
-        hi[k] = to_bf16x2(y0 * c[2 * k] + x0 * s[2 * k], y1 * c[2 * k + 1] + x1 * s[2 * k + 1]);
+      if constexpr (F8) {
+        k8[dst] = make_uint2(e4m3x4(lo[0], lo[1], lo[2], lo[3], ksc), e4m3x4(lo[4], lo[5], lo[6], lo[7], ksc));
+        k8[dst + partner] = make_uint2(e4m3x4(hi[0], hi[1], hi[2], hi[3], ksc), e4m3x4(hi[4], hi[5], hi[6], hi[7], ksc));
+      } else {
+        p.k_pool[dst] = make_uint4(to_bf16x2(lo[0], lo[1]), to_bf16x2(lo[2], lo[3]), to_bf16x2(lo[4], lo[5]), to_bf16x2(lo[6], lo[7]));
+        p.k_pool[dst + partner] = make_uint4(to_bf16x2(hi[0], hi[1]), to_bf16x2(hi[2], hi[3]), to_bf16x2(hi[4], hi[5]), to_bf16x2(hi[6], hi[7]));
       }
-      p.k_pool[dst] = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-      p.k_pool[dst + vph / 2] = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-      p.v_pool[dst] = p.v_new[src];
-      p.v_pool[dst + vph / 2] = p.v_new[src + vph / 2];
     }
-  }
   }
 }
 
@@ -159,9 +157,11 @@ static void fill_inv_freq(ScatterParams& p, int head_dim, float rope_base) {
     p.inv_freq[k] = (rope_base > 0.f && k < head_dim / 2)
                         ? exp2(-2.0 * (double)k / (double)head_dim * log2((double)rope_base)) : 0.0;
 }
-// enough (token, head, piece) items per CTA to keep 256 threads busy: four CTAs per slot once a
-// slot holds 32 tokens of at least four KV heads
-static int scatter_ctas_per_slot(const fb_config& c) { return c.block_len >= 32 && c.n_kv_heads >= 4 ? 4 : 1; }
+// one (token, head, pair of pieces) item per thread (two with the embedding off)
+static int scatter_ctas_per_slot(const fb_config& c) {
+  const int n = c.block_len * c.n_kv_heads * (c.head_dim / 16) / kScatterThreads;
+  return n < 1 ? 1 : n < c.block_len ? n : c.block_len;
+}
 
 int launch_scatter(fb_ctx* ctx, const fb_pack* pk, const int32_t* page_table, const void* k_new,
                    const void* v_new, void* k_pool, void* v_pool, float rope_base, int32_t* status,
