@@ -33,6 +33,7 @@ struct AttnParams {
   float* part_o;
   int32_t* status;
   int32_t bl, n_q_heads, n_kv_heads, group, max_pages_per_req, num_pages;
+  int32_t max_items, max_units;
   int32_t resident;     // 1: the window is read from the pages (every key tile is a paged one)
   const float* k_scale; // 8-bit pages only: value = code * scale of the KV head, [n_kv_heads]
   const float* v_scale;
@@ -65,16 +66,25 @@ __device__ __forceinline__ bool load_item(const AttnParams& p, int idx, ItemGeom
 
 // Work item records in shared memory: 4 words of the item, 16 of the unit, 1 = there is one.
 constexpr int kItemWords = 24;
-// One warp copies item idx and its unit there (or the end mark).
-__device__ __forceinline__ void publish_item(const AttnParams& p, int idx, bool more, int* dst, int lane) {
-  int v = 0;
-  if (more) {
-    const int* it = reinterpret_cast<const int*>(&p.items[idx]);
-    const int* un = reinterpret_cast<const int*>(&p.units[it[0]]);
-    v = lane < 4 ? it[lane] : lane < 20 ? un[lane - 4] : 1;
-  }
-  if (lane < 21) dst[lane] = v;
+// One warp copies item idx (and its unit) there, or the end mark if there are no more than n_items.
+// The first item is fetched before n_items is known, so that the two loads run together: every
+// index is clamped to the list, a record beyond the last item is never used.  `pages`: called with
+// the item's request and first key tile while the unit record is on its way.
+template <typename F>
+__device__ __forceinline__ bool publish_item(const AttnParams& p, int idx, const int* n_items, int* dst, int lane, F&& pages) {
+  const int* it = reinterpret_cast<const int*>(&p.items[min(idx, p.max_items - 1)]);
+  int v = lane < 5 ? it[lane] : 0;
+  const int n = *n_items;
+  const int unit = min(max(__shfl_sync(0xffffffffu, v, 0), 0), p.max_units - 1);
+  const int u = lane >= 4 && lane < 20 ? reinterpret_cast<const int*>(&p.units[unit])[lane - 4] : 1;
+  const bool more = idx < n;
+  const int jb = __shfl_sync(0xffffffffu, v, 2), req = __shfl_sync(0xffffffffu, v, 4);
+  if (more) pages(req, jb);
+  if (lane >= 4) v = u;
+  if (lane < 20) dst[lane] = v;
+  if (lane == 20) dst[lane] = more;
   __syncwarp();
+  return more;
 }
 // Returns false at the end mark.  g.n <= 0: an item without visible keys.
 __device__ __forceinline__ bool load_item(const int* src, ItemGeom& g) {

@@ -210,7 +210,6 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   pdl_wait();                     // the work list (and everything else) of the previous kernels is complete
-  const int n_items = p.hdr->n_items;
 
   // The control warpgroup (warps 0-3) hands registers to the softmax
   // warpgroups.  All four warps of a warpgroup execute the same setmaxnreg
@@ -306,8 +305,11 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
         }
         // the record goes to shared memory: the other roles would each pay two dependent
         // global loads (~1300 cycles per item) for it
-        more = idx < n_items;
-        publish_item(p, idx, more, s_item + (k & 1) * kItemWords, lane);
+        more = publish_item(p, idx, &p.hdr->n_items, s_item + (k & 1) * kItemWords, lane, [&](int req, int jb) {
+          pc_blk = (jb * 2) >> 5;
+          pc_cur = load_pages(req, pc_blk);
+          pc_next = load_pages(req, pc_blk + 1);
+        });
         if (lane == 0) mbar_arrive(&item_full[k & 1]);
         load_item_uniform(s_item + (k & 1) * kItemWords, p, g);
         __syncwarp();
@@ -318,11 +320,11 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
         __syncwarp();
         if (lane == 0) mbar_arrive(&item_empty[k & 1]);
         if (!more) break;
+        pc_blk = (g.jb * 2) >> 5;
+        pc_cur = load_pages(g.req, pc_blk);
+        pc_next = load_pages(g.req, pc_blk + 1);
       }
       if (g.n <= 0) continue;
-      pc_blk = (g.jb * 2) >> 5;
-      pc_cur = load_pages(g.req, pc_blk);
-      pc_next = load_pages(g.req, pc_blk + 1);
       if (warp == 0) {
         if (q_uses > 0 && !warp_wait(q_empty, (q_uses - 1) & 1, abortf, LIM)) { ok = false; break; }
         ++q_uses;
@@ -353,6 +355,9 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
         }
       }
     }
+    // The last CTA to draw its last ticket re-arms the counter, so that the same work list can be
+    // run again (also after a launch that gave up half way through its items).
+    if (warp == 0 && lane == 0 && atomicAdd(&p.hdr->done, 1) == (int)gridDim.x - 1) { p.hdr->ticket = 0; p.hdr->done = 0; }
   } else if (warp == 1) {
     // ---------------------------------------------------------- MMA issuer
     // The tensor pipe takes 64 cycles per MMA and queues about 250 cycles of work behind the
@@ -700,9 +705,6 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
   // ---------------------------------------------------------------- teardown
   tc_fence_before();
   __syncthreads();
-  // Last one out re-arms the work ticket, so that the same work list can be run again (also after
-  // a launch that gave up half way through its items).  This thread drew this CTA's tickets.
-  if (tid == 0 && atomicAdd(&p.hdr->done, 1) == (int)gridDim.x - 1) { p.hdr->ticket = 0; p.hdr->done = 0; }
   if (*abortf) {
     // A bounded wait gave up.  Nothing may still be running on this CTA's shared memory or
     // TMEM when they are handed on: (1) the MMA warp commits everything it has issued to a
@@ -749,16 +751,26 @@ __global__ void __launch_bounds__(kCombineThreads, 3) attn_combine_kernel(const 
   const int first_row = ((sub / (D / 8)) * 8 + warp) * rpw;             // of the unit's 256
   const int X = first_row >= kTileM, row = first_row % kTileM + lane % rpw;
   for (int u0 = blockIdx.x / per_unit; u0 < n_units; u0 += 32 * G) {
+    // lane i holds what matters of the i-th of the CTA's next 32 units
     const int mine = u0 + lane * G;
-    unsigned todo = __ballot_sync(0xffffffffu, mine < n_units && p.units[mine].n_chunks > 1);
+    int u_slot = -1, u_kvh = 0, u_t0 = 0, u_nt = 1, u_nch = 0, u_nvis = 0, u_part = 0;
+    if (mine < n_units) {
+      const int4* up = reinterpret_cast<const int4*>(&p.units[mine]);
+      const int4 a = up[0], b = up[1], c = up[2];
+      u_slot = X == 0 ? a.z : a.w; u_kvh = X == 0 ? a.y & 0xffff : a.y >> 16;
+      u_t0 = X == 0 ? b.x : b.y; u_nt = b.z; u_nch = b.w;
+      u_nvis = X == 0 ? c.x : c.y; u_part = c.z;
+    }
+    unsigned todo = __ballot_sync(0xffffffffu, u_nch > 1 && u_slot >= 0);
     for (; todo; todo &= todo - 1) {
-      const AttnUnit un = p.units[u0 + (__ffs(todo) - 1) * G];
-      const int slot = X == 0 ? un.slotA : un.slotB;
-      if (slot < 0) continue;                                           // (uniform: X is the warp's)
-      const int nvis = X == 0 ? un.nvisA : un.nvisB, t0 = X == 0 ? un.t0A : un.t0B;
+      const int src = __ffs(todo) - 1;
+      const int slot = __shfl_sync(0xffffffffu, u_slot, src), kvh = __shfl_sync(0xffffffffu, u_kvh, src);
+      const int t0 = __shfl_sync(0xffffffffu, u_t0, src), nt = __shfl_sync(0xffffffffu, u_nt, src);
+      const int nch = __shfl_sync(0xffffffffu, u_nch, src), nvis = __shfl_sync(0xffffffffu, u_nvis, src);
+      const int part_base = __shfl_sync(0xffffffffu, u_part, src);
       // chunks that hold keys visible to this tile: those that start before tile nvis
-      const int nc = min(un.n_chunks, (int)(((long long)nvis * un.n_chunks + un.n_tiles - 1) / un.n_tiles));
-      const size_t tile0 = (size_t)un.part_base * 2 + X;              // chunk c: + 2 c
+      const int nc = min(nch, (int)(((long long)nvis * nch + nt - 1) / nt));
+      const size_t tile0 = (size_t)part_base * 2 + X;                 // chunk c: + 2 c
       const float2* ml = reinterpret_cast<const float2*>(p.part_ml) + tile0 * kTileM + row;
       float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
       float M = -INFINITY, L = 0.f;
@@ -803,7 +815,7 @@ __global__ void __launch_bounds__(kCombineThreads, 3) attn_combine_kernel(const 
       if (way == 0) {
         const float inv = 1.0f / L;
         const int grow_ = slot * p.bl + t0 + row / p.group;
-        const int head = (X == 0 ? (un.kvh & 0xffff) : (un.kvh >> 16)) * p.group + row % p.group;
+        const int head = kvh * p.group + row % p.group;
         *reinterpret_cast<uint4*>(p.out + ((size_t)grow_ * p.n_q_heads + head) * D + cols * 8) =
             make_uint4(pack_bf16x2(acc[0] * inv, acc[1] * inv), pack_bf16x2(acc[2] * inv, acc[3] * inv),
                        pack_bf16x2(acc[4] * inv, acc[5] * inv), pack_bf16x2(acc[6] * inv, acc[7] * inv));
@@ -876,6 +888,7 @@ void fill_attn_params(fb_ctx* ctx, AttnParams& p, const int32_t* page_table, voi
   p.out = static_cast<__nv_bfloat16*>(out);
   p.part_ml = reinterpret_cast<float*>(w + ctx->ws.l[list].part_ml);
   p.part_o = reinterpret_cast<float*>(w + ctx->ws.l[list].part_o);
+  p.max_items = ctx->ws.l[list].max_items; p.max_units = ctx->ws.l[list].max_units;
   p.status = status;
   p.bl = c.block_len; p.n_q_heads = c.n_q_heads; p.n_kv_heads = c.n_kv_heads; p.group = ctx->group;
   p.max_pages_per_req = c.max_pages_per_req; p.num_pages = c.num_pages;

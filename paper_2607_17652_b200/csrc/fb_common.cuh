@@ -33,6 +33,7 @@ struct __align__(16) AttnUnit {
 };
 struct __align__(16) AttnItem {
   int32_t unit, chunk, jb, je;         // key tiles [jb, je) of the unit
+  int32_t req, pad[3];                 // (the unit's request: its page ids are fetched beside the unit record)
 };
 
 struct SchedHeader {

@@ -141,6 +141,7 @@ __device__ void build_sched(const PackParams& p, const int list) {
   __shared__ SplitRule sh_rule;
   __shared__ int s_ub[T + 1], s_pb[T], s_first[T], s_wb[T], s_w[T], s_P[T];
   __shared__ int4 s_info[kUnitInfo];
+  __shared__ int s_req[kUnitInfo];
   const int tid = threadIdx.x;
   if (tid == 0) { sh_total = 0; sh_units = 0; sh_chunks = 0; sh_longest = 0; }
   if (tid < kSplitCandidates) sh_stat[tid] = SplitStat{};
@@ -270,7 +271,7 @@ __device__ void build_sched(const PackParams& p, const int list) {
         if (c0 == 0) units[mult * u + rr] = un[rr];
         nvA = max(nvA, un[rr].nvisA); nvB = max(nvB, un[rr].nvisB);
       }
-      if (c0 == 0 && u < kUnitInfo) s_info[u] = make_int4(nvA, nvB, q.nt, nch);
+      if (c0 == 0 && u < kUnitInfo) { s_info[u] = make_int4(nvA, nvB, q.nt, nch); s_req[u] = r0 + k; }
       for (int c = c0; c < nch; c += lanes) {
         const int jb = c * q.nt / nc, je = (c + 1) * q.nt / nc;
         int cost = item_cost(max(0, min(je, nvA) - jb), max(0, min(je, nvB) - jb));
@@ -312,13 +313,14 @@ __device__ void build_sched(const PackParams& p, const int list) {
   while (lanes < 32 && lanes < sh_chunks && 2 * lanes * n_sched <= T) lanes *= 2;
   for (int j = tid; j < n_sched * lanes; j += T) {
     const int u = j / lanes;
-    int nvA, nvB, nt, nch;
+    int nvA, nvB, nt, nch, req;
     if (u < kUnitInfo) {
+      req = s_req[u];
       const int4 f = s_info[u];
       nvA = f.x; nvB = f.y; nt = f.z; nch = f.w;
     } else {
       const AttnUnit un = units[mult * u];
-      nvA = un.nvisA; nvB = un.nvisB; nt = un.n_tiles; nch = un.n_chunks;
+      nvA = un.nvisA; nvB = un.nvisB; nt = un.n_tiles; nch = un.n_chunks; req = un.req;
       if (mult == 2) { const AttnUnit u1 = units[2 * u + 1]; nvA = max(nvA, u1.nvisA); nvB = max(nvB, u1.nvisB); }
     }
     for (int c = j % lanes; c < nch; c += lanes) {
@@ -327,6 +329,7 @@ __device__ void build_sched(const PackParams& p, const int list) {
       const int at = atomicAdd(&bins[min(cost, kCostBins - 1)], 1);
       if (at < max_items) {
         AttnItem it; it.unit = mult * u; it.chunk = c; it.jb = jb; it.je = je;
+        it.req = req; it.pad[0] = it.pad[1] = it.pad[2] = 0;
         items[at] = it;
       }
     }
