@@ -42,6 +42,37 @@ __device__ __forceinline__ bool lm_warp_wait(uint64_t* bar, uint32_t parity, vol
   return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort, limit));
 }
 
+// 32 more columns of a row: running maximum with its first index, sum of exponentials relative to it
+// (an equal later maximum keeps the first index; all -inf adds nothing).
+__device__ __forceinline__ void absorb32(const uint32_t* v, int col, float& mx, float& sum, int& arg) {
+  float m4[4];
+#pragma unroll
+  for (int t = 0; t < 4; ++t) m4[t] = fmaxf(__uint_as_float(v[t]), __uint_as_float(v[4 + t]));
+#pragma unroll
+  for (int i = 8; i < 32; i += 8)
+#pragma unroll
+    for (int t = 0; t < 4; ++t) m4[t] = max3(m4[t], __uint_as_float(v[i + t]), __uint_as_float(v[i + 4 + t]));
+  const float cm = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
+  if (cm > mx) {
+    int first = 31;
+#pragma unroll
+    for (int j = 30; j >= 0; --j) first = __uint_as_float(v[j]) == cm ? j : first;
+    sum *= ex2_approx((mx - cm) * kLmLog2e);                          // 0 * 2^-inf = 0 at the first maximum
+    mx = cm; arg = col + first;
+  }
+  if (mx == -INFINITY) return;
+  const float mb = -mx * kLmLog2e;
+  const float2 mb2 = make_float2(mb, mb), l2 = make_float2(kLmLog2e, kLmLog2e);
+  float2 s4[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+#pragma unroll
+  for (int j = 0; j < 32; j += 2) {
+    const float2 x = __ffma2_rn(make_float2(__uint_as_float(v[j]), __uint_as_float(v[j + 1])), l2, mb2);
+    s4[(j >> 1) & 3] = __fadd2_rn(s4[(j >> 1) & 3], make_float2(ex2_approx(x.x), ex2_approx(x.y)));
+  }
+  const float2 t = __fadd2_rn(__fadd2_rn(s4[0], s4[1]), __fadd2_rn(s4[2], s4[3]));
+  sum += t.x + t.y;
+}
+
 __global__ void __launch_bounds__(kLmThreads, 1)
 lm_head_stats_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW,
                      const LmParams p) {
@@ -143,23 +174,15 @@ lm_head_stats_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
         const uint32_t* v = buf[c & 1];
         tmem_ld_wait();
         if (c + 1 < kLmBN / 32) tmem_ld32(tacc + (c + 1) * 32, buf[(c + 1) & 1]);
-        const int valid = min(32, p.vocab - (col0 + c * 32));        // columns of this chunk inside the vocabulary
-        float cm = -INFINITY;
+        const int valid = p.vocab - (col0 + c * 32);                 // columns of this chunk inside the vocabulary
+        if (valid >= 32) {
+          absorb32(v, col0 + c * 32, mx, sum, arg);
+        } else if (valid > 0) {                                      // (the last tile: columns past the vocabulary count as -inf)
+          uint32_t z[32];
 #pragma unroll
-        for (int j = 0; j < 32; ++j) cm = fmaxf(cm, j < valid ? __uint_as_float(v[j]) : -INFINITY);
-        if (cm > mx) {                                              // strict: an equal later maximum keeps the first index
-          int first = 31;
-#pragma unroll
-          for (int j = 31; j >= 0; --j) if (j < valid && __uint_as_float(v[j]) == cm) first = j;
-          sum *= ex2_approx((mx - cm) * kLmLog2e);                    // 0 * 2^-inf = 0 on the first chunk
-          mx = cm; arg = col0 + c * 32 + first;
+          for (int j = 0; j < 32; ++j) z[j] = j < valid ? v[j] : __float_as_uint(-INFINITY);
+          absorb32(z, col0 + c * 32, mx, sum, arg);
         }
-        const float mb = mx * kLmLog2e;
-        float s4[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-        for (int j = 0; j < 32; ++j)
-          s4[j & 3] += j < valid ? ex2_approx(fmaf(__uint_as_float(v[j]), kLmLog2e, -mb)) : 0.f;
-        sum += (s4[0] + s4[1]) + (s4[2] + s4[3]);
       }
       tc_fence_before();
       __syncwarp();
@@ -187,39 +210,55 @@ lm_head_stats_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
 }
 
 // Tiles of a row -> top-1 token (lowest index on ties) and its confidence 1 / sum exp(z - max).
-__global__ void __launch_bounds__(256) lm_head_merge_kernel(const LmParams p, int32_t* argmax, float* conf,
-                                                            int max_rows) {
-  const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (row >= max_rows) return;
-  if (row >= *p.n_live * p.bl) {
-    if (lane == 0) { argmax[row] = -1; conf[row] = 0.f; }
+// A CTA takes 32 rows, one per lane, so that a tile's results are read as whole lines; its 32 warps
+// take the tiles in turn and meet in shared memory (5120 rows of 592 tiles: 41 us with a warp per row
+// that read 16 bytes of a line, now about 10).
+constexpr int kLmMergeWarps = 32;
+__global__ void __launch_bounds__(32 * kLmMergeWarps) lm_head_merge_kernel(const LmParams p, int32_t* argmax, float* conf,
+                                                                          int max_rows) {
+  pdl_wait();
+  __shared__ float s_m[kLmMergeWarps][32], s_s[kLmMergeWarps][32];
+  __shared__ int s_a[kLmMergeWarps][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, row = blockIdx.x * 32 + lane;
+  const int live = *p.n_live * p.bl;
+  if (blockIdx.x * 32 >= live) {                    // (the whole CTA)
+    if (warp == 0 && row < max_rows) { argmax[row] = -1; conf[row] = 0.f; }
     return;
   }
-  float M = -INFINITY;
-  for (int n = lane; n < p.n_tiles_n; n += 32) M = fmaxf(M, p.part[(size_t)n * p.rows_pad + row].x);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
-  float S = 0.f;
+  float M = -INFINITY, S = 0.f;
   int arg = 0x7fffffff;
-  for (int n = lane; n < p.n_tiles_n; n += 32) {
-    const float4 q = p.part[(size_t)n * p.rows_pad + row];
-    S += q.y * ex2_approx((q.x - M) * kLmLog2e);
-    if (q.x == M) arg = min(arg, __float_as_int(q.z));
-  }
+  auto add = [&](float m, float s, int a) {         // tiles come in ascending order: an equal maximum keeps the first index
+    if (m > M) { S = S * (M == -INFINITY ? 0.f : ex2_approx((M - m) * kLmLog2e)) + s; M = m; arg = a; }
+    else S += m == -INFINITY ? 0.f : s * ex2_approx((m - M) * kLmLog2e);
+  };
+  if (row < live) {
+    constexpr int kDepth = 4;
+    for (int n0 = warp; n0 < p.n_tiles_n; n0 += kDepth * kLmMergeWarps) {
+      float4 q[kDepth];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    S += __shfl_xor_sync(0xffffffffu, S, o);
-    arg = min(arg, __shfl_xor_sync(0xffffffffu, arg, o));
-  }
-  if (lane == 0) {
-    if (!(S >= 1.0f) || S > FLT_MAX || arg == 0x7fffffff) {
-      atomicOr(p.status, FB_ST_NAN_LOGIT);
-      argmax[row] = arg == 0x7fffffff ? 0 : arg;
-      conf[row] = 0.f;
-    } else {
-      argmax[row] = arg;
-      conf[row] = 1.0f / S;
+      for (int k = 0; k < kDepth; ++k) q[k] = p.part[(size_t)min(n0 + k * kLmMergeWarps, p.n_tiles_n - 1) * p.rows_pad + row];
+#pragma unroll
+      for (int k = 0; k < kDepth; ++k)
+        if (n0 + k * kLmMergeWarps < p.n_tiles_n) add(q[k].x, q[k].y, __float_as_int(q[k].z));
     }
+  }
+  s_m[warp][lane] = M; s_s[warp][lane] = S; s_a[warp][lane] = arg;
+  __syncthreads();
+  if (warp != 0 || row >= max_rows) return;
+  if (row >= live) { argmax[row] = -1; conf[row] = 0.f; return; }
+  for (int k = 1; k < kLmMergeWarps; ++k) {
+    const float m = s_m[k][lane], s = s_s[k][lane];
+    const int a = s_a[k][lane];
+    if (m == M && m != -INFINITY) { S += s; arg = min(arg, a); }
+    else add(m, s, a);
+  }
+  if (!(S >= 1.0f) || S > FLT_MAX || arg == 0x7fffffff) {
+    atomicOr(p.status, FB_ST_NAN_LOGIT);
+    argmax[row] = arg == 0x7fffffff ? 0 : arg;
+    conf[row] = 0.f;
+  } else {
+    argmax[row] = arg;
+    conf[row] = 1.0f / S;
   }
 }
 
@@ -277,8 +316,9 @@ int launch_lm_head(fb_ctx* ctx, const fb_pack* pk, const void* x, const void* w,
   p.wait_cycles = ctx->wait_cycles;
   lm_head_stats_kernel<<<ctx->num_sms, kLmThreads, kLmSmem, stream>>>(tmX, tmW, p);
   if (int e = cuda_err(ctx, cudaGetLastError(), "lm_head_stats_kernel launch")) return e;
-  lm_head_merge_kernel<<<(rows + 7) / 8, 256, 0, stream>>>(p, argmax, conf, rows);
-  if (int e = cuda_err(ctx, cudaGetLastError(), "lm_head_merge_kernel launch")) return e;
+  if (int e = cuda_err(ctx, launch_pdl(lm_head_merge_kernel, (rows + 31) / 32, 32 * kLmMergeWarps, 0, stream, p, argmax, conf, rows),
+                       "lm_head_merge_kernel launch"))
+    return e;
   return launch_t2t_update(ctx, pk, st, argmax, conf, action, slot_stats, stream);
 }
 
