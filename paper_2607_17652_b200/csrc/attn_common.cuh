@@ -8,8 +8,8 @@ namespace fb {
 
 constexpr int kAttnThreads = 384;   // 3 warpgroups: control, softmax A, softmax B
 constexpr float kLog2eF = 1.4426950408889634f;
-constexpr float kRescaleThreshold = 8.0f;   // log2 units (8-bit P: bound on every element)
-// bf16 P: the reference is re-based when the exponentials of one key tile sum to more than 2^8
+constexpr float kRescaleThreshold = 8.0f;   // log2 units (tiles that take a max pass)
+// The reference is re-based when the exponentials of one key tile (8-bit P: of an eighth of it) sum to more than 2^8
 // (a bound on every element that costs no per-element work; inf and NaN fail the test too).
 // Kept this low on purpose: after a re-base the largest weight is exactly 1, so a row that one key
 // dominates carries no rounding error of P on that key.
@@ -86,6 +86,9 @@ __device__ __forceinline__ bool publish_item(const AttnParams& p, int idx, const
   __syncwarp();
   return more;
 }
+// Words of a record; those that differ between tiles A and B are A's, tile X's is at + X.
+enum { kRecChunk = 1, kRecJb = 2, kRecJe = 3, kRecKvh = 5, kRecSlot = 6, kRecT0 = 8, kRecChunks = 11, kRecNvis = 12,
+       kRecPartBase = 14, kRecPrefix = 15, kRecNpt = 16, kRecWin = 18, kRecMore = 20 };
 // Returns false at the end mark.  g.n <= 0: an item without visible keys.
 __device__ __forceinline__ bool load_item(const int* src, ItemGeom& g) {
   const int4* v = reinterpret_cast<const int4*>(src);

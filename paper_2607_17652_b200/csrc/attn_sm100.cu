@@ -55,23 +55,23 @@ __device__ __forceinline__ float max_cols(const uint32_t* s) {
 }
 
 // P of N scores against the reference behind mb = m_ref * sl2 - shift: packed into pk, the sum of
-// the unrounded values returned, for 8-bit P the largest exponent in xmax.  A masked score (-inf)
-// comes out as exactly 0.  All exponentials run on the MUFU pipe: moving a quarter of them to a
-// polynomial on the FMA pipe shortens the loop in cycles, but at full load this kernel runs at the
-// board's power limit, where the ~13 extra instructions per pair cost more clock than that
-// gains (long-context workload, sustained: 1205 us without against 1262 us with the polynomial;
-// 64 requests 442 against 464; 8-bit pages 970 against 974).
+// the unrounded values returned; `most`: the largest of eight partial sums of N / 8 values each, a
+// bound on every value that costs three instructions a row (8-bit P saturates, so it needs one:
+// the largest value itself took one instruction per pair and 10 % of that kernel's time).  A masked
+// score (-inf) comes out as exactly 0.  All exponentials run on the MUFU pipe: moving a quarter of
+// them to a polynomial on the FMA pipe shortens the loop in cycles, but at full load this kernel
+// runs at the board's power limit, where the ~13 extra instructions per pair cost more clock than
+// that gains (long-context workload, sustained: 1205 us without against 1262 us with the
+// polynomial; 64 requests 442 against 464; 8-bit pages 970 against 974).
 template <bool F8, int N>
-__device__ __forceinline__ float exp_cols(const uint32_t* s, uint32_t* pk, float sl2, float mb, float& xmax) {
+__device__ __forceinline__ float exp_cols(const uint32_t* s, uint32_t* pk, float sl2, float mb, float& most) {
   const float2 sl2v = make_float2(sl2, sl2), nmb = make_float2(-mb, -mb);
   float2 acc[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-  float xm4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
   float2 prev = make_float2(0.f, 0.f);
 #pragma unroll
   for (int i = 0; i < N; i += 2) {
     const int pr = i >> 1;
     const float2 x = __ffma2_rn(make_float2(__uint_as_float(s[i]), __uint_as_float(s[i + 1])), sl2v, nmb);
-    if constexpr (F8) xm4[pr & 3] = max3(xm4[pr & 3], x.x, x.y);    // 8-bit P saturates: tracked element by element
     const float2 pv = make_float2(ex2_approx(x.x), ex2_approx(x.y));
     acc[pr & 3] = __fadd2_rn(acc[pr & 3], pv);
     if constexpr (F8) {
@@ -81,7 +81,8 @@ __device__ __forceinline__ float exp_cols(const uint32_t* s, uint32_t* pk, float
       pk[pr] = pack_bf16x2(pv.x, pv.y);
     }
   }
-  if constexpr (F8) xmax = fmaxf(fmaxf(xm4[0], xm4[1]), fmaxf(xm4[2], xm4[3]));
+  if constexpr (F8)
+    most = fmaxf(max3(acc[0].x, acc[0].y, acc[1].x), max3(max3(acc[1].y, acc[2].x, acc[2].y), acc[3].x, acc[3].y));
   const float2 t = __fadd2_rn(__fadd2_rn(acc[0], acc[1]), __fadd2_rn(acc[2], acc[3]));
   return t.x + t.y;
 }
@@ -558,17 +559,19 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     if (!ok) *abortf = 1;
     for (int k = 0; ok; ++k) {
       if (!warp_wait_ready(&item_full[k & 1], (k >> 1) & 1, abortf, LIM)) { ok = false; break; }
-      ItemGeom g;
-      const bool more = load_item(s_item + (k & 1) * kItemWords, g);
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&item_empty[k & 1]);
-      if (!more) break;
-      if (g.n <= 0) continue;
+      // The record stays in shared memory until this warp is done with the item and is read
+      // where it is needed: its words would only take registers from the key loop.
+      const volatile int* rec = s_item + (k & 1) * kItemWords;
+      auto release = [&]() { __syncwarp(); if (lane == 0) mbar_arrive(&item_empty[k & 1]); };
+      if (!rec[kRecMore]) { release(); break; }
+      // key tiles this item has for tile X, and for both (none: the item is passed over by all roles)
+      const int slotB = rec[kRecSlot + 1], span = rec[kRecJe];
+      const int nA = max(0, min(span, rec[kRecNvis]) - rec[kRecJb]);
+      const int nB = slotB >= 0 ? max(0, min(span, rec[kRecNvis + 1]) - rec[kRecJb]) : 0;
+      const int nMine = X == 0 ? nA : nB;
       const int q_par = qcnt & 1;        // phase of q_full that carries this item's Q tiles
-      ++qcnt;
-      const int nMine = X == 0 ? g.nA : g.nB;
-      if (nMine == 0) continue;
-      const int winX = X == 0 ? g.un.winA : g.un.winB;
+      if (max(nA, nB) > 0) ++qcnt;
+      if (nMine == 0) { release(); continue; }
       if constexpr (F8) {
         // This thread's Q row, bf16 -> E4M3 with the power of two that brings its largest
         // magnitude into [128, 256) (exact), into the tile the MMAs read.  The 128-byte swizzle
@@ -603,42 +606,43 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
         }
         fence_proxy_async_smem();
         mbar_arrive(&q8_full[X]);
-        const int kvh = X == 0 ? g.kvhA : g.kvhB;
+        const int kvh = (rec[kRecKvh] >> (16 * X)) & 0xffff;
         sl2 = p.scale_log2 * __ldg(&p.k_scale[kvh]) * __int_as_float((127 - kq) << 23);
         out_scale = __ldg(&p.v_scale[kvh]);
       }
       float m_ref = -INFINITY, l = 0.f;
-      for (int j = 0; j < nMine; ++j) {
-        if (!warp_wait_ready(&s_full[X], cntS & 1, abortf, LIM)) { ok = false; break; }
-        ++cntS;
-        tc_fence_after();
-        const int limit = tile_limit(g, j, winX, p.resident);
-        if (limit == kTileN) {
-          // A full tile.  The whole row of S is read at once and the exponentials are taken against
-          // the running reference m_ref, which is only re-based when they grow past 2^8 (lazy
-          // rescale), so the common tile needs no separate max pass; the first tile of an item
-          // has no reference yet and takes one.  P goes over the last columns of S while the
-          // sum is still being formed: what it overwrites is kept in registers (s + P_COL) and
-          // the rest stays in TMEM, so the rare tile that has to be redone can be, and the
-          // check costs nothing on the way to the hand-off.
+      for (int j = 0; j < nMine;) {
+        // Tiles [j, full_end) are full: the whole prefix but its last tile, whole tiles of the window.
+        // They run in a loop of their own, without a call or a limit in it.
+        const int jb = rec[kRecJb], npt = rec[kRecNpt], winX = rec[kRecWin + X], prefix = rec[kRecPrefix] + (p.resident ? winX : 0);
+        const int full_end = min(nMine, (jb + j < npt ? prefix / kTileN : npt + winX / kTileN) - jb);
+        bool redo = false, grow = false;
+        for (; j < full_end; ++j) {
+          if (!warp_wait_ready(&s_full[X], cntS & 1, abortf, LIM)) { ok = false; break; }
+          ++cntS;
+          tc_fence_after();
+          // The whole row of S is read at once and the exponentials are taken against the running
+          // reference m_ref, which is only re-based when they grow past 2^8 (lazy rescale), so the
+          // common tile needs no separate max pass; the first tile of an item has no reference
+          // yet and takes one.  P goes over the last columns of S while the sum is still being
+          // formed: what it overwrites is kept in registers (s + P_COL) and the rest stays in
+          // TMEM, so the rare tile that has to be redone can be, and the check costs nothing on
+          // the way to the hand-off.
           uint32_t s[128], pk[32];
           tmem_ld32(tS, s); tmem_ld32(tS + 32, s + 32); tmem_ld32(tS + 64, s + 64); tmem_ld32(tS + 96, s + 96);
           tmem_ld_wait();
           if (j == 0) m_ref = max_cols<128>(s);
           const float mb = m_ref * sl2 - kShift;
-          float tile_sum;
-          bool grow;
+          float tile_sum, most;
           if constexpr (F8) {
-            float xm;
-            tile_sum = exp_cols<true, 128>(s, pk, sl2, mb, xm);
+            tile_sum = exp_cols<true, 128>(s, pk, sl2, mb, most);
             tmem_st32(tS + P_COL, pk);
-            grow = xm > kRescaleThreshold;
+            grow = !(most <= kGrowSum);
           } else {
-            float none;
             uint32_t pk2[32];
-            tile_sum = exp_cols<false, 64>(s, pk, sl2, mb, none);
+            tile_sum = exp_cols<false, 64>(s, pk, sl2, mb, most);
             tmem_st32(tS + P_COL, pk);
-            tile_sum += exp_cols<false, 64>(s + 64, pk2, sl2, mb, none);
+            tile_sum += exp_cols<false, 64>(s + 64, pk2, sl2, mb, most);
             tmem_st32(tS + P_COL + 32, pk2);
             grow = !(tile_sum <= kGrowSum);
           }
@@ -648,27 +652,38 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
 #pragma unroll
             for (int c = P_COL; c < 128; c += 32) tmem_st32(tS + c, s + c);
             tmem_st_wait();
-            const float2 r = tile_compact<D, F8>(tS, tO, kTileN, j == 0, grow, sl2, kShift, m_ref, l);
-            l = r.x; m_ref = r.y;
-          } else {
-            l += tile_sum;
+            redo = true;
+            break;
           }
-        } else {
-          const float2 r = tile_compact<D, F8>(tS, tO, limit, j == 0, false, sl2, kShift, m_ref, l);
-          l = r.x; m_ref = r.y;
+          l += tile_sum;
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&p_full[X]);
         }
+        if (!ok || j >= nMine) break;
+        // a ragged tile, or one that has to be taken again
+        if (!redo) {
+          if (!warp_wait_ready(&s_full[X], cntS & 1, abortf, LIM)) { ok = false; break; }
+          ++cntS;
+          tc_fence_after();
+        }
+        const int jj = rec[kRecJb] + j, np = rec[kRecNpt], wx = rec[kRecWin + X];
+        const int limit = redo ? kTileN
+                          : jj < np ? rec[kRecPrefix] + (p.resident ? wx : 0) - jj * kTileN : wx - (jj - np) * kTileN;
+        const float2 r = tile_compact<D, F8>(tS, tO, min(limit, kTileN), j == 0, redo && grow, sl2, kShift, m_ref, l);
+        l = r.x; m_ref = r.y;
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&p_full[X]);
+        ++j;
       }
       if (!ok) break;
       if (!warp_wait_ready(&o_full[X], cntO & 1, abortf, LIM)) { ok = false; break; }
       ++cntO;
       tc_fence_after();
-      if (g.un.n_chunks <= 1) {
-        const int slot = X == 0 ? g.un.slotA : g.un.slotB, t0 = X == 0 ? g.un.t0A : g.un.t0B;
-        const int grow_ = slot * p.bl + t0 + row / p.group;
-        const int head = (X == 0 ? g.kvhA : g.kvhB) * p.group + row % p.group;
+      if (rec[kRecChunks] <= 1) {
+        const int grow_ = rec[kRecSlot + X] * p.bl + rec[kRecT0 + X] + row / p.group;
+        const int head = ((rec[kRecKvh] >> (16 * X)) & 0xffff) * p.group + row % p.group;
         uint4* dst = reinterpret_cast<uint4*>(p.out + ((size_t)grow_ * p.n_q_heads + head) * D);
         const float inv = out_scale / l;
 #pragma unroll
@@ -686,7 +701,7 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
           }
         }
       } else {
-        const size_t tile = (size_t)(g.un.part_base + g.chunk) * 2 + X;
+        const size_t tile = (size_t)(rec[kRecPartBase] + rec[kRecChunk]) * 2 + X;
         // the reference the exponentials were taken against, and the sum (the merge divides by
         // it: the V scale goes in here)
         reinterpret_cast<float2*>(p.part_ml)[tile * kTileM + row] = make_float2(m_ref * sl2 - kShift, l / out_scale);
@@ -700,6 +715,7 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
         }
       }
       tc_fence_before();
+      release();
     }
   }
   // ---------------------------------------------------------------- teardown
