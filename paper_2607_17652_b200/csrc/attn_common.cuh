@@ -16,9 +16,11 @@ constexpr float kRescaleThreshold = 8.0f;   // log2 units (tiles that take a max
 constexpr float kGrowSum = 256.0f;
 // Dynamic shared memory per CTA.  Both sizes exceed half of the 227 KB an SM
 // offers, so two CTAs never share an SM: each CTA allocates all 512 TMEM columns.
-constexpr int kSmem64 = 120 * 1024;
-constexpr int kSmem128 = 6 * 32768 + 8192;
-constexpr int kSmemF8 = 2 * 32768 + 6 * 16384 + 8192;   // Q staging (bf16), Q / K / V tiles in 8 bits
+// Q, K and V tiles, 4 KB of output staging per softmax warp, barriers and 1 KB of alignment slack.
+constexpr int kStageBytes = 4096, kSmemExtra = 8 * kStageBytes + 2048;
+constexpr int kSmem64 = 6 * 16384 + kSmemExtra;
+constexpr int kSmem128 = 6 * 32768 + kSmemExtra;
+constexpr int kSmemF8 = 2 * 32768 + 6 * 16384 + kSmemExtra;   // Q staging (bf16), Q / K / V tiles in 8 bits
 // 8-bit pages: the exponentials are taken 2^4 above the reference, so that E4M3 (normal down to
 // 2^-6, largest value 448) holds P from 2^-10 of the reference up to the 2^8 bound of the lazy re-base
 constexpr float kF8PShift = 4.0f;

@@ -154,7 +154,8 @@ template <int D, bool F8>
 __global__ void __launch_bounds__(kAttnThreads, 1)
 wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmKwin,
                       const __grid_constant__ CUtensorMap tmVwin, const __grid_constant__ CUtensorMap tmKpool,
-                      const __grid_constant__ CUtensorMap tmVpool, const AttnParams p) {
+                      const __grid_constant__ CUtensorMap tmVpool, const __grid_constant__ CUtensorMap tmOut,
+                      const AttnParams p) {
   static_assert(!F8 || D == 128, "8-bit pages: head_dim 128 only (one 128-byte swizzle row per key)");
   constexpr int NH = D / 64;                 // 64-element halves of the head dim (bf16 tiles)
   constexpr int Q_TILE_BYTES = NH * 16384;   // one 128-row bf16 tile
@@ -169,7 +170,8 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
   uint8_t* sQ8 = sQ + 2 * Q_TILE_BYTES;      // [2] the same in E4M3 (F8 only)
   uint8_t* sK = sQ8 + (F8 ? 2 * 16384 : 0);  // [2] stages
   uint8_t* sV = sK + 2 * TILE_BYTES;         // [2] stages
-  uint64_t* bars = reinterpret_cast<uint64_t*>(sV + 2 * TILE_BYTES);
+  uint8_t* sOut = sV + 2 * TILE_BYTES;       // [8] output staging of the softmax warps
+  uint64_t* bars = reinterpret_cast<uint64_t*>(sOut + 8 * kStageBytes);
   uint64_t* q_full = bars + 0;
   uint64_t* q_empty = bars + 1;
   uint64_t* k_full = bars + 2;    // [2]
@@ -203,7 +205,7 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     mbar_init(&q8_full[0], 128); mbar_init(&q8_full[1], 128);
     fence_mbar_init();
     tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmKwin); tma_prefetch_desc(&tmVwin);
-    tma_prefetch_desc(&tmKpool); tma_prefetch_desc(&tmVpool);
+    tma_prefetch_desc(&tmKpool); tma_prefetch_desc(&tmVpool); tma_prefetch_desc(&tmOut);
   }
   if (warp == 1) { tmem_alloc(tmem_slot, 512); tmem_relinquish(); }
   tc_fence_before();
@@ -216,11 +218,12 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
   // warpgroups.  All four warps of a warpgroup execute the same setmaxnreg
   // instruction, and each role's code is dominated by its warpgroup's one.
   // Registers only move inside the CTA: what the two softmax warpgroups take
-  // (2 x 128 x (192 - 168)) must not exceed what the control warpgroup gives up
-  // (128 x (168 - 120)), or setmaxnreg.inc blocks for good.  (88 / 208 measured 1 % slower on
-  // the long-context workload: the control roles spill.)
+  // (2 x 128 x (200 - 168)) must not exceed what the control warpgroup gives up
+  // (128 x (168 - 104)), or setmaxnreg.inc blocks for good.  (Cycles per launch on the long-context
+  // workload, bf16 / 8-bit pages: 88 / 208 registers 1.478 M / 1.364 M, 104 / 200 1.464 M / 1.344 M,
+  // 120 / 192 1.477 M / 1.361 M, 136 / 184 1.483 M / 1.413 M.)
   if (warp < 4) {
-  asm volatile("setmaxnreg.dec.sync.aligned.u32 120;");
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 104;");
   if (warp == 0 || warp == 2) {
     // ----------------------------------------------------------- producers
     // Warp 0 owns K/V stage 0, warp 2 owns stage 1; warp 0 also draws the work
@@ -544,7 +547,7 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     // Four warps per Q tile, one thread per query row (its TMEM lane).  Every wait is
     // taken by the whole warp with one outcome (warp_wait): tcgen05.ld / st below are
     // warp-wide and must never run with part of a warp gone.
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 192;");
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 200;");
     const int X = (warp - 4) >> 2;                 // 0: tile A, 1: tile B
     const int quad = warp & 3;                     // TMEM lane quadrant of this warp
     const int row = quad * 32 + lane;              // query row of the tile
@@ -682,23 +685,32 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       ++cntO;
       tc_fence_after();
       if (rec[kRecChunks] <= 1) {
-        const int grow_ = rec[kRecSlot + X] * p.bl + rec[kRecT0 + X] + row / p.group;
-        const int head = ((rec[kRecKvh] >> (16 * X)) & 0xffff) * p.group + row % p.group;
-        uint4* dst = reinterpret_cast<uint4*>(p.out + ((size_t)grow_ * p.n_q_heads + head) * D);
+        // 64 columns of the warp's 32 rows at a time through its staging area (swizzled like the
+        // tiles: 16-byte piece c of row r at c ^ (r & 7)) and out as one box of whole lines.  Plain
+        // stores from the lanes' rows kept the softmax warps for 4,000 cycles per item.
+        const int row0 = quad * 32, kvh = (rec[kRecKvh] >> (16 * X)) & 0xffff;
+        const int y = kvh * p.group + row0 % p.group, z = rec[kRecSlot + X] * p.bl + rec[kRecT0 + X] + row0 / p.group;
+        uint8_t* stage = sOut + (warp - 4) * kStageBytes;
         const float inv = out_scale / l;
 #pragma unroll
-        for (int c = 0; c < D / 32; ++c) {
-          uint32_t o[32];
-          tmem_ld32(tO + c * 32, o);
+        for (int h = 0; h < NH; ++h) {
+          uint32_t o[64];
+          tmem_ld32(tO + h * 64, o);
+          tmem_ld32(tO + h * 64 + 32, o + 32);
+          if (lane == 0) bulk_wait_read();           // the staging area's previous contents are out
+          __syncwarp();
           tmem_ld_wait();
 #pragma unroll
-          for (int i = 0; i < 2; ++i) {              // two 32-byte stores: whole sectors
-            uint32_t v[8];
+          for (int c = 0; c < 8; ++c) {
+            uint32_t v[4];
 #pragma unroll
-            for (int k = 0; k < 8; ++k)
-              v[k] = pack_bf16x2(__uint_as_float(o[16 * i + 2 * k]) * inv, __uint_as_float(o[16 * i + 2 * k + 1]) * inv);
-            st_global_v8(dst + c * 4 + 2 * i, v);
+            for (int i = 0; i < 4; ++i)
+              v[i] = pack_bf16x2(__uint_as_float(o[8 * c + 2 * i]) * inv, __uint_as_float(o[8 * c + 2 * i + 1]) * inv);
+            *reinterpret_cast<uint4*>(stage + lane * 128 + ((c ^ (lane & 7)) << 4)) = make_uint4(v[0], v[1], v[2], v[3]);
           }
+          fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0) { tma_store_3d(&tmOut, stage, h * 64, y, z); bulk_commit(); }
         }
       } else {
         const size_t tile = (size_t)(rec[kRecPartBase] + rec[kRecChunk]) * 2 + X;
@@ -717,6 +729,7 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       tc_fence_before();
       release();
     }
+    if (lane == 0) bulk_wait_done();
   }
   // ---------------------------------------------------------------- teardown
   tc_fence_before();
@@ -925,13 +938,16 @@ int launch_attn_combine(fb_ctx* ctx, const AttnParams& p, int list, cudaStream_t
                   "attn_combine_kernel launch");
 }
 
-static int encode_q(fb_ctx* ctx, const void* q) {
+// q and out have one shape; Q is loaded as whole tiles, the output leaves 32 rows at a time
+static int encode_q_out(fb_ctx* ctx, const void* q, const void* out) {
   const fb_config& c = ctx->cfg;
   const cuuint64_t rows = (cuuint64_t)c.max_requests * c.wmax * c.block_len, D = c.head_dim;
   cuuint64_t dims[3] = {D, (cuuint64_t)c.n_q_heads, rows};
   cuuint64_t str[2] = {D * 2, (cuuint64_t)c.n_q_heads * D * 2};
   cuuint32_t box[3] = {64, (cuuint32_t)ctx->group, (cuuint32_t)ctx->tokens_per_tile};
-  return encode(ctx, &ctx->tm_q, q, 3, dims, str, box);
+  if (int e = encode(ctx, &ctx->tm_q, q, 3, dims, str, box)) return e;
+  cuuint32_t obox[3] = {64, (cuuint32_t)(ctx->group < 32 ? ctx->group : 32), (cuuint32_t)(ctx->group < 32 ? 32 / ctx->group : 1)};
+  return encode(ctx, &ctx->tm_out, out, 3, dims, str, obox);
 }
 
 int launch_attn(fb_ctx* ctx, const fb_pack* pk, const void* q, const void* k_win, const void* v_win,
@@ -942,9 +958,9 @@ int launch_attn(fb_ctx* ctx, const fb_pack* pk, const void* q, const void* k_win
   const fb_config& c = ctx->cfg;
   const cuuint64_t rows = (cuuint64_t)c.max_requests * c.wmax * c.block_len;
   const cuuint64_t D = c.head_dim;
-  const void* ptrs[5] = {q, k_win, v_win, k_pool, v_pool};
+  const void* ptrs[6] = {q, k_win, v_win, k_pool, v_pool, out};
   if (ctx->maps_f8 || memcmp(ptrs, ctx->map_ptrs, sizeof(ptrs)) != 0) {
-    if (int e = encode_q(ctx, q)) return e;
+    if (int e = encode_q_out(ctx, q, out)) return e;
     {
       cuuint64_t dims[3] = {D, (cuuint64_t)c.n_kv_heads, rows};
       cuuint64_t str[2] = {D * 2, (cuuint64_t)c.n_kv_heads * D * 2};
@@ -970,7 +986,7 @@ int launch_attn(fb_ctx* ctx, const fb_pack* pk, const void* q, const void* k_win
   const int grid = ctx->num_sms;
   if (c.head_dim == 64) {
     if (int e = cuda_err(ctx, launch_pdl(wavefront_attn_kernel<64, false>, grid, kAttnThreads, kSmem64, stream, ctx->tm_q,
-                                         ctx->tm_kwin, ctx->tm_vwin, ctx->tm_kpool, ctx->tm_vpool, p),
+                                         ctx->tm_kwin, ctx->tm_vwin, ctx->tm_kpool, ctx->tm_vpool, ctx->tm_out, p),
                          "wavefront_attn_kernel launch"))
       return e;
     return launch_attn_combine(ctx, p, 0, stream);
@@ -979,7 +995,7 @@ int launch_attn(fb_ctx* ctx, const fb_pack* pk, const void* q, const void* k_win
   if (ctx->pair_on)
     if (int e = launch_attn_pair(ctx, page_table, out, ws, status, stream)) return e;
   if (int e = cuda_err(ctx, launch_pdl(wavefront_attn_kernel<128, false>, grid, kAttnThreads, kSmem128, stream, ctx->tm_q,
-                                       ctx->tm_kwin, ctx->tm_vwin, ctx->tm_kpool, ctx->tm_vpool, p),
+                                       ctx->tm_kwin, ctx->tm_vwin, ctx->tm_kpool, ctx->tm_vpool, ctx->tm_out, p),
                        "wavefront_attn_kernel launch"))
     return e;
   return launch_attn_combine(ctx, p, 0, stream);
@@ -993,9 +1009,9 @@ int launch_attn_fp8(fb_ctx* ctx, const fb_pack* pk, const void* q, const void* k
   (void)pk;
   if (int e = ensure_device(ctx)) return e;
   const fb_config& c = ctx->cfg;
-  const void* ptrs[5] = {q, nullptr, nullptr, k_pool8, v_pool8};
+  const void* ptrs[6] = {q, nullptr, nullptr, k_pool8, v_pool8, out};
   if (!ctx->maps_f8 || memcmp(ptrs, ctx->map_ptrs, sizeof(ptrs)) != 0) {
-    if (int e = encode_q(ctx, q)) return e;
+    if (int e = encode_q_out(ctx, q, out)) return e;
     cuuint64_t dims[2] = {128, (cuuint64_t)c.num_pages * c.n_kv_heads * kPage};
     cuuint64_t str[1] = {128};
     cuuint32_t box[2] = {128, 64};
@@ -1009,7 +1025,7 @@ int launch_attn_fp8(fb_ctx* ctx, const fb_pack* pk, const void* q, const void* k
   fill_attn_params(ctx, p, page_table, out, ws, status, 0);
   p.k_scale = k_scale; p.v_scale = v_scale;
   if (int e = cuda_err(ctx, launch_pdl(wavefront_attn_kernel<128, true>, ctx->num_sms, kAttnThreads, (size_t)kSmemF8, stream,
-                                       ctx->tm_q, ctx->tm_kwin, ctx->tm_vwin, ctx->tm_kpool, ctx->tm_vpool, p),
+                                       ctx->tm_q, ctx->tm_kwin, ctx->tm_vwin, ctx->tm_kpool, ctx->tm_vpool, ctx->tm_out, p),
                        "wavefront_attn_kernel (8-bit pages) launch"))
     return e;
   return launch_attn_combine(ctx, p, 0, stream);

@@ -237,8 +237,9 @@ struct fb_ctx {
   void* encode_fn = nullptr;
   // cached tensor maps (re-encoded when a base pointer changes)
   CUtensorMap tm_kwin_half;   // 64-row boxes of the window keys (CTA-pair kernel)
-  const void* map_ptrs[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
+  const void* map_ptrs[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
   bool maps_f8 = false;   // the cached pool maps describe 8-bit pages
+  CUtensorMap tm_out;        // 64-column boxes of 32 output rows
   CUtensorMap tm_q, tm_kwin, tm_vwin, tm_kpool, tm_vpool;
 };
 
