@@ -504,37 +504,27 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
         issue_qk(1, 1, round16(g.limit(0, g.winB, p.resident)));
         commit(&k_empty[1]);
         if (n == 1) commit(q_empty);
-        // The streams do not depend on each other: serve whichever tile's P is ready.
-        int jA = 0, jB = 0, qk_left = 2 * (n - 1), spins = 0;
-        long long t0 = clock64();
-        while (jA < n || jB < n) {
-          int X = -1;
-          if (jA < n && __all_sync(0xffffffffu, mbar_test(&p_full[0], cntPA & 1))) X = 0;
-          else if (jB < n && __all_sync(0xffffffffu, mbar_test(&p_full[1], cntPB & 1))) X = 1;
-          if (X < 0) {
-            if ((++spins & 63) == 0) {
-              bool give_up = *abortf != 0;
-              if (!give_up && clock64() - t0 > LIM) { *abortf = 1; give_up = true; }
-              if (__any_sync(0xffffffffu, give_up)) { ok = false; break; }
-            }
-            continue;
-          }
-          const int j = X ? jB : jA;
-          if (X) { ++jB; ++cntPB; } else { ++jA; ++cntPA; }
-          if (!wait_v(X)) { ok = false; break; }
-          tc_fence_after();
-          issue_pv(X, X, pv_steps(g.limit(j, g.winA, p.resident)), j > 0);
-          commit(&v_empty[X]);
-          if (j + 1 < n) {
-            // this stream's next K tile could only be requested when its last Q K^T had
-            // finished, one softmax ago: give it the time of the P V as well
-            if (!wait_k(X)) { ok = false; break; }
+        // The streams do not depend on each other but run alike: taken in turn.  (Serving whichever
+        // tile's P is ready first means polling.)
+        for (int j = 0; j < n && ok; ++j) {
+#pragma unroll 1
+          for (int X = 0; X < 2; ++X) {
+            if (!wait_v(X)) { ok = false; break; }
+            if (!wait(&p_full[X], (X ? cntPB : cntPA) & 1)) { ok = false; break; }
+            if (X) ++cntPB; else ++cntPA;
             tc_fence_after();
-            issue_qk(X, X, round16(g.limit(j + 1, g.winA, p.resident)));
-            commit(&k_empty[X]);
-            if (--qk_left == 0) commit(q_empty);
+            issue_pv(X, X, pv_steps(g.limit(j, g.winA, p.resident)), j > 0);
+            commit(&v_empty[X]);
+            if (j + 1 < n) {
+              // this stream's next K tile could only be requested when its last Q K^T had
+              // finished, one softmax ago: give it the time of the P V as well
+              if (!wait_k(X)) { ok = false; break; }
+              tc_fence_after();
+              issue_qk(X, X, round16(g.limit(j + 1, g.winA, p.resident)));
+              commit(&k_empty[X]);
+              if (j + 2 == n && X == 1) commit(q_empty);
+            }
           }
-          t0 = clock64();
         }
       }
       if (!ok) break;
