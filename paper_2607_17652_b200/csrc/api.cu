@@ -47,7 +47,7 @@ WsLayout make_ws_layout(const fb_ctx* ctx) {
     // split pieces: the bound that split_rule derives (per scheduling unit; list 1 has two records
     // per unit), and never more than every unit cut into pieces of the minimum length (a unit spans
     // at most the keys its page-table row can address)
-    const int min_chunk = l == 0 && ctx->auto_min_chunk < ctx->min_chunk_tiles ? ctx->auto_min_chunk : ctx->min_chunk_tiles;
+    const int min_chunk = l == 0 && estimates_split(c) && ctx->auto_min_chunk < ctx->min_chunk_tiles ? ctx->auto_min_chunk : ctx->min_chunk_tiles;
     const long long every = max_tiles > min_chunk ? units * ((max_tiles + min_chunk - 1) / min_chunk) : 0;
     const long long by_target = mult * ((long long)kPartsPerTarget * target + 8);
     x.max_units = (int)units;
@@ -137,7 +137,7 @@ int fb_create(const fb_config* cfg, fb_ctx** out) {
   ctx->target_items = fb::kDefaultTargetItems;
   ctx->min_chunk_tiles = fb::kDefaultMinChunkTiles;
   ctx->wait_cycles = fb::kDefaultWaitCycles;
-  ctx->auto_split = 1;
+  ctx->auto_split = fb::estimates_split(c);
   ctx->auto_min_chunk = fb::kAutoMinChunkTiles;
   ctx->pair_on = 0;                      // the CTA-pair kernel is opt-in (fb_tuning.attn_pair)
   ctx->sm_scale = c.sm_scale > 0.f ? c.sm_scale : 1.0f / sqrtf((float)c.head_dim);
@@ -154,7 +154,7 @@ int fb_set_tuning(fb_ctx* ctx, const fb_tuning* t) {
     return fail(ctx, FB_ERR_INVALID_ARG, "a tuning value is out of range");
   ctx->target_items = t->attn_target_items ? t->attn_target_items : fb::kDefaultTargetItems;
   ctx->min_chunk_tiles = t->attn_min_chunk_tiles ? t->attn_min_chunk_tiles : fb::kDefaultMinChunkTiles;
-  ctx->auto_split = t->attn_target_items == 0;
+  ctx->auto_split = t->attn_target_items == 0 && fb::estimates_split(ctx->cfg);
   ctx->auto_min_chunk = t->attn_min_chunk_tiles ? t->attn_min_chunk_tiles : fb::kAutoMinChunkTiles;
   ctx->wait_cycles = t->wait_cycles ? (long long)t->wait_cycles : fb::kDefaultWaitCycles;
   ctx->pair_on = ctx->cfg.head_dim == 128 && !ctx->cfg.kv_fp8 && t->attn_pair;

@@ -139,6 +139,10 @@ __host__ __device__ inline SplitRule split_rule(int total, int units, int target
 // 2 to 3 us less on 64 and 128 requests.
 // With two units an SM and more, and items so long that half of one outweighs their cost twice,
 // the last 15 % of the work are cut into filler pieces as above (16 long contexts: 1064 -> 1030).
+// Not with 8-bit pages: E4M3 weights are rounded (2^-4 a step) against the reference of their piece,
+// so two splits of a range differ by up to 3.5e-2 in the 2-norm where bf16 ones differ by 2e-3.
+// There the rule without an estimate stands, two items an SM: the same results whatever the rest.
+__host__ __device__ inline bool estimates_split(const fb_config& c) { return !c.kv_fp8; }
 constexpr int kTileCost = 16, kTileDualCost = 22, kItemCost = 40, kPieceCost = 45, kMergeCost = 50, kMergePieceNs = 26;
 constexpr int kSplitCandidates = 32;
 // Candidate i: the longest range (`longest` key tiles) divided by 1, 1.25, 1.5, 1.75, 2, 2.25, 2.5,

@@ -34,6 +34,17 @@ def test_estimated_split_fits_and_leaves_nothing_out():
     assert ctx.attn_plan([300] * 28, [4] * 28)["parts"] == 0
 
 
+def test_eight_bit_pages_are_not_split_by_estimate():
+    # (their weights are rounded against a reference per piece: another split, another rounding)
+    rg = np.random.default_rng(12)
+    fp8 = dict(kv_fp8=1, window_in_pages=1)
+    ctx, fixed = B.Context(**_cfg(**fp8)), B.Context(tuning=dict(attn_target_items=296, attn_min_chunk_tiles=4), **_cfg(**fp8))
+    for _ in range(100):
+        n = int(rg.integers(1, 65))
+        P, w = rg.integers(0, int(2 ** rg.uniform(5, 15)), size=n), rg.integers(0, 5, size=n)
+        assert ctx.attn_plan(P, w) == fixed.attn_plan(P, w)
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("n_requests,prefix,w,resident", [
     (1, (64, 64), (2, 2), 0), (1, (3001, 3001), (1, 1), 1), (2, (9000, 12000), (3, 3), 0), (9, (100, 2500), (1, 4), 1),
