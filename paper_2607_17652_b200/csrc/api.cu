@@ -48,7 +48,8 @@ WsLayout make_ws_layout(const fb_ctx* ctx) {
     // per unit), and never more than every unit cut into pieces of the minimum length (a unit spans
     // at most the keys its page-table row can address)
     const int min_chunk = l == 0 && estimates_split(c) && ctx->auto_min_chunk < ctx->min_chunk_tiles ? ctx->auto_min_chunk : ctx->min_chunk_tiles;
-    const long long every = max_tiles > min_chunk ? units * ((max_tiles + min_chunk - 1) / min_chunk) : 0;
+    const bool never = l == 0 && ctx->auto_split && ctx->auto_min_chunk == kAutoMinChunkTiles && max_tiles <= kNeverSplitTiles;
+    const long long every = !never && max_tiles > min_chunk ? units * ((max_tiles + min_chunk - 1) / min_chunk) : 0;
     const long long by_target = mult * ((long long)kPartsPerTarget * target + 8);
     x.max_units = (int)units;
     x.max_parts = units ? (int)(by_target < every ? by_target : every) : 0;

@@ -17,6 +17,13 @@ constexpr int kPage = 64;
 constexpr int kSms = 148;
 constexpr int kDefaultMinChunkTiles = 4;
 constexpr int kAutoMinChunkTiles = 2;          // the same where the split is chosen by estimate (no target given)
+// A context whose page-table rows reach no further than this many key tiles is never split without a
+// target from the caller: the estimate below would not (a merge costs what three tiles do), and
+// then neither room for pieces nor the launch of the merge is needed, 2 us of a call that takes 7
+// to 30 (one request of a 4-head model, 2 / 6 tiles: 7.9 -> 6.9, 14.1 -> 13.0 us; 8 requests of a
+// 32-head model: 11.8 -> 9.6, 21.7 -> 18.8).  At 7 tiles a single request is better cut in three: 12.0
+// against 14.5 us.
+constexpr int kNeverSplitTiles = 6;
 constexpr int kDefaultTargetItems = 2 * kSms;  // about two work items per SM before key ranges are split
 
 // One unit = two Q tiles of one request that run side by side in a CTA: either

@@ -45,6 +45,16 @@ def test_eight_bit_pages_are_not_split_by_estimate():
         assert ctx.attn_plan(P, w) == fixed.attn_plan(P, w)
 
 
+def test_short_contexts_have_no_pieces():
+    # rows of 10 and 11 pages: a prefix of 608 / 672 tokens and a window of one block, 6 / 7 key tiles
+    plan = lambda tuning, pages: B.Context(tuning=tuning, **_cfg(max_pages_per_req=pages)).attn_plan([128] * 2, [4] * 2)
+    assert plan(None, 10)["max_parts"] == 0 and plan(None, 10)["parts"] == 0
+    assert plan(None, 11)["max_parts"] > 0
+    # what the caller asks for is done
+    assert plan(dict(attn_target_items=8), 10)["max_parts"] > 0
+    assert plan(dict(attn_min_chunk_tiles=1), 10)["max_parts"] > 0
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("n_requests,prefix,w,resident", [
     (1, (64, 64), (2, 2), 0), (1, (3001, 3001), (1, 1), 1), (2, (9000, 12000), (3, 3), 0), (9, (100, 2500), (1, 4), 1),
