@@ -36,6 +36,13 @@ if ROOT not in sys.path:
 METRIC = "packed-wavefront attn TFLOP/s & T2T-step GB/s (fraction of B200 peak)"
 DEFAULT_WORKLOAD = 2
 KERNELS_PER_STEP = 6   # pack, attention, split-KV combine, T2T rows, T2T update, gate/commit
+
+
+def kernels_per_step(ctx):
+    """A context that never splits a key range launches no combine kernel."""
+    return KERNELS_PER_STEP - (ctx.attn_plan([1], [1])["max_parts"] == 0)
+
+
 # dram__bytes_read.sum + dram__bytes_write.sum from the ncu captures summarised
 # under profiles/, as a ratio to the algorithmic bytes of the captured (smaller)
 # case of the same workload; a full launch's traffic is that ratio times its
@@ -582,7 +589,7 @@ def run_ours(args):
                     "ms_per_step": round(e2e_ms_max, 3), "h2d_bytes_per_step": h2d,
                     "d2h_bytes_per_step": d2h,
                     "t2t_gbs": round(t2tb_all / e2e_ms_max / 1e6, 2)},
-            "gpu_launches": KERNELS_PER_STEP * args.steps,
+            "gpu_launches": kernels_per_step(ctx) * args.steps,
             "kernels": {"pack_ms": round(float(seg[:, 0].mean()), 4), "attn_ms": round(attn_ms, 4),
                         "t2t_ms": round(t2t_ms, 4), "gate_commit_ms": round(float(seg[:, 3].mean()), 4),
                         "attn_tflops": round(attn_tf, 2), "t2t_gbs": round(t2t_gbs, 1),
@@ -755,7 +762,7 @@ def run_sweep(args):
         "clocks": clocks,
         "e2e": {"value": None, "unit": "TFLOP/s", "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 0,
                 "note": "the sweep is timed with resident inputs only; see the default run for host buffers"},
-        "gpu_launches": KERNELS_PER_STEP * n_steps,
+        "gpu_launches": kernels_per_step(ctx) * n_steps,
         "kernels": {"pack_ms": round(float(seg[:, 0].mean()), 4), "attn_ms": round(attn_ms / n_steps, 4),
                     "t2t_ms": round(t2t_ms / n_steps, 4), "gate_commit_ms": round(float(seg[:, 3].mean()), 4),
                     "attn_tflops": round(attn_tf, 2), "t2t_gbs": round(t2t_gbs, 1)},

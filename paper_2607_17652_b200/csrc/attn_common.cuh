@@ -49,23 +49,6 @@ struct ItemGeom {
   int jb, n, nA, nB, chunk, kvhA, kvhB;
 };
 
-__device__ __forceinline__ bool load_item(const AttnParams& p, int idx, ItemGeom& g) {
-  const int4 it = *reinterpret_cast<const int4*>(&p.items[idx]);
-  const int4* up = reinterpret_cast<const int4*>(&p.units[it.x]);
-  const int4 u0 = up[0], u1 = up[1], u2 = up[2], u3 = up[3];
-  g.un.req = u0.x; g.un.kvh = u0.y; g.un.slotA = u0.z; g.un.slotB = u0.w;
-  g.kvhA = u0.y & 0xffff; g.kvhB = u0.y >> 16;
-  g.un.t0A = u1.x; g.un.t0B = u1.y; g.un.n_tiles = u1.z; g.un.n_chunks = u1.w;
-  g.un.nvisA = u2.x; g.un.nvisB = u2.y; g.un.part_base = u2.z; g.un.prefix_len = u2.w;
-  g.un.npt = u3.x; g.un.win_row0 = u3.y; g.un.winA = u3.z; g.un.winB = u3.w;
-  g.chunk = it.y; g.jb = it.z;
-  const int je = it.w;
-  g.nA = max(0, min(je, g.un.nvisA) - g.jb);
-  g.nB = g.un.slotB >= 0 ? max(0, min(je, g.un.nvisB) - g.jb) : 0;
-  g.n = max(g.nA, g.nB);
-  return g.n > 0;
-}
-
 // Work item records in shared memory: 4 words of the item, 16 of the unit, 1 = there is one.
 constexpr int kItemWords = 24;
 // One warp copies item idx (and its unit) there, or the end mark if there are no more than n_items.
@@ -146,17 +129,6 @@ struct ItemU {
   }
 };
 
-__device__ __forceinline__ bool load_item_uniform(const AttnParams& p, int idx, ItemU& u) {
-  ItemGeom g;
-  load_item(p, idx, g);
-  u.req = uni(g.un.req); u.kvhA = uni(g.kvhA); u.kvhB = uni(g.kvhB);
-  u.rowA = uni(g.un.slotA * p.bl + g.un.t0A); u.rowB = uni(g.un.slotB * p.bl + g.un.t0B);
-  u.jb = uni(g.jb); u.n = uni(g.n); u.nA = uni(g.nA); u.nB = uni(g.nB);
-  u.npt = uni(g.un.npt); u.prefix_len = uni(g.un.prefix_len); u.win_row0 = uni(g.un.win_row0);
-  u.winA = uni(g.un.winA); u.winB = uni(g.un.winB);
-  return u.n > 0;
-}
-
 __device__ __forceinline__ bool load_item_uniform(const int* src, const AttnParams& p, ItemU& u) {
   ItemGeom g;
   const bool more = load_item(src, g);
@@ -183,13 +155,6 @@ __device__ __forceinline__ bool warp_wait_ready(uint64_t* bar, uint32_t parity, 
   return warp_wait(bar, parity, abort, limit);
 }
 
-// number of keys of local tile j that tile X (window reach winX) may see
-__device__ __forceinline__ int tile_limit(const ItemGeom& g, int j, int winX, int resident) {
-  const int gj = g.jb + j;
-  const int lim = gj < g.un.npt ? g.un.prefix_len + (resident ? winX : 0) - gj * kTileN
-                                : winX - (gj - g.un.npt) * kTileN;
-  return min(lim, kTileN);
-}
 // Unnormalised O of a split piece in the workspace: `tile` = 2 * piece + Q tile, 8 columns (32 bytes)
 // of a row together and the 128 rows of a tile side by side, so that a warp whose lanes hold
 // successive rows stores and loads whole kilobytes (a row-major layout took 6000 cycles a piece).

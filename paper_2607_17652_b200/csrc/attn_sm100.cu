@@ -16,16 +16,17 @@
 //               last columns of S in TMEM; epilogue
 //   warps 8-11  the same for tile B
 // What bounds it: at full load the board's power limit (the SM clock falls from 1965
-// to about 1500 MHz), so both fewer cycles and fewer instructions pay; below that,
-// the chain S -> P -> P V -> next S of a tile (about 2500 cycles against 2048 of
-// MMA time for the two tiles of a CTA).  Sustained, back to back, before and after
-// the present form of the loop: long-context workload 1259 -> 1184 us, 64 requests
-// 458 -> 428 us, 128 requests 498 -> 466 us, long context in 8 bits 996 -> 962 us.
+// to about 1450 MHz), so both fewer cycles and fewer instructions pay; below that,
+// the chain S -> P -> P V -> next S of a tile (2600 to 2900 cycles against 2048 of
+// MMA time and as many of MUFU time for the two tiles of a CTA).  Sustained, back to
+// back, with the loop's former form and now: long-context workload 1259 -> 1165 us,
+// 64 requests 458 -> 424 us, 128 requests 498 -> 469 us, long context in 8 bits 996 ->
+// 880 us.
 // A Q tile is 128 rows = (128/G tokens) x (G query heads of one KV head) of one
 // slot.  A unit runs two Q tiles side by side: two tiles of one request and KV
 // head, which share each K/V tile from shared memory, or the odd tile left
 // over, run under two adjacent KV heads at once (two K/V streams, served in
-// readiness order).  The mask is per tile: a tile of the frozen prefix is
+// turn).  The mask is per tile: a tile of the frozen prefix is
 // fully visible except the ragged last one; the window tile is visible up to
 // (s+1)*bl keys for a query in window slot s.  Tiles nobody can see are never
 // loaded (the work list only spans visible tiles), and ragged tiles run the
@@ -58,11 +59,11 @@ __device__ __forceinline__ float max_cols(const uint32_t* s) {
 // the unrounded values returned; `most`: the largest of eight partial sums of N / 8 values each, a
 // bound on every value that costs three instructions a row (8-bit P saturates, so it needs one:
 // the largest value itself took one instruction per pair and 10 % of that kernel's time).  A masked
-// score (-inf) comes out as exactly 0.  All exponentials run on the MUFU pipe: moving a quarter of
-// them to a polynomial on the FMA pipe shortens the loop in cycles, but at full load this kernel
-// runs at the board's power limit, where the ~13 extra instructions per pair cost more clock than
-// that gains (long-context workload, sustained: 1205 us without against 1262 us with the
-// polynomial; 64 requests 442 against 464; 8-bit pages 970 against 974).
+// score (-inf) comes out as exactly 0.  All exponentials run on the MUFU pipe: moving 1/16 to 1/4 of
+// them to a polynomial on the FMA pipe shortens the loop in cycles by up to 2.5 %, but at full load
+// this kernel runs at the board's power limit, where the ~13 extra instructions per pair cost more
+// clock than that gains (long-context workload, sustained: 1164 us without against 1174 to 1205 with
+// a polynomial share; 64 requests 424 against 426 to 439; 8-bit pages 883 against 883 to 896).
 template <bool F8, int N>
 __device__ __forceinline__ float exp_cols(const uint32_t* s, uint32_t* pk, float sl2, float mb, float& most) {
   const float2 sl2v = make_float2(sl2, sl2), nmb = make_float2(-mb, -mb);
@@ -748,11 +749,13 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
 // of at least 256 bytes.  Each lane carries a running maximum along, the groups meet by shuffles.
 // A CTA keeps its rows and columns and goes over every G-th unit, picking the split ones 32 at a
 // time; it returns at once when no unit was split.
-// Bound by latency (a round of loads takes 2 to 3 us under this load), so W grows with the longest
-// split of the batch, up to the point where the CTAs no longer run together: attention call in us
-// with W = 1 / 2 / 4: one request of 3,000 tokens (6 pieces a unit) 20.9 / 19.3 / 20.1, 28,000
-// tokens (12 pieces) 84 / 76 / 65, 8 requests (3 pieces, 40 units) 23.6 / 26.9 / 29; with a warp
-// per row over a row-major layout these took 23.1, 97 and 26.4.
+// Bound by the partials' way through the L2 (12 to 19 MB written on one SM and read on another) and
+// by the latency of a round of such loads, 2 to 3 us, so W grows with the longest split of the
+// batch, up to the point where the CTAs no longer run together: attention call in us with W = 1 / 2 / 4:
+// one request of 3,000 tokens (6 pieces a unit) 20.9 / 19.3 / 20.1, 28,000 tokens (12 pieces) 84 / 76 /
+// 65, 8 requests (3 pieces, 40 units) 23.6 / 26.9 / 29; with a warp per row over a row-major layout
+// these took 23.1, 97 and 26.4.  Of the present calls (18.3, 55, 23.1) the merge is 6, 10 and 6 us, an
+// empty one 2.
 constexpr int kCombineThreads = 256, kCombineCtasPerSm = 8, kCombineDepth = 4, kCombineMostCtas = 1024, kCombineMaxWays = 4;
 template <int D>
 __global__ void __launch_bounds__(kCombineThreads, 3) attn_combine_kernel(const AttnParams p) {
