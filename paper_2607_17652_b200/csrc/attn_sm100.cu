@@ -213,7 +213,12 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  pdl_wait();                     // the work list (and everything else) of the previous kernels is complete
+  // The work list (and everything else) of the previous kernels is complete.  Without an early start
+  // of the next kernel: where no merge stands between, the row pass came up under this kernel's
+  // division of the SM and read at 0.9 of its rate (attention + row pass, 36 requests of 100 tokens, 6912
+  // rows: 352 us, the two alone 14 + 309, now 325; a step of 24 short requests with four layers and
+  // their scatters 319 -> 290).  Where a merge follows it makes no difference (8 requests 23.4 / 23.2).
+  pdl_wait_only();
 
   // The control warpgroup (warps 0-3) hands registers to the softmax
   // warpgroups.  All four warps of a warpgroup execute the same setmaxnreg

@@ -288,6 +288,11 @@ __device__ __forceinline__ void pdl_wait() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
+// The wait alone: the next kernel is scheduled when this one is complete.  For a kernel that takes
+// nearly all shared memory of its SM: CTAs that move in beside its last ones inherit its division
+// between shared memory and L1, which only changes on an idle SM, and kernels that live on loads in
+// flight keep too little of the latter.
+__device__ __forceinline__ void pdl_wait_only() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 #endif
 
 int launch_pack(fb_ctx*, const fb_state*, const fb_pack*, void* ws, int32_t* status, cudaStream_t);
