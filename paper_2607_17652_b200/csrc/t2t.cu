@@ -304,6 +304,17 @@ __global__ void __launch_bounds__(128) t2t_update_kernel(const UpdParams p) {
 //    640 of  1024:  47.3 |  60.7   43.0   42.5   51.3   68.7
 //   3072 of  4608:   160 |   155    159    170    212    307
 //   5120 of  8192:   259 |   252    262    279    351    511
+// Many short rows: there the machine is full with any number of threads a row, and the fewer there
+// are the less is merged and the longer each one streams; what speaks for more is the tail, in which
+// the last rows run alone (their time is nvec / threads).  So 64 threads from rows = 2 nvec on, a warp
+// from 6 nvec on.  us, 128 / 64 / 32 threads (in front the former two CTAs or 128 threads):
+//   9600 of 12800, V =  2,048:  25.2 |  27.3   20.2   17.8
+//                       8,000:  58.9 |  50.9   40.2   37.4
+//                      24,000:   101 |  91.7   83.0   84.1
+//                      64,000 (6400 live):  141 |   136    137    154
+//   6144 of  8192, V = 16,000:  54.3 |  48.5   43.8   43.6
+//                      32,000:  78.3 |  75.2   75.3   82.6
+//   2304 of  3072, V =  4,096:  11.0 |  10.8    9.4   10.8
 struct RowShape { int threads, ctas; };
 static RowShape row_shape(int rows, int nvec) {
   const int floor_ = rows < 2048 ? 256 : 128;
@@ -311,6 +322,7 @@ static RowShape row_shape(int rows, int nvec) {
   while (w < 4096 && (long long)w * 1448 / 1024 * rows < 180000) w *= 2;   // nearest power of two (in the log)
   w = w < floor_ ? floor_ : w;
   while (w > 128 && 2 * w > nvec) w /= 2;
+  if (rows >= 2048 && 2ll * nvec <= rows) w = rows >= 4096 && 6ll * nvec <= rows ? 32 : 64;
   RowShape s;
   s.threads = w < 512 ? w : 512;
   s.ctas = w / s.threads;
@@ -330,8 +342,11 @@ int launch_t2t(fb_ctx* ctx, const fb_pack* pk, const void* logits, const fb_stat
                                             c.vocab / 8, argmax, conf, status),
                     "t2t_rows_kernel launch");
   };
-  const int e = T == 128 ? launch(t2t_rows_kernel<128>, 128) : T == 256 ? launch(t2t_rows_kernel<256>, 256)
-                                                                        : launch(t2t_rows_kernel<512>, 512);
+  const int e = T == 32    ? launch(t2t_rows_kernel<32>, 32)
+                : T == 64  ? launch(t2t_rows_kernel<64>, 64)
+                : T == 128 ? launch(t2t_rows_kernel<128>, 128)
+                : T == 256 ? launch(t2t_rows_kernel<256>, 256)
+                           : launch(t2t_rows_kernel<512>, 512);
   if (e) return e;
   return launch_t2t_update(ctx, pk, st, argmax, conf, action, slot_stats, stream);
 }

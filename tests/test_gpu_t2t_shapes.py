@@ -17,7 +17,8 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("n_requests,vocab", [
     (1, 8), (1, 1000), (1, 4096), (1, 4104), (1, 16384), (1, 16392), (1, 32768), (1, 65536), (1, 65544), (1, 151552),
-    (3, 8200), (3, 40000), (11, 8200), (11, 20008), (22, 5000), (22, 8200), (70, 1032), (70, 4104)])
+    (3, 8200), (3, 40000), (11, 8200), (11, 20008), (22, 5000), (22, 8200), (70, 1032), (70, 4104),
+    (22, 12008), (70, 11208), (70, 27008)])
 def test_every_row_shape(n_requests, vocab):
     wl = synth.tiny_workload(n_requests=n_requests, wmax=1 if n_requests == 1 else 3, w_lo=1,
                              w_hi=1 if n_requests == 1 else 3, prefix_lo=5, prefix_hi=60, vocab=vocab)
