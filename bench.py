@@ -762,7 +762,7 @@ def run_sweep(args):
         "clocks": clocks,
         "e2e": {"value": None, "unit": "TFLOP/s", "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 0,
                 "note": "the sweep is timed with resident inputs only; see the default run for host buffers"},
-        "gpu_launches": kernels_per_step(ctx) * n_steps,
+        "gpu_launches": kernels_per_step(run.ctx) * n_steps,
         "kernels": {"pack_ms": round(float(seg[:, 0].mean()), 4), "attn_ms": round(attn_ms / n_steps, 4),
                     "t2t_ms": round(t2t_ms / n_steps, 4), "gate_commit_ms": round(float(seg[:, 3].mean()), 4),
                     "attn_tflops": round(attn_tf, 2), "t2t_gbs": round(t2t_gbs, 1)},
