@@ -177,9 +177,11 @@ typedef struct {
                                     minimum.  Default: the split with the least
                                     estimated time for the batch at hand (bf16
                                     pages), two items per SM (8-bit pages)    */
-  int32_t attn_min_chunk_tiles;  /* shortest key range of a split piece, in
-                                    128-key tiles (default 2 where the split is
-                                    estimated, else 4)                        */
+  int32_t attn_min_chunk_tiles;  /* shortest chunk a key range is cut by, in
+                                    128-key tiles: n tiles give at most
+                                    ceil(n / this) pieces of even length
+                                    (default 2 where the split is estimated,
+                                    else 4)                                   */
   int32_t attn_pair;             /* 1: four Q tiles of one request and KV head
                                     at a time run on a pair of CTAs that share
                                     every K/V tile (tcgen05 cta_group::2; bf16

@@ -207,7 +207,7 @@ int fb_attn_plan_host(const fb_ctx* ctx, const int32_t* h_prefix_len, const int3
         const float e = fb::split_estimate(st, ctx->ws.l[0].max_parts);
         if (e >= 0.f && (best < 0.f || e < best)) { best = e; ct = cand > 0 ? cand : 1; }
       }
-      rule = fb::split_auto((int)total, (int)units, ct);
+      rule = fb::split_auto((int)total, (int)units, ct, ctx->min_chunk_tiles);
     }
     long long wbase = 0, items = 0, parts = 0;
     for (int r = 0; r < n; ++r) {

@@ -185,11 +185,12 @@ __host__ __device__ inline float split_estimate(const SplitStat& s, int max_part
 __host__ __device__ inline bool split_worth_estimating(int total, int units, int longest) {
   return units < 4 * kSms || longest > total / (2 * kSms);
 }
-// The chosen candidate's chunk length, or the filler rule where it pays.
-__host__ __device__ inline SplitRule split_auto(int total, int units, int ct) {
+// The chosen candidate's chunk length, or the filler rule where it pays.  `min_chunk`: the context's
+// minimum, as for split_rule; the workspace has room for pieces of that length and no shorter ones.
+__host__ __device__ inline SplitRule split_auto(int total, int units, int ct, int min_chunk) {
   SplitRule s;
   if (units >= kDefaultTargetItems) {
-    s = split_rule(total, units, kDefaultTargetItems, kDefaultMinChunkTiles);
+    s = split_rule(total, units, kDefaultTargetItems, min_chunk);
     const int pieces = total / 100 * kFillerPercent / s.fine_ct;
     if (s.fine_from != 0x7fffffff &&
         total / units * (kTileCost / 4) > pieces * kPieceCost / kSms + pieces * kMergePieceNs / 100 + kMergeCost) return s;

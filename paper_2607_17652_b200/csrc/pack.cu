@@ -171,7 +171,7 @@ __device__ void build_sched(const PackParams& p, const int list) {
   }
   __syncthreads();
   if (list == 0 && p.auto_split && !split_worth_estimating(sh_total, sh_units, sh_longest)) {
-    if (tid == 0) sh_rule = split_auto(sh_total, sh_units, max(sh_longest, 1));
+    if (tid == 0) sh_rule = split_auto(sh_total, sh_units, max(sh_longest, 1), p.min_chunk_tiles);
   } else if (list == 0 && p.auto_split) {
     // every lane a candidate chunk length, the requests dealt to the warps; then the least
     // (estimate, candidate) wins
@@ -196,7 +196,7 @@ __device__ void build_sched(const PackParams& p, const int list) {
         if (b2 < best || (b2 == best && a2 < at)) { best = b2; at = a2; }
       }
       const int chosen = __shfl_sync(0xffffffffu, ct, at);
-      if (lane == 0) sh_rule = split_auto(sh_total, sh_units, chosen);
+      if (lane == 0) sh_rule = split_auto(sh_total, sh_units, chosen, p.min_chunk_tiles);
     }
   } else if (tid == 0) {
     sh_rule = split_rule(sh_total, sh_units, p.target_items[list], p.min_chunk_tiles);

@@ -55,6 +55,38 @@ def test_short_contexts_have_no_pieces():
     assert plan(dict(attn_min_chunk_tiles=1), 10)["max_parts"] > 0
 
 
+def _tiles(P, w):           # key tiles of a request's units (window beside the pages, one Q tile per slot)
+    return -(-P // 128) + -(-(w * 32) // 128)
+
+
+@pytest.mark.parametrize("min_chunk", [1, 3, 8, 62, 64, 128, 300, 1000])
+def test_callers_shortest_range_holds_without_a_target(min_chunk):
+    # batches large enough for filler pieces at the end of the list
+    rg = np.random.default_rng(min_chunk)
+    for pages in (124, 260, 520):
+        ctx = B.Context(tuning=dict(attn_min_chunk_tiles=min_chunk), **_cfg(max_pages_per_req=pages))
+        for _ in range(40):
+            n = int(rg.integers(19, 65))
+            lo = int(rg.integers(0, pages * 64 - 128))
+            P = rg.integers(lo, pages * 64 - 127, size=n)
+            pl = ctx.attn_plan(P, [4] * n)
+            assert pl["parts"] <= pl["max_parts"] and pl["items"] <= pl["max_items"], (pl, P)
+            # 16 units a request, cut into no more than ceil(tiles / shortest) pieces each
+            pieces = sum(16 * -(-_tiles(int(x), 4) // min_chunk) for x in P)
+            assert pl["items"] <= pieces, (pl, P)
+            if min_chunk >= _tiles(int(P.max()), 4):
+                assert pl["parts"] == 0 and pl["items"] == 16 * n, (pl, P)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("min_chunk", [0, 8, 30, 64])
+def test_shortest_range_on_the_device(min_chunk):
+    # 300 units of 34 to 45 key tiles; with 64 no range may be cut and the context has no room for pieces
+    wl = synth.tiny_workload(n_requests=50, wmax=4, w_lo=4, w_hi=4, prefix_lo=4200, prefix_hi=5600, head_dim=64,
+                             n_q_heads=12, n_kv_heads=3)
+    _plan_and_attention(wl, (dict(attn_min_chunk_tiles=min_chunk), dict(attn_target_items=1)), 0)
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("n_requests,prefix,w,resident", [
     (1, (64, 64), (2, 2), 0), (1, (3001, 3001), (1, 1), 1), (2, (9000, 12000), (3, 3), 0), (9, (100, 2500), (1, 4), 1),
@@ -62,13 +94,17 @@ def test_short_contexts_have_no_pieces():
 def test_device_builds_the_announced_list(n_requests, prefix, w, resident):
     wl = synth.tiny_workload(n_requests=n_requests, wmax=4, w_lo=w[0], w_hi=w[1], prefix_lo=prefix[0],
                              prefix_hi=prefix[1], head_dim=128, n_q_heads=12, n_kv_heads=3)
+    _plan_and_attention(wl, (None, dict(attn_target_items=1)), resident)
+
+
+def _plan_and_attention(wl, tunings, resident):
     stc = synth.make_structure(wl)
     tokens = synth.make_tokens(stc)
     q, kw, vw, kp, vp = (t.to(DEV) for t in synth.make_attn_inputs(stc))
     if resident:
         kw = vw = None
     outs = []
-    for tuning in (None, dict(attn_target_items=1)):
+    for tuning in tunings:
         ctx = B.Context(tuning=tuning, **synth.config_dict(stc, window_in_pages=resident))
         st = B.DeviceState.from_numpy(DEV, stc.active, stc.prefix_len, stc.L, stc.R, tokens,
                                       np.zeros((wl.n_requests, wl.wmax), np.uint8), stc.page_table)
