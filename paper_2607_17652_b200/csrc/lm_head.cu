@@ -43,7 +43,7 @@ __device__ __forceinline__ bool lm_warp_wait(uint64_t* bar, uint32_t parity, vol
 }
 
 // 32 more columns of a row: running maximum with its first index, sum of exponentials relative to it
-// (an equal later maximum keeps the first index; all -inf adds nothing).
+// (an equal later maximum keeps the first index; all -inf adds nothing, a NaN makes the sum NaN).
 __device__ __forceinline__ void absorb32(const uint32_t* v, int col, float& mx, float& sum, int& arg) {
   float m4[4];
 #pragma unroll
@@ -60,7 +60,11 @@ __device__ __forceinline__ void absorb32(const uint32_t* v, int col, float& mx, 
     sum *= ex2_approx((mx - cm) * kLmLog2e);                          // 0 * 2^-inf = 0 at the first maximum
     mx = cm; arg = col + first;
   }
-  if (mx == -INFINITY) return;
+  if (mx == -INFINITY) {                // (the maximum passes NaN by)
+#pragma unroll
+    for (int j = 0; j < 32; ++j) sum += __uint_as_float(v[j]) == -INFINITY ? 0.f : __uint_as_float(v[j]);
+    return;
+  }
   const float mb = -mx * kLmLog2e;
   const float2 mb2 = make_float2(mb, mb), l2 = make_float2(kLmLog2e, kLmLog2e);
   float2 s4[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
@@ -229,7 +233,7 @@ __global__ void __launch_bounds__(32 * kLmMergeWarps) lm_head_merge_kernel(const
   int arg = 0x7fffffff;
   auto add = [&](float m, float s, int a) {         // tiles come in ascending order: an equal maximum keeps the first index
     if (m > M) { S = S * (M == -INFINITY ? 0.f : ex2_approx((M - m) * kLmLog2e)) + s; M = m; arg = a; }
-    else S += m == -INFINITY ? 0.f : s * ex2_approx((m - M) * kLmLog2e);
+    else S += m == -INFINITY ? s : s * ex2_approx((m - M) * kLmLog2e);      // (no maximum: s is 0 or NaN)
   };
   if (row < live) {
     constexpr int kDepth = 4;

@@ -869,6 +869,30 @@ def test_lm_head_fused_row_pass(name, hidden):
     assert int((action == O.ACT_M2T).sum()) > 0
 
 
+@pytest.mark.parametrize("first,last,minus_inf", [
+    (0, 1, 0), (0, 32, 0), (256, 288, 0), (0, 256, 0), (256, 512, 0), (0, 1000, 0), (992, 1000, 0), (31, 32, 31)])
+def test_lm_head_reports_nan_wherever_it_stands(first, last, minus_inf):
+    """Head weights with NaN rows: single ones, whole 32-column chunks and whole 256-column tiles of the
+    vocabulary, or one NaN behind columns of -inf.  Every live row reports it and reveals nothing."""
+    case = make_case(WORKLOADS["tiny_v1000"], with_attn=False, with_logits=False)
+    stc = case["stc"]
+    wl = stc.wl
+    x, w, tokens = synth.make_lm_head_inputs(stc, case["tokens"], 64)
+    x = x.abs() + 0.5                       # (a weight of -inf gives a logit of -inf)
+    case["tokens"] = tokens
+    w[:minus_inf] = -float("inf")
+    w[first:last] = float("nan")
+    ctx, st, pk, sb = gpu_objects(case)
+    ws = torch.zeros(B.lib().fb_lm_head_workspace_bytes(ctx.handle), dtype=torch.uint8, device=DEV)
+    B.fb_pack_wavefronts(ctx, st, pk, sb.ws, sb.status)
+    B.fb_lm_head_t2t(ctx, pk, x.to(DEV), w.to(DEV), st, sb.argmax, sb.conf, sb.action, sb.slot_stats, ws,
+                     sb.status)
+    torch.cuda.synchronize()
+    assert int(sb.status.item()) & B.FB_ST_NAN_LOGIT
+    assert float(sb.conf.abs().max()) == 0.0 and int(sb.action.max()) == 0
+    np.testing.assert_array_equal(st.tokens.cpu().numpy(), tokens)
+
+
 def test_step_host_with_the_window_in_pages():
     """fb_step_host in a window_in_pages context: scatter, attention over the
     pages, T2T, pointer-bump commit -- against the same calls made one by one."""
