@@ -35,6 +35,10 @@ __device__ __forceinline__ float fast_ex2(float x) {
   return y;
 }
 
+// What a logit adds to the sum of a thread that has no maximum yet: nothing if it is -inf, but a NaN
+// (the maximum passes it by) makes the sum NaN for good.
+__device__ __forceinline__ float no_max_term(float z) { return z == -INFINITY ? 0.f : z; }
+
 struct RowAcc {
   float m;    // running max
   float s;    // sum of exp(z - m)
@@ -57,16 +61,21 @@ __device__ __forceinline__ void absorb8(RowAcc& a, const uint4 v, int base) {
                 bf16_lo(v.z), bf16_hi(v.z), bf16_lo(v.w), bf16_hi(v.w)};
   float cm = fmaxf(fmaxf(fmaxf(z[0], z[1]), fmaxf(z[2], z[3])), fmaxf(fmaxf(z[4], z[5]), fmaxf(z[6], z[7])));
   if (cm > a.m) {                       // rare after the first few chunks
-    a.s *= a.m == -INFINITY ? 0.f : fast_ex2((a.m - cm) * kLog2e);
+    a.s *= a.m == -INFINITY ? 0.f : fast_ex2((a.m - cm) * kLog2e);   // (0 * NaN stays NaN)
     a.m = cm;
     int k = 7;
 #pragma unroll
     for (int i = 6; i >= 0; --i) k = z[i] == cm ? i : k;
     a.idx = base + k;
   }
-  if (a.m == -INFINITY) return;          // nothing but -inf so far: contributes 0
-  const float mb = a.m * kLog2e;
   float acc = 0.f;
+  if (a.m == -INFINITY) {                // no maximum so far
+#pragma unroll
+    for (int i = 0; i < 8; ++i) acc += no_max_term(z[i]);
+    a.s += acc;
+    return;
+  }
+  const float mb = a.m * kLog2e;
 #pragma unroll
   for (int i = 0; i < 8; ++i) acc += fast_ex2(fmaf(z[i], kLog2e, -mb));
   a.s += acc;
@@ -96,7 +105,11 @@ __device__ __forceinline__ void absorb16(RowAcc& a, float2& s2, const uint4 v, c
       if (bf16_lo(q[i]) == cm) a.idx = at;
     }
   }
-  if (a.m == -INFINITY) return;          // nothing but -inf so far: contributes 0
+  if (a.m == -INFINITY) {                // no maximum so far
+#pragma unroll
+    for (int i = 0; i < 8; ++i) s2.x += no_max_term(bf16_lo(q[i])) + no_max_term(bf16_hi(q[i]));
+    return;
+  }
   const float mb = -a.m * kLog2e;
   const float2 mb2 = make_float2(mb, mb), l2 = make_float2(kLog2e, kLog2e);
   float2 t = make_float2(0.f, 0.f);      // a sum of its own first: short chains of roundings

@@ -39,3 +39,41 @@ def test_every_row_shape(n_requests, vocab):
     xhat, conf = O.t2t_rows(H.oracle_cfg(stc), opk, H.f64(z))
     np.testing.assert_array_equal(sb.argmax.cpu().numpy(), xhat)
     assert float(np.abs(sb.conf.cpu().numpy() - conf).max()) <= P.CONF_TOL
+
+
+@pytest.mark.parametrize("n_requests,vocab", [(1, 8), (1, 1000), (1, 16384), (1, 65544), (11, 20008), (70, 4104), (70, 1032)])
+def test_nan_is_reported_wherever_it_stands(n_requests, vocab):
+    """Rows with a NaN that no finite logit of its thread precedes: whole pieces, the head of the row, all of it
+    but one logit, or behind -inf.  Each reports and reveals nothing; the rows between them are as without."""
+    wl = synth.tiny_workload(n_requests=n_requests, wmax=1 if n_requests == 1 else 3, w_lo=1,
+                             w_hi=1 if n_requests == 1 else 3, prefix_lo=5, prefix_hi=60, vocab=vocab)
+    case = P.make_case(wl, logits_kind="normal2", with_attn=False)
+    stc, z = case["stc"], case["logits"]
+    opk = O.pack_wavefronts(H.oracle_cfg(stc), H.oracle_state(stc, case["tokens"]))
+    live = opk.n_live * wl.block_len
+    _, conf = O.t2t_rows(H.oracle_cfg(stc), opk, H.f64(z))
+    nan, bad = float("nan"), list(range(0, live, 5))
+    for k, r in enumerate(bad):
+        if k % 5 == 0:
+            z[r, :8] = nan
+        elif k % 5 == 1:
+            z[r, :min(vocab, 4096)] = nan
+        elif k % 5 == 2:
+            z[r, :vocab - 1] = nan
+        elif k % 5 == 3:
+            z[r, :min(vocab, 4096) - 1], z[r, min(vocab, 4096) - 1] = -float("inf"), nan
+        else:
+            z[r, vocab // 2:] = nan
+    for rows in (bad, bad[:1], bad[1:2], bad[2:3], bad[3:4], bad[4:5]):       # together, then each kind by itself
+        zz = z.clone()
+        drop = [r for r in bad if r not in rows]
+        zz[drop] = 0.0
+        ctx, st, pk, sb = P.gpu_objects(case)
+        B.fb_pack_wavefronts(ctx, st, pk, sb.ws, sb.status)
+        B.fb_t2t_step(ctx, pk, zz.to(P.DEV), st, sb.argmax, sb.conf, sb.action, sb.slot_stats, sb.status)
+        torch.cuda.synchronize()
+        assert int(sb.status.item()) == B.FB_ST_NAN_LOGIT
+        got = sb.conf.cpu().numpy()
+        assert (got[rows] == 0.0).all() and int(sb.action[rows].max()) == 0
+        keep = [r for r in range(live) if r not in bad]
+        assert float(np.abs(got[keep] - conf[keep]).max()) <= P.CONF_TOL
