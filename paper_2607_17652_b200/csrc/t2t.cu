@@ -75,9 +75,8 @@ __device__ __forceinline__ void absorb8(RowAcc& a, const uint4 v, int base) {
     a.s += acc;
     return;
   }
-  const float mb = a.m * kLog2e;
 #pragma unroll
-  for (int i = 0; i < 8; ++i) acc += fast_ex2(fmaf(z[i], kLog2e, -mb));
+  for (int i = 0; i < 8; ++i) acc += fast_ex2((z[i] - a.m) * kLog2e);
   a.s += acc;
 }
 
@@ -89,6 +88,9 @@ __device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b) {
 
 // Two 16-byte pieces at once (`base` < `base2`: their first vocabulary indices): the maximum of the
 // 16 logits on the packed values, the exponentials with packed fp32 arithmetic into two sums.
+// The difference to the maximum comes first, then the scaling: the maximum's own term is exactly 1 and
+// the sum never below it.  One fused multiply-add z log2(e) - m log2(e) leaves the rounding error of
+// the product m log2(e) in the exponent of every term (1e-6 at m = 28).
 __device__ __forceinline__ void absorb16(RowAcc& a, float2& s2, const uint4 v, const uint4 w, int base, int base2) {
   const uint32_t q[8] = {v.x, v.y, v.z, v.w, w.x, w.y, w.z, w.w};
   const uint32_t mm = max_bf16x2(max_bf16x2(max_bf16x2(q[0], q[1]), max_bf16x2(q[2], q[3])),
@@ -110,12 +112,11 @@ __device__ __forceinline__ void absorb16(RowAcc& a, float2& s2, const uint4 v, c
     for (int i = 0; i < 8; ++i) s2.x += no_max_term(bf16_lo(q[i])) + no_max_term(bf16_hi(q[i]));
     return;
   }
-  const float mb = -a.m * kLog2e;
-  const float2 mb2 = make_float2(mb, mb), l2 = make_float2(kLog2e, kLog2e);
+  const float2 nm2 = make_float2(-a.m, -a.m), l2 = make_float2(kLog2e, kLog2e);
   float2 t = make_float2(0.f, 0.f);      // a sum of its own first: short chains of roundings
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
-    const float2 x = __ffma2_rn(make_float2(bf16_lo(q[i]), bf16_hi(q[i])), l2, mb2);
+    const float2 x = __fmul2_rn(__fadd2_rn(make_float2(bf16_lo(q[i]), bf16_hi(q[i])), nm2), l2);
     t = __fadd2_rn(t, make_float2(fast_ex2(x.x), fast_ex2(x.y)));
   }
   s2 = __fadd2_rn(s2, t);
@@ -213,7 +214,7 @@ t2t_rows_kernel(const uint4* __restrict__ logits, const int32_t* __restrict__ n_
     if (rank != 0) return;
   }
   if (tid == 0) {
-    const float pr = 1.0f / b.s;         // the max itself contributes exp(0) = 1
+    const float pr = 1.0f / b.s;         // the max itself contributes exp(0) = 1 exactly: b.s >= 1
     if (!(b.s >= 1.0f) || !(pr == pr) || b.s > FLT_MAX) {
       atomicOr(status, FB_ST_NAN_LOGIT);
       argmax[row] = b.idx == 0x7fffffff ? 0 : b.idx;

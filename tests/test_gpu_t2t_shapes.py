@@ -77,3 +77,31 @@ def test_nan_is_reported_wherever_it_stands(n_requests, vocab):
         assert (got[rows] == 0.0).all() and int(sb.action[rows].max()) == 0
         keep = [r for r in range(live) if r not in bad]
         assert float(np.abs(got[keep] - conf[keep]).max()) <= P.CONF_TOL
+
+
+@pytest.mark.parametrize("n_requests,vocab", [(1, 8), (1, 1000), (1, 65544), (11, 20008), (70, 1032), (70, 4104)])
+def test_certain_rows(n_requests, vocab):
+    """One logit far above the rest, up to where nothing else shows in 32 bits: never reported as NaN, revealed,
+    and its confidence that of the oracle to 2e-6 (a chain of at most 32 additions behind the term 1, 2^-24 each;
+    the tail's 1.4e-4 have relative errors of 1e-6)."""
+    wl = synth.tiny_workload(n_requests=n_requests, wmax=1 if n_requests == 1 else 3, w_lo=1,
+                             w_hi=1 if n_requests == 1 else 3, prefix_lo=5, prefix_hi=60, vocab=vocab)
+    case = P.make_case(wl, logits_kind="normal2", with_attn=False)
+    stc, z = case["stc"], case["logits"]
+    opk = O.pack_wavefronts(H.oracle_cfg(stc), H.oracle_state(stc, case["tokens"]))
+    live = opk.n_live * wl.block_len
+    rg = np.random.default_rng(vocab)
+    z[:] = -10.0
+    for r in range(live):
+        z[r, int(rg.integers(0, vocab))] = (10.0, 16.5, 20.0, 28.0, 33.0, 40.0, 61.0, 1000.0)[r % 8]
+    ctx, st, pk, sb = P.gpu_objects(case)
+    B.fb_pack_wavefronts(ctx, st, pk, sb.ws, sb.status)
+    B.fb_t2t_step(ctx, pk, z.to(P.DEV), st, sb.argmax, sb.conf, sb.action, sb.slot_stats, sb.status)
+    torch.cuda.synchronize()
+    assert int(sb.status.item()) == 0
+    xhat, conf = O.t2t_rows(H.oracle_cfg(stc), opk, H.f64(z))
+    np.testing.assert_array_equal(sb.argmax.cpu().numpy(), xhat)
+    got = sb.conf.cpu().numpy()
+    assert float(np.abs(got - conf).max()) <= 2e-6 and float(got.max()) <= 1.0
+    masked = opk.qtok[:live] == stc.mask_id
+    assert (sb.action.cpu().numpy()[:live][masked] == O.ACT_M2T).all() and masked.any()
