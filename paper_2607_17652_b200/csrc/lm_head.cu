@@ -65,12 +65,12 @@ __device__ __forceinline__ void absorb32(const uint32_t* v, int col, float& mx, 
     for (int j = 0; j < 32; ++j) sum += __uint_as_float(v[j]) == -INFINITY ? 0.f : __uint_as_float(v[j]);
     return;
   }
-  const float mb = -mx * kLmLog2e;
-  const float2 mb2 = make_float2(mb, mb), l2 = make_float2(kLmLog2e, kLmLog2e);
+  // difference first, then the scaling: the maximum's own term is exactly 1 (see absorb16 in t2t.cu)
+  const float2 nm2 = make_float2(-mx, -mx), l2 = make_float2(kLmLog2e, kLmLog2e);
   float2 s4[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
 #pragma unroll
   for (int j = 0; j < 32; j += 2) {
-    const float2 x = __ffma2_rn(make_float2(__uint_as_float(v[j]), __uint_as_float(v[j + 1])), l2, mb2);
+    const float2 x = __fmul2_rn(__fadd2_rn(make_float2(__uint_as_float(v[j]), __uint_as_float(v[j + 1])), nm2), l2);
     s4[(j >> 1) & 3] = __fadd2_rn(s4[(j >> 1) & 3], make_float2(ex2_approx(x.x), ex2_approx(x.y)));
   }
   const float2 t = __fadd2_rn(__fadd2_rn(s4[0], s4[1]), __fadd2_rn(s4[2], s4[3]));

@@ -893,6 +893,37 @@ def test_lm_head_reports_nan_wherever_it_stands(first, last, minus_inf):
     np.testing.assert_array_equal(st.tokens.cpu().numpy(), tokens)
 
 
+@pytest.mark.parametrize("name", ["tiny", "tiny_v1000"])
+def test_lm_head_certain_rows(name):
+    """One token's logit far above the rest, up to where nothing else shows in 32 bits: never reported as NaN,
+    revealed, confidence that of the oracle to 2e-6 (a chain of at most 32 additions of 2^-24 behind the term 1)."""
+    case = make_case(WORKLOADS[name], with_attn=False, with_logits=False)
+    stc = case["stc"]
+    wl = stc.wl
+    rg = np.random.default_rng(5)
+    rows, top = wl.n_requests * wl.wmax * wl.block_len, int(rg.integers(0, wl.vocab))
+    x, w = torch.zeros(rows, 64, dtype=torch.bfloat16), torch.zeros(wl.vocab, 64, dtype=torch.bfloat16)
+    x[:, 0] = 1.0                                  # (products and sums of two exact terms)
+    x[:, 1] = torch.tensor([20.0, 26.5, 30.0, 38.0, 43.0, 50.0, 71.0, 1000.0]).repeat(rows // 8)
+    w[:, 0] = -10.0
+    w[top, 1] = 1.0
+    ctx, st, pk, sb = gpu_objects(case)
+    ws = torch.zeros(B.lib().fb_lm_head_workspace_bytes(ctx.handle), dtype=torch.uint8, device=DEV)
+    B.fb_pack_wavefronts(ctx, st, pk, sb.ws, sb.status)
+    B.fb_lm_head_t2t(ctx, pk, x.to(DEV), w.to(DEV), st, sb.argmax, sb.conf, sb.action, sb.slot_stats, ws,
+                     sb.status)
+    torch.cuda.synchronize()
+    assert int(sb.status.item()) == 0
+    ocfg = H.oracle_cfg(stc)
+    opk = O.pack_wavefronts(ocfg, H.oracle_state(stc, case["tokens"]))
+    xhat, conf = O.lm_head_rows(ocfg, opk, H.f64(x), H.f64(w))
+    np.testing.assert_array_equal(sb.argmax.cpu().numpy(), xhat)
+    got, live = sb.conf.cpu().numpy(), opk.n_live * wl.block_len
+    assert float(np.abs(got - conf).max()) <= 2e-6 and float(got.max()) <= 1.0
+    masked = opk.qtok[:live] == stc.mask_id
+    assert (sb.action.cpu().numpy()[:live][masked] == O.ACT_M2T).all() and masked.any()
+
+
 def test_step_host_with_the_window_in_pages():
     """fb_step_host in a window_in_pages context: scatter, attention over the
     pages, T2T, pointer-bump commit -- against the same calls made one by one."""
