@@ -171,13 +171,21 @@ __host__ __device__ inline void split_stat_add(SplitStat& s, const ReqGeom& g, i
   const int item = len * (duals > 0 ? kTileDualCost : kTileCost) + fixed;
   s.longest = item > s.longest ? item : s.longest;
 }
-// As a float whose operations round alike on the host and on the device (no product that
-// feeds a sum is inexact).  Negative: not allowed (more pieces than the workspace holds).
+// a product that no compiler fuses with the sum it feeds
+__host__ __device__ inline float rounded_product(float a, float b) {
+#ifdef __CUDA_ARCH__
+  return __fmul_rn(a, b);
+#else
+  return a * b;
+#endif
+}
+// As a float whose operations round alike on the host and on the device.  Negative: not allowed (more
+// pieces than the workspace holds).
 __host__ __device__ inline float split_estimate(const SplitStat& s, int max_parts) {
   if (s.parts > max_parts || s.items <= 0) return -1.f;
   const float work = (float)s.work, even = work / (float)kSms;
   const int waves = (s.items + kSms - 1) / kSms;
-  const float over = work / (float)s.items * (float)waves;
+  const float over = rounded_product(work / (float)s.items, (float)waves);
   float e = waves >= 3 ? 0.5f * (even + over) : (over > even ? over : even);
   e = e < (float)s.longest ? (float)s.longest : e;
   return s.parts ? e + (float)(kMergeCost + kMergePieceNs * s.parts / 100) : e;

@@ -79,6 +79,29 @@ def test_callers_shortest_range_holds_without_a_target(min_chunk):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("seed", [36154492, 54453613, 40045238, 42664750, 51996146, 31555111, 63399331])
+def test_near_ties_of_the_estimate(seed):
+    # batches in which the two best chunk lengths are estimated within a unit in the last place of each other:
+    # device and host have to round alike to agree on one
+    def draw():
+        nonlocal seed
+        seed = (seed * 1664525 + 1013904223) & 0xFFFFFFFF
+        return seed >> 8
+    n, hi = 60 + draw() % 40, 3000 + draw() % 6000
+    P, w = zip(*[(draw() % hi, 1 + draw() % 4) for _ in range(n)])
+    ctx = B.Context(**_cfg(max_requests=n, n_q_heads=12, n_kv_heads=3, max_pages_per_req=150))
+    st = B.DeviceState.from_numpy(DEV, np.ones(n, np.int32), np.array(P, np.int32), np.zeros(n, np.int32),
+                                  np.array(w, np.int32), np.zeros((n, 32 * 32), np.int32), np.zeros((n, 4), np.uint8),
+                                  np.zeros((n, 150), np.int32))
+    pk, sb = B.PackBuffers.alloc(ctx, DEV), B.StepBuffers(ctx, DEV)
+    B.fb_pack_wavefronts(ctx, st, pk, sb.ws, sb.status)
+    torch.cuda.synchronize()
+    assert int(sb.status.item()) == 0
+    hdr, plan = sb.ws[:64].cpu().numpy().view(np.int32), ctx.attn_plan(P, w)
+    assert (int(hdr[1]), int(hdr[0]), int(hdr[3])) == (plan["units"], plan["items"], plan["parts"])
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("min_chunk", [0, 8, 30, 64])
 def test_shortest_range_on_the_device(min_chunk):
     # 300 units of 34 to 45 key tiles; with 64 no range may be cut and the context has no room for pieces
