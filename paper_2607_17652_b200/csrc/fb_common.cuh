@@ -152,11 +152,20 @@ __host__ __device__ inline SplitRule split_rule(int total, int units, int target
 __host__ __device__ inline bool estimates_split(const fb_config& c) { return !c.kv_fp8; }
 constexpr int kTileCost = 16, kTileDualCost = 22, kItemCost = 40, kPieceCost = 45, kMergeCost = 50, kMergePieceNs = 26;
 constexpr int kSplitCandidates = 32;
-// Candidate i: the longest range (`longest` key tiles) divided by 1, 1.25, 1.5, 1.75, 2, 2.25, 2.5,
-// 2.75, 3, 3.5, 4, 4.5, 5, 5.5, 6, 6.5, 7, 8, 9, 10, 11, 12, 14, 16, 18, 20, 24, 28, 32, 36, 40, 48
-// (quarters, a byte each).
+// Candidate i: the longest range (`longest` key tiles) divided by the i-th of the divisors below, which are in quarters
+// (1, 1.25, ... 48) and packed eight to a word, a byte each.
+constexpr unsigned long long eight_bytes(int a, int b, int c, int d, int e, int f, int g, int h) {
+  const int v[8] = {a, b, c, d, e, f, g, h};
+  unsigned long long w = 0;
+  for (int i = 0; i < 8; ++i) w |= (unsigned long long)v[i] << (8 * i);
+  return w;
+}
 __host__ __device__ inline int split_candidate(int i, int longest) {
-  const unsigned long long w = i < 8 ? 795458214266537220ull : i < 16 ? 1880277119885381132ull : i < 24 ? 4627501583333335068ull : 13880252932871442504ull;
+  constexpr unsigned long long w0 = eight_bytes(4, 5, 6, 7, 8, 9, 10, 11);
+  constexpr unsigned long long w1 = eight_bytes(12, 14, 16, 18, 20, 22, 24, 26);
+  constexpr unsigned long long w2 = eight_bytes(28, 32, 36, 40, 44, 48, 56, 64);
+  constexpr unsigned long long w3 = eight_bytes(72, 80, 96, 112, 128, 144, 160, 192);
+  const unsigned long long w = i < 8 ? w0 : i < 16 ? w1 : i < 24 ? w2 : w3;
   const unsigned q = (unsigned)(w >> (8 * (i & 7))) & 0xffu;
   return (int)((4u * (unsigned)longest + q - 1u) / q);
 }
