@@ -133,7 +133,11 @@ def lib() -> C.CDLL:
             if n not in ("fb_last_error", "fb_workspace_bytes",
                          "fb_lm_head_workspace_bytes"):
                 getattr(l, n).restype = I
-        from . import _marshal
+        try:
+            from . import _marshal
+        except ImportError as e:
+            raise RuntimeError("the marshalling module has not been built for this Python; run "
+                               "`python -m paper_2607_17652_b200.build`") from e
         _marshal.bind(*(C.cast(getattr(l, n), P).value for n in _FAST))
         _lib, _m = l, _marshal
     return _lib

@@ -16,7 +16,8 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 ROOT = os.path.dirname(HERE)
 LIB = os.path.join(HERE, "libflowblock.so")
-MARSHAL = os.path.join(HERE, "_marshal.so")
+# named for the Python it is built against: another one does not load it
+MARSHAL = os.path.join(HERE, "_marshal" + sysconfig.get_config_var("EXT_SUFFIX"))
 SOURCES = ["api.cu", "pack.cu", "t2t.cu", "gate_commit.cu", "attn_sm100.cu", "scatter.cu", "lm_head.cu",
            "attn_static.cu", "attn_pair_sm100.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo",
@@ -61,6 +62,9 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if jobs or not os.path.exists(LIB) or force:
         run([_nvcc(), "-shared", "-o", LIB, *objs, "-gencode",
              "arch=compute_100a,code=sm_100a"])
+    untagged = os.path.join(HERE, "_marshal.so")        # what earlier builds left, which any Python would load
+    if os.path.exists(untagged):
+        os.remove(untagged)
     src = os.path.join(CSRC, "marshal.c")
     if force or not os.path.exists(MARSHAL) or \
             os.path.getmtime(MARSHAL) < max(os.path.getmtime(src), hdr_time):

@@ -36,6 +36,14 @@ def test_header_symbols_are_exported():
         assert getattr(lib, name).argtypes is not None, name
 
 
+def test_marshalling_module_is_named_for_this_python():
+    import sysconfig
+    B.lib()
+    here = os.path.dirname(B.LIB_PATH)
+    assert os.path.basename(B._m.__file__) == "_marshal" + sysconfig.get_config_var("EXT_SUFFIX")
+    assert not os.path.exists(os.path.join(here, "_marshal.so"))       # (any Python would load that one)
+
+
 def test_struct_layouts_match_header_order():
     hdr = open(os.path.join(ROOT, "include", "flowblock.h")).read()
     for cls in (B.fb_config, B.fb_tuning, B.fb_state, B.fb_pack, B.fb_host_io, B.fb_device_bufs):
