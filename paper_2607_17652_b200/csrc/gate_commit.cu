@@ -39,40 +39,43 @@ struct GateParams {
   int32_t clustered;       // the whole grid is one cluster
 };
 
-// What a request's own block counts say (Alg. 1 l.7-9 before any batch rule): its window,
-// the post-edit counters after this forward, the finished prefix c (stopping after a block
-// that holds EOS), and whether retiring those c blocks ends the request.
+// Post-edit forwards of a block after this one, which it went into with m0 masks.
+__device__ __forceinline__ int post_edits(int before, int m0) { return min(before + (m0 == 0 ? 1 : 0), 255); }
+// Locally finished (Sec. 2.1): no masks left (m1), and either a quiet post-edit forward or the S_pe
+// budget is used up.
+__device__ __forceinline__ bool finished(const GateParams& p, int m0, int m1, int n_updates, int pe) {
+  return m1 == 0 && ((m0 == 0 && n_updates == 0) || pe >= p.s_pe);
+}
+
+// blocks of the finished prefix, before EOS is looked at (a window has at most 8: there is a zero bit)
+__device__ __forceinline__ int leading_blocks(unsigned fin) { return __ffs(~fin) - 1; }
+
+// What a request's own block counts say to the batch reduction (Alg. 1 l.7-9 before any batch rule):
+// its window, the finished prefix c (stopping after a block that holds EOS), and whether retiring
+// those c blocks ends the request.
 struct ReqEval {
   int first, w, L, R, c;
-  bool ok, eos, ends;
-  uint8_t pe_new[8];
-  int m2t, t2t;
+  bool ok, ends;
 };
 __device__ __forceinline__ ReqEval eval_request(const GateParams& p, int r) {
   ReqEval e;
   e.first = p.req_slot_begin[r];
   e.w = p.req_slot_begin[r + 1] - e.first;
   e.L = p.L[r]; e.R = p.R[r];
-  e.c = 0; e.eos = false; e.ends = false; e.m2t = 0; e.t2t = 0;
+  e.c = 0; e.ends = false;
   e.ok = !(e.w != e.R - e.L || e.w < 0 || e.w > p.wmax);
   if (!e.ok) return e;
-  bool fin[8];
+  unsigned fin = 0, eos = 0;                         // bit s: window block s
   for (int s = 0; s < e.w; ++s) {
     const int32_t* st = p.slot_stats + (e.first + s) * FB_SLOT_STATS;
-    const int m0 = st[FB_STAT_M0], m1 = st[FB_STAT_M1], nupd = st[FB_STAT_M2T] + st[FB_STAT_T2T];
-    int pn = p.pe_done[r * p.wmax + s] + (m0 == 0 ? 1 : 0);
-    pn = pn > 255 ? 255 : pn;
-    e.pe_new[s] = (uint8_t)pn;
-    // locally finished (Sec. 2.1): no masks left, and either a quiet
-    // post-edit forward or the S_pe budget is used up
-    fin[s] = m1 == 0 && ((m0 == 0 && nupd == 0) || pn >= p.s_pe);
-    e.m2t += st[FB_STAT_M2T]; e.t2t += st[FB_STAT_T2T];
+    const int m0 = st[FB_STAT_M0], pe = post_edits(p.pe_done[r * p.wmax + s], m0);
+    fin |= (unsigned)finished(p, m0, st[FB_STAT_M1], st[FB_STAT_M2T] + st[FB_STAT_T2T], pe) << s;
+    eos |= (unsigned)(st[FB_STAT_EOS] != 0) << s;
   }
-  while (e.c < e.w && fin[e.c]) {                    // Alg. 1 l.7-9, in order
-    ++e.c;
-    if (p.slot_stats[(e.first + e.c - 1) * FB_SLOT_STATS + FB_STAT_EOS]) { e.eos = true; break; }
-  }
-  e.ends = e.eos || e.L + e.c == p.max_blocks;
+  const int lead = leading_blocks(fin);
+  const unsigned ending = eos & ((1u << lead) - 1u);
+  e.c = ending ? __ffs(ending) : lead;
+  e.ends = ending || e.L + e.c == p.max_blocks;
   return e;
 }
 // Eq. 2 on the frontier block as it went into this forward (m0 masks, rdy of them ready; an
@@ -145,12 +148,11 @@ __global__ void __launch_bounds__(kGateThreads) gate_commit_kernel(const GatePar
         m0 = st[FB_STAT_M0]; rdy = st[FB_STAT_RDY]; m2t = st[FB_STAT_M2T]; t2t = st[FB_STAT_T2T]; m1 = st[FB_STAT_M1];
         eos = st[FB_STAT_EOS] != 0;
         nupd = m2t + t2t;
-        pn = min(p.pe_done[r * p.wmax + tid] + (m0 == 0 ? 1 : 0), 255);
+        pn = post_edits(p.pe_done[r * p.wmax + tid], m0);
       }
-      // locally finished (Sec. 2.1): no masks left, and either a quiet post-edit forward or the
-      // S_pe budget is used up; Alg. 1 l.7-9: the finished prefix, stopping after a block with EOS
-      const bool fin = tid < w && m1 == 0 && ((m0 == 0 && nupd == 0) || pn >= p.s_pe);
-      const int lead = __ffs(~__ballot_sync(0xffffffffu, fin)) - 1;              // w <= 8: there is a zero
+      // Alg. 1 l.7-9: the finished prefix, stopping after a block with EOS
+      const bool fin = tid < w && finished(p, m0, m1, nupd, pn);
+      const int lead = leading_blocks(__ballot_sync(0xffffffffu, fin));
       const unsigned ends = __ballot_sync(0xffffffffu, eos && tid < lead);
       const int own = ends ? __ffs(ends) : lead;
       // batch_sync: the batch's retire count caps the sequence's own; a block holding EOS
