@@ -756,11 +756,12 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
 // time; it returns at once when no unit was split.
 // Bound by the partials' way through the L2 (12 to 19 MB written on one SM and read on another) and
 // by the latency of a round of such loads, 2 to 3 us, so W grows with the longest split of the
-// batch, up to the point where the CTAs no longer run together: attention call in us with W = 1 / 2 / 4:
-// one request of 3,000 tokens (6 pieces a unit) 20.9 / 19.3 / 20.1, 28,000 tokens (12 pieces) 84 / 76 /
-// 65, 8 requests (3 pieces, 40 units) 23.6 / 26.9 / 29; with a warp per row over a row-major layout
-// these took 23.1, 97 and 26.4.  Of the present calls (18.3, 55, 23.1) the merge is 6, 10 and 6 us, an
-// empty one 2.
+// batch, up to the point where the CTAs no longer run together.  Attention call in us with W = 1 / 2 / 4,
+// taken when ranges were cut for two items an SM: one request of 3,000 tokens (then 6 pieces a unit)
+// 20.9 / 19.3 / 20.1, 28,000 tokens (12 pieces) 84 / 76 / 65, 8 requests (3 pieces, 40 units) 23.6 /
+// 26.9 / 29; with a warp per row over a row-major layout these took 23.1, 97 and 26.4.  Of the calls with
+// the split chosen by estimate (18.3, 55, 23.1; the first in 12 pieces a unit, W = 4) the merge is 6, 10
+// and 6 us, an empty one 2.
 constexpr int kCombineThreads = 256, kCombineCtasPerSm = 8, kCombineDepth = 4, kCombineMostCtas = 1024, kCombineMaxWays = 4;
 template <int D>
 __global__ void __launch_bounds__(kCombineThreads, 3) attn_combine_kernel(const AttnParams p) {

@@ -136,11 +136,14 @@ __host__ __device__ inline SplitRule split_rule(int total, int units, int target
 // 32 lengths from the longest key range down to 1/48 of it, the one with the least
 //   makespan = max(W / SMs, longest item, waves * W / items) + merge,
 // W the work of all items.  A batch of equal items that just misses whole waves pays for the last
-// one in full; from three waves on handing out longest first fills half of that in.  The costs
-// are measured (in units of 100 ns; the merge per piece in ns): a key tile of a pair, of two K/V
-// streams; what an item costs beside its tiles, whole or as a piece; the merge.  Against always aiming at two items
-// an SM: 28,000-token request 72 -> 64 us, 24 requests of 700 to 5,000 tokens 161 -> 151 (not split
-// at all), 8 requests 24.6 (the same split).
+// one in full; from three waves on handing out longest first fills half of that in.  The costs (in
+// units of 100 ns; the merge per piece in ns) are a key tile of a pair, of two K/V streams; what an
+// item costs beside its tiles, whole or as a piece; the merge.  They were measured at head_dim 128 when
+// the estimate was written, before the key loop, the epilogue and the start of an item got shorter, and
+// head_dim 64, whose tiles and partials are half the size, uses the same: they rank the candidates, they do
+// not predict a time.  Against always aiming at two items an SM, with the kernel of then: 28,000-token
+// request 72 -> 64 us, 24 requests of 700 to 5,000 tokens 161 -> 151 (not split at all), 8 requests 24.6
+// (the same split).
 // With four whole items an SM and more, none longer than half of an SM's share, the estimate is skipped
 // (longest items first leave nothing to gain that a split would not cost): the pack kernel takes
 // 2 to 3 us less on 64 and 128 requests.
