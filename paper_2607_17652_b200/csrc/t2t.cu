@@ -90,7 +90,9 @@ __device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b) {
 // 16 logits on the packed values, the exponentials with packed fp32 arithmetic into two sums.
 // The difference to the maximum comes first, then the scaling: the maximum's own term is exactly 1 and
 // the sum never below it.  One fused multiply-add z log2(e) - m log2(e) leaves the rounding error of
-// the product m log2(e) in the exponent of every term (1e-6 at m = 28).
+// the product m log2(e) in the exponent of every term (1e-6 at m = 28).  The separate multiply shows in
+// neither large nor small passes (call in us, without / with: 5120 rows 255.0 / 255.1, 640 rows 56.3 /
+// 56.3, 64 rows 17.4 / 17.4, events around it and a cold L2) and costs whole steps 0.1 to 0.7 %.
 __device__ __forceinline__ void absorb16(RowAcc& a, float2& s2, const uint4 v, const uint4 w, int base, int base2) {
   const uint32_t q[8] = {v.x, v.y, v.z, v.w, w.x, w.y, w.z, w.w};
   const uint32_t mm = max_bf16x2(max_bf16x2(max_bf16x2(q[0], q[1]), max_bf16x2(q[2], q[3])),
