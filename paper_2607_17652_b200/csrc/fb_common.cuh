@@ -309,6 +309,13 @@ __device__ __forceinline__ void pdl_wait() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
+// The same the other way round: the next kernel of the stream starts when everything before this one is
+// complete, so what is older than this kernel it may read (past the L1, __ldcg) ahead of its own wait.
+// Only between two kernels of one call: between calls the caller's stream may hold anything.
+__device__ __forceinline__ void pdl_wait_then_release() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
 // The wait alone: the next kernel is scheduled when this one is complete.  For a kernel that takes
 // nearly all shared memory of its SM: CTAs that move in beside its last ones inherit its division
 // between shared memory and L1, which only changes on an idle SM, and kernels that live on loads in

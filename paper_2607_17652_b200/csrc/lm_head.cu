@@ -220,7 +220,7 @@ lm_head_stats_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
 constexpr int kLmMergeWarps = 32;
 __global__ void __launch_bounds__(32 * kLmMergeWarps) lm_head_merge_kernel(const LmParams p, int32_t* argmax, float* conf,
                                                                           int max_rows) {
-  pdl_wait();
+  pdl_wait_then_release();          // (the update is next)
   __shared__ float s_m[kLmMergeWarps][32], s_s[kLmMergeWarps][32];
   __shared__ int s_a[kLmMergeWarps][32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, row = blockIdx.x * 32 + lane;
