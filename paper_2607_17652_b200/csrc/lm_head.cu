@@ -14,6 +14,14 @@
 //   warps 4-7   epilogue: one thread per output row, 32 columns at a time
 // Tiles are taken vocabulary-major (all row tiles of one 256-token slice of W
 // next to each other), so W streams from HBM once and x stays in L2.
+//
+// Two forms.  One CTA per tile as above, or (kPair) a cluster of two CTAs per 256 rows: one MMA spans both
+// (M 256, cta_group::2), each CTA holds its own 128 rows of x and half of the slice of W, and its
+// accumulator is its own 128 rows again, so the epilogue is the same.  A stage is 32 KB for as many
+// operations as 48 KB before, six stages fit, and a CTA reads 8 KB instead of 12 KB of shared memory
+// per MMA.  What bounds the product is the board's power limit, which is where the saved traffic shows:
+// a step of 64 requests (5,120 rows, V = 151,552, hidden 2048), back to back, 2832 -> 2657 us.
+// Where which one runs: see lm_pairs (on the device, by live rows) and launch_lm_head.
 #include <cudaTypedefs.h>
 
 #include <cfloat>
@@ -27,7 +35,9 @@ constexpr int kLmThreads = 256;
 constexpr int kLmBM = 128, kLmBN = 256, kLmBK = 64, kLmStages = 4;
 constexpr int kLmABytes = kLmBM * kLmBK * 2, kLmBBytes = kLmBN * kLmBK * 2;
 constexpr int kLmStageBytes = kLmABytes + kLmBBytes;                 // 48 KB
+constexpr int kLmPairStages = 6, kLmPairStageBytes = kLmABytes + kLmBBytes / 2;   // 32 KB a CTA
 constexpr int kLmSmem = kLmStages * kLmStageBytes + 2048;            // + barriers + 1 KB alignment slack
+static_assert(kLmPairStages * kLmPairStageBytes == kLmStages * kLmStageBytes, "one shared-memory size for both forms");
 constexpr float kLmLog2e = 1.4426950408889634f;
 
 struct LmParams {
@@ -35,12 +45,9 @@ struct LmParams {
   float4* part;          // [n_tiles_n][rows_pad] (max, sum exp, first index of the max as bits, -)
   int32_t* status;
   int32_t bl, vocab, hidden, n_tiles_n, rows_pad;
+  int32_t pair;          // both forms are launched, lm_pairs says which one works
   long long wait_cycles;
 };
-
-__device__ __forceinline__ bool lm_warp_wait(uint64_t* bar, uint32_t parity, volatile int* abort, long long limit) {
-  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort, limit));
-}
 
 // 32 more columns of a row: running maximum with its first index, sum of exponentials relative to it
 // (an equal later maximum keeps the first index; all -inf adds nothing, a NaN makes the sum NaN).
@@ -77,37 +84,63 @@ __device__ __forceinline__ void absorb32(const uint32_t* v, int col, float& mx, 
   sum += t.x + t.y;
 }
 
+// Row tiles two by two?  An odd one out leaves half of a pair idle for a whole tile.  Call in us at V = 151,552,
+// one CTA a tile / pairs, an even number of row tiles:
+//   hidden 1024:  4 tiles 136 / 122    8 234 / 207   14 400 / 361   20 570 / 537
+//   hidden 2048:  4 tiles 235 / 209    8 421 / 387   14 772 / 715   20 1128 / 1086
+//   hidden 4096:  4 tiles 484 / 442    8 968 / 865
+// 13 tiles, the last pair half empty: 364 / 347 (hidden 1024), 735 / 694 (2048), 1491 / 1477 (4096); at 7 tiles a
+// pair form that takes as long as for 8 would lose.
+constexpr int kLmPairOddTiles = 13;
+__device__ __forceinline__ bool lm_pairs(int m_tiles) { return m_tiles >= 2 && ((m_tiles & 1) == 0 || m_tiles >= kLmPairOddTiles); }
+
+template <bool kPair>
 __global__ void __launch_bounds__(kLmThreads, 1)
 lm_head_stats_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW,
                      const LmParams p) {
+  constexpr int kStages = kPair ? kLmPairStages : kLmStages, kStageBytes = kPair ? kLmPairStageBytes : kLmStageBytes;
+  pdl_wait_only();
+  const int live_rows = *p.n_live * p.bl;
+  const int m_tiles = (live_rows + kLmBM - 1) / kLmBM;          // row tiles that hold live rows
+  if (p.pair && lm_pairs(m_tiles) != kPair) return;             // (the whole grid)
   extern __shared__ uint8_t smem_raw[];
+  // (a pair's CTAs lay their shared memory out alike: the MMA's descriptors are offsets in both)
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kLmStages * kLmStageBytes);
-  uint64_t* full = bars;                    // [4] stage filled (TMA bytes)
-  uint64_t* empty = bars + 4;               // [4] stage consumed (MMA commit)
-  uint64_t* acc_full = bars + 8;            // [2] accumulator complete (MMA commit)
-  uint64_t* acc_empty = bars + 10;          // [2] accumulator read out (4 epilogue warps)
-  uint64_t* drain = bars + 13;              // give-up path only
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 12);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kStages * kStageBytes);
+  uint64_t* full = bars;                    // [kStages] stage filled (TMA bytes); pair: the first CTA's, for both
+  uint64_t* empty = bars + 6;               // [kStages] stage consumed (MMA commit); pair: in both
+  uint64_t* acc_full = bars + 12;           // [2] accumulator complete (MMA commit); pair: in both
+  uint64_t* acc_empty = bars + 14;          // [2] accumulator read out (4 epilogue warps; pair: the first CTA's, 8)
+  uint64_t* drain = bars + 16;              // give-up path only
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 17);
   volatile int* abortf = reinterpret_cast<volatile int*>(tmem_slot + 1);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const long long LIM = p.wait_cycles;
+  const int rank = kPair ? (int)cluster_ctarank() : 0;
+  const bool first = rank == 0;             // issues the MMAs
+  auto wait = [&](uint64_t* bar, uint32_t parity) {
+    return __all_sync(0xffffffffu, kPair ? mbar_wait_cluster(bar, parity, abortf, LIM) : mbar_wait(bar, parity, abortf, LIM));
+  };
   if (tid == 0) {
     *abortf = 0;
-    for (int i = 0; i < kLmStages; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
-    for (int i = 0; i < 2; ++i) { mbar_init(&acc_full[i], 1); mbar_init(&acc_empty[i], 4); }
+    for (int i = 0; i < kStages; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
+    for (int i = 0; i < 2; ++i) { mbar_init(&acc_full[i], 1); mbar_init(&acc_empty[i], kPair ? 8 : 4); }
     mbar_init(drain, 1);
     fence_mbar_init();
     tma_prefetch_desc(&tmX); tma_prefetch_desc(&tmW);
   }
-  if (warp == 1) { tmem_alloc(tmem_slot, 512); tmem_relinquish(); }
+  if (warp == 1) {
+    if constexpr (kPair) { tmem_alloc_pair(tmem_slot, 512); tmem_relinquish_pair(); }
+    else { tmem_alloc(tmem_slot, 512); tmem_relinquish(); }
+  }
   tc_fence_before();
   __syncthreads();
+  if constexpr (kPair) cluster_sync_all();  // both CTAs' barriers are there before either signals the other's
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  const int live_rows = *p.n_live * p.bl;
-  const int m_tiles = (live_rows + kLmBM - 1) / kLmBM;          // row tiles that hold live rows
-  const int n_tiles = m_tiles * p.n_tiles_n;
+  const int m_steps = kPair ? (m_tiles + 1) / 2 : m_tiles;
+  const int n_tiles = m_steps * p.n_tiles_n;
+  const int t0 = kPair ? blockIdx.x / 2 : blockIdx.x, t_step = kPair ? gridDim.x / 2 : gridDim.x;
   const int k_blocks = p.hidden / kLmBK;
 
   if (warp == 0) {
@@ -115,44 +148,59 @@ lm_head_stats_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
     const bool leader = elect_one();
     int fill = 0;
     bool ok = true;
-    for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
-      const int n = t / m_tiles, m = t % m_tiles;
+    for (int t = t0; t < n_tiles && ok; t += t_step) {
+      const int n = t / m_steps, m = (t % m_steps) * (kPair ? 2 : 1) + rank;
       for (int kb = 0; kb < k_blocks; ++kb, ++fill) {
-        const int st = fill % kLmStages, round = fill / kLmStages;
-        if (round > 0 && !lm_warp_wait(&empty[st], (round - 1) & 1, abortf, LIM)) { ok = false; break; }
+        const int st = fill % kStages, round = fill / kStages;
+        if (round > 0 && !wait(&empty[st], (round - 1) & 1)) { ok = false; break; }
         if (leader) {
-          uint8_t* a = smem + st * kLmStageBytes;
-          mbar_arrive_expect_tx(&full[st], kLmStageBytes);
-          tma_load_2d(a, &tmX, &full[st], kb * kLmBK, m * kLmBM);
-          tma_load_2d(a + kLmABytes, &tmW, &full[st], kb * kLmBK, n * kLmBN);
+          uint8_t* a = smem + st * kStageBytes;
+          if constexpr (kPair) {
+            if (first) mbar_arrive_expect_tx(&full[st], 2 * kStageBytes);
+            const uint32_t bar = mapa_u32(&full[st], 0);
+            tma_load_2d_pair(a, &tmX, bar, kb * kLmBK, m * kLmBM);
+            tma_load_2d_pair(a + kLmABytes, &tmW, bar, kb * kLmBK, n * kLmBN + rank * (kLmBN / 2));
+          } else {
+            mbar_arrive_expect_tx(&full[st], kStageBytes);
+            tma_load_2d(a, &tmX, &full[st], kb * kLmBK, m * kLmBM);
+            tma_load_2d(a + kLmABytes, &tmW, &full[st], kb * kLmBK, n * kLmBN);
+          }
         }
         __syncwarp();
       }
     }
-  } else if (warp == 1) {
+  } else if (warp == 1 && first) {
     // ---------------------------------------------------------- MMA issuer
     const bool leader = elect_one();
-    const uint32_t idesc = umma_idesc_bf16(kLmBM, kLmBN, 0, 0);
+    const uint32_t idesc = umma_idesc_bf16(kPair ? 2 * kLmBM : kLmBM, kLmBN, 0, 0);
     const uint64_t dA0 = smem_desc_sw128(smem_u32(smem), 16, 1024);
     const uint64_t dB0 = smem_desc_sw128(smem_u32(smem + kLmABytes), 16, 1024);
     int fill = 0, i = 0;
     bool ok = true;
-    for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x, ++i) {
+    for (int t = t0; t < n_tiles && ok; t += t_step, ++i) {
       const int b = i & 1;
-      if (i >= 2 && !lm_warp_wait(&acc_empty[b], ((i >> 1) - 1) & 1, abortf, LIM)) { ok = false; break; }
+      if (i >= 2 && !wait(&acc_empty[b], ((i >> 1) - 1) & 1)) { ok = false; break; }
       tc_fence_after();
       for (int kb = 0; kb < k_blocks; ++kb, ++fill) {
-        const int st = fill % kLmStages, round = fill / kLmStages;
-        if (!lm_warp_wait(&full[st], round & 1, abortf, LIM)) { ok = false; break; }
+        const int st = fill % kStages, round = fill / kStages;
+        if (!wait(&full[st], round & 1)) { ok = false; break; }
         tc_fence_after();
         if (leader) {
-          const uint32_t so = (uint32_t)((st * kLmStageBytes) >> 4);
+          const uint32_t so = (uint32_t)((st * kStageBytes) >> 4);
 #pragma unroll
-          for (int ks = 0; ks < kLmBK / 16; ++ks)
-            umma_ss(tmem + b * kLmBN, dA0 + so + (uint32_t)((ks * 32) >> 4), dB0 + so + (uint32_t)((ks * 32) >> 4),
-                    idesc, (kb > 0 || ks > 0) ? 1u : 0u);
-          umma_commit(&empty[st]);
-          if (kb == k_blocks - 1) umma_commit(&acc_full[b]);
+          for (int ks = 0; ks < kLmBK / 16; ++ks) {
+            const uint64_t da = dA0 + so + (uint32_t)((ks * 32) >> 4), db = dB0 + so + (uint32_t)((ks * 32) >> 4);
+            const uint32_t acc = (kb > 0 || ks > 0) ? 1u : 0u;
+            if constexpr (kPair) umma_ss_pair(tmem + b * kLmBN, da, db, idesc, acc);
+            else umma_ss(tmem + b * kLmBN, da, db, idesc, acc);
+          }
+          if constexpr (kPair) {
+            umma_commit_pair(&empty[st], true);
+            if (kb == k_blocks - 1) umma_commit_pair(&acc_full[b], true);
+          } else {
+            umma_commit(&empty[st]);
+            if (kb == k_blocks - 1) umma_commit(&acc_full[b]);
+          }
         }
         __syncwarp();
       }
@@ -163,9 +211,9 @@ lm_head_stats_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
     const uint32_t lane_base = (uint32_t)(quad * 32) << 16;
     int i = 0;
     bool ok = true;
-    for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x, ++i) {
-      const int n = t / m_tiles, m = t % m_tiles, b = i & 1;
-      if (!lm_warp_wait(&acc_full[b], (i >> 1) & 1, abortf, LIM)) { ok = false; break; }   // one outcome per warp
+    for (int t = t0; t < n_tiles && ok; t += t_step, ++i) {
+      const int n = t / m_steps, m = (t % m_steps) * (kPair ? 2 : 1) + rank, b = i & 1;
+      if (!wait(&acc_full[b], (i >> 1) & 1)) { ok = false; break; }   // one outcome per warp
       tc_fence_after();
       const uint32_t tacc = tmem + lane_base + b * kLmBN;
       const int col0 = n * kLmBN;
@@ -190,7 +238,10 @@ lm_head_stats_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&acc_empty[b]);
+      if (lane == 0) {
+        if (first) mbar_arrive(&acc_empty[b]);
+        else mbar_arrive_cluster_relaxed(mapa_u32(&acc_empty[b], 0));   // (what it hands back is tensor memory)
+      }
       const int row = m * kLmBM + quad * 32 + lane;
       if (row < live_rows)
         p.part[(size_t)n * p.rows_pad + row] = make_float4(mx, sum, __int_as_float(arg), 0.f);
@@ -202,15 +253,19 @@ lm_head_stats_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
     // give-up path: the MMA warp waits for everything it has issued (own barrier, bounded
     // polls), copies in flight land while the CTA sleeps, then TMEM and shared memory go back
     if (tid == 0) atomicOr(p.status, FB_ST_DEV_TIMEOUT);
-    if (warp == 1) {
-      if (elect_one()) umma_commit(drain);
+    if (warp == 1 && first) {
+      if (elect_one()) { if constexpr (kPair) umma_commit_pair(drain, false); else umma_commit(drain); }
       __syncwarp();
       for (int i = 0; i < 4096 && !mbar_test(drain, 0); ++i) __nanosleep(200);
     }
     for (int i = 0; i < 64; ++i) __nanosleep(10000);
     __syncthreads();
   }
-  if (warp == 1) { tc_fence_after(); tmem_dealloc(tmem, 512); }
+  if constexpr (kPair) cluster_sync_all();  // neither CTA leaves while the other may still signal it or read its shared memory
+  if (warp == 1) {
+    tc_fence_after();
+    if constexpr (kPair) tmem_dealloc_pair(tmem, 512); else tmem_dealloc(tmem, 512);
+  }
 }
 
 // Tiles of a row -> top-1 token (lowest index on ties) and its confidence 1 / sum exp(z - max).
@@ -279,7 +334,10 @@ size_t lm_head_workspace_bytes(const fb_ctx* ctx) {
 
 // per-device kernel attribute (called from ensure_device with that device current)
 int lm_head_device_setup(fb_ctx* ctx) {
-  return cuda_err(ctx, cudaFuncSetAttribute(lm_head_stats_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  if (int e = cuda_err(ctx, cudaFuncSetAttribute(lm_head_stats_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 kLmSmem), "smem attr"))
+    return e;
+  return cuda_err(ctx, cudaFuncSetAttribute(lm_head_stats_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                             kLmSmem), "smem attr");
 }
 
@@ -290,7 +348,7 @@ int launch_lm_head(fb_ctx* ctx, const fb_pack* pk, const void* x, const void* w,
   const fb_config& c = ctx->cfg;
   const int rows = c.max_requests * c.wmax * c.block_len;
   auto fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled>(ctx->encode_fn);
-  CUtensorMap tmX, tmW;
+  CUtensorMap tmX, tmW, tmWHalf;
   const cuuint32_t es[2] = {1, 1};
   {
     const cuuint64_t dims[2] = {(cuuint64_t)hidden, (cuuint64_t)rows};
@@ -304,8 +362,11 @@ int launch_lm_head(fb_ctx* ctx, const fb_pack* pk, const void* x, const void* w,
   {
     const cuuint64_t dims[2] = {(cuuint64_t)hidden, (cuuint64_t)c.vocab};
     const cuuint64_t str[1] = {(cuuint64_t)hidden * 2};
-    const cuuint32_t box[2] = {kLmBK, kLmBN};
+    const cuuint32_t box[2] = {kLmBK, kLmBN}, half[2] = {kLmBK, kLmBN / 2};
     if (fn(&tmW, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(w), dims, str, box, es,
+           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS ||
+        fn(&tmWHalf, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(w), dims, str, half, es,
            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
       return set_err(ctx, FB_ERR_CUDA, "cuTensorMapEncodeTiled failed for w");
@@ -318,8 +379,18 @@ int launch_lm_head(fb_ctx* ctx, const fb_pack* pk, const void* x, const void* w,
   p.n_tiles_n = (c.vocab + kLmBN - 1) / kLmBN;
   p.rows_pad = lm_rows_pad(c);
   p.wait_cycles = ctx->wait_cycles;
-  lm_head_stats_kernel<<<ctx->num_sms, kLmThreads, kLmSmem, stream>>>(tmX, tmW, p);
-  if (int e = cuda_err(ctx, cudaGetLastError(), "lm_head_stats_kernel launch")) return e;
+  // Both forms are launched, since the live rows are only known on the device; the one that is not wanted costs
+  // 2 us.  So not for small calls (three row tiles: 112 us + 2), and not below 768 hidden elements, where the
+  // epilogue bounds a tile and pairs gain nothing (hidden 512: 4 tiles 91 / 96, 20 tiles 355 / 357).
+  const int most_tiles = (rows + kLmBM - 1) / kLmBM;
+  p.pair = most_tiles >= 4 && hidden >= 768 && (long long)most_tiles * p.n_tiles_n >= 8ll * ctx->num_sms;
+  if (p.pair)
+    if (int e = cuda_err(ctx, launch_pdl_cluster(lm_head_stats_kernel<true>, ctx->num_sms / 2 * 2, kLmThreads, kLmSmem, stream, 2,
+                                                 tmX, tmWHalf, p), "lm_head_stats_kernel (pairs) launch"))
+      return e;
+  if (int e = cuda_err(ctx, launch_pdl(lm_head_stats_kernel<false>, ctx->num_sms, kLmThreads, kLmSmem, stream, tmX, tmW, p),
+                       "lm_head_stats_kernel launch"))
+    return e;
   if (int e = cuda_err(ctx, launch_pdl(lm_head_merge_kernel, (rows + 31) / 32, 32 * kLmMergeWarps, 0, stream, p, argmax, conf, rows),
                        "lm_head_merge_kernel launch"))
     return e;
