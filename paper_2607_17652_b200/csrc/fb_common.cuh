@@ -173,15 +173,20 @@ __host__ __device__ inline int split_candidate(int i, int longest) {
   return (int)((4u * (unsigned)longest + q - 1u) / q);
 }
 struct SplitStat { unsigned work; int items, parts, longest; };
-__host__ __device__ inline void split_stat_add(SplitStat& s, const ReqGeom& g, int n_kv_heads, int ct) {
-  if (g.nt <= 0) return;
-  const int nch = (g.nt + ct - 1) / ct, len = (g.nt + nch - 1) / nch, fixed = nch > 1 ? kPieceCost : kItemCost;
-  const int pairs = g.nfull * n_kv_heads, duals = g.nunits - pairs;
-  s.work += (unsigned)g.nt * (unsigned)(pairs * kTileCost + duals * kTileDualCost) + (unsigned)(g.nunits * nch * fixed);
-  s.items += g.nunits * nch;
-  s.parts += nch > 1 ? g.nunits * nch : 0;
+// one request of `nt` key tiles, `nunits` units of which `pairs` are pairs of tiles, cut into `nch` pieces of at
+// most `len` tiles
+__host__ __device__ inline void split_stat_add_pieces(SplitStat& s, int nt, int pairs, int nunits, int nch, int len) {
+  const int fixed = nch > 1 ? kPieceCost : kItemCost, duals = nunits - pairs;
+  s.work += (unsigned)nt * (unsigned)(pairs * kTileCost + duals * kTileDualCost) + (unsigned)(nunits * nch * fixed);
+  s.items += nunits * nch;
+  s.parts += nch > 1 ? nunits * nch : 0;
   const int item = len * (duals > 0 ? kTileDualCost : kTileCost) + fixed;
   s.longest = item > s.longest ? item : s.longest;
+}
+__host__ __device__ inline void split_stat_add(SplitStat& s, const ReqGeom& g, int n_kv_heads, int ct) {
+  if (g.nt <= 0) return;
+  const int nch = (g.nt + ct - 1) / ct;
+  split_stat_add_pieces(s, g.nt, g.nfull * n_kv_heads, g.nunits, nch, (g.nt + nch - 1) / nch);
 }
 // a product that no compiler fuses with the sum it feeds
 __host__ __device__ inline float rounded_product(float a, float b) {

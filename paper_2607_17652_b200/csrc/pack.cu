@@ -12,7 +12,7 @@ namespace fb {
 
 // Threads per block: bound by latency (dependent loads, block barriers), so small batches take
 // small blocks: call in us with 256 / 512 / 1024 threads, 1 request 5.5 / 6.0 / 7.0, 8 requests 5.9 /
-// 6.6 / 7.6, 24 requests 8.6 / 8.0 / 8.9, 128 requests 19.0 / 16.9 / 17.2.
+// 6.6 / 7.6, 24 requests 8.6 / 8.0 / 8.9, 128 requests 19.0 / 16.9 / 17.2 (measured before build_sched got shorter).
 constexpr int kPackThreads = 512, kPackThreadsSmall = 256, kPackSmallRequests = 8;
 constexpr int kSlotsPerBlock = 32;
 constexpr int kCostBins = 1024;
@@ -97,22 +97,31 @@ __device__ __forceinline__ ReqGeom req_geom(const PackParams& p, int r, int list
   return geom_of(p, w, w ? P : 0, list);
 }
 
+// a / d for 0 <= a, 0 < d with a quotient below 2^20: a reciprocal (inv_of(d)) off by a few units in the last
+// place puts the product within one of the quotient, the remainder says which way.  The list is built by
+// chains of such quotients; a hardware-less integer division is four times as long.
+__device__ __forceinline__ float inv_of(int d) { return __fdividef(1.0f, (float)d); }
+__device__ __forceinline__ int quot(int a, int d, float inv) {
+  const int q = (int)((float)a * inv), r = a - q * d;
+  return q + (r >= d) - (r < 0);
+}
+
 // unit record of two Q tiles qa, qb (absolute tile indices of the request; qb < 0: none) under
 // KV heads hA, hB
 __device__ __forceinline__ AttnUnit make_unit(const PackParams& p, const ReqGeom& q, int req, int first, int qa, int qb,
-                                              int hA, int hB) {
+                                              int hA, int hB, float inv_tps) {
   AttnUnit un;
   un.req = req;
   un.kvh = hA | (hB << 16);
-  const int sA = qa / p.tiles_per_slot;
+  const int sA = quot(qa, p.tiles_per_slot, inv_tps);
   un.slotA = first + sA;
-  un.t0A = (qa % p.tiles_per_slot) * p.tokens_per_tile;
+  un.t0A = (qa - sA * p.tiles_per_slot) * p.tokens_per_tile;
   un.winA = (sA + 1) * p.bl;
   un.nvisA = p.resident ? (q.P + un.winA + kTileN - 1) / kTileN : q.npt + (un.winA + kTileN - 1) / kTileN;
   if (qb >= 0) {
-    const int sB = qb / p.tiles_per_slot;
+    const int sB = quot(qb, p.tiles_per_slot, inv_tps);
     un.slotB = first + sB;
-    un.t0B = (qb % p.tiles_per_slot) * p.tokens_per_tile;
+    un.t0B = (qb - sB * p.tiles_per_slot) * p.tokens_per_tile;
     un.winB = (sB + 1) * p.bl;
     un.nvisB = p.resident ? (q.P + un.winB + kTileN - 1) / kTileN : q.npt + (un.winB + kTileN - 1) / kTileN;
   } else {
@@ -126,117 +135,94 @@ __device__ __forceinline__ AttnUnit make_unit(const PackParams& p, const ReqGeom
 // `list` 0: pairs of tiles and leftover tiles, one record per scheduling unit.  `list` 1: quads,
 // two records per scheduling unit (2u for the first CTA of the pair, 2u + 1 for the second), both
 // cut into the same chunks; an item names record 2u.
+//
+// Bound by the chain of dependent steps in one block.  Up to kPackSmallRequests every warp holds all of them, a
+// lane each, and forms sums, split and bases for itself, without a barrier; above, a thread holds a request
+// (a lane each up to 32 requests: 24 requests 9.8 us, a thread each 7.7).  Call in us, back to back, before and with
+// this and the quotients by reciprocal: one request of 3,000 tokens 5.7 / 4.2, 8 requests 6.1 / 5.4, 24 requests
+// 8.2 / 7.7, 64 requests 9.7 to 11 / 8.2 to 9.4, in 8 bits 10 to 13 / 8.8, 128 requests 14 to 18 / 12.4 to 16.
+// Steps: a toy request 23.3 / 21.3, one request with four layers 110.1 / 107.5, a 28,000-token one 83.2 / 82.2.
 template <int T>
 __device__ void build_sched(const PackParams& p, const int list) {
+  constexpr unsigned kAll = 0xffffffffu;
+  constexpr int NW = T / 32;
   const int mult = list + 1;            // unit records (and partial-result ranges) per scheduling unit
   SchedHeader* const hdr = p.hdr[list];
   AttnItem* const items = p.items[list];
   AttnUnit* const units = p.units[list];
   const int max_items = p.max_items[list], max_units = p.max_units[list], max_parts = p.max_parts[list];
-  __shared__ int sh_scan[3 * T / 32], sh_scan2[T / 32], sh_scan3[T / 32];
+  __shared__ int sh_scan[3 * NW], sh_scan2[NW], sh_scan3[NW];
   __shared__ int bins[kCostBins];
   __shared__ int sh_total, sh_units, sh_chunks, sh_longest;
   __shared__ SplitStat sh_stat[kSplitCandidates];
   static_assert(kSplitCandidates == 32, "one lane per candidate");
   __shared__ SplitRule sh_rule;
-  __shared__ int s_ub[T + 1], s_pb[T], s_first[T], s_wb[T], s_w[T], s_P[T];
+  __shared__ int s_ub[T], s_pb[T], s_first[T], s_wb[T], s_w[T], s_P[T];
   __shared__ int4 s_info[kUnitInfo];
   __shared__ int s_req[kUnitInfo];
-  const int tid = threadIdx.x;
-  if (tid == 0) { sh_total = 0; sh_units = 0; sh_chunks = 0; sh_longest = 0; }
-  if (tid < kSplitCandidates) sh_stat[tid] = SplitStat{};
-  for (int i = tid; i < kCostBins; i += T) bins[i] = 0;
-  // phase 1: total key-tile work, longest key range -> chunk length.  The requests' geometry is
-  // loaded once where one pass over the requests holds all of them.
-  const bool one_pass = p.max_requests <= T;
-  ReqGeom g0{};
-  int mine = 0, mine_units = 0, mine_longest = 0;
-  for (int r = tid; r < p.max_requests; r += T) {
-    const ReqGeom g = req_geom(p, r, list);
-    mine += g.nunits * g.nt;
-    mine_units += g.nt ? g.nunits : 0;
-    mine_longest = max(mine_longest, g.nt);
-    g0 = g;
-  }
-  s_w[tid] = g0.w; s_P[tid] = g0.P;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    mine += __shfl_xor_sync(0xffffffffu, mine, o);
-    mine_units += __shfl_xor_sync(0xffffffffu, mine_units, o);
-    mine_longest = max(mine_longest, __shfl_xor_sync(0xffffffffu, mine_longest, o));
-  }
-  __syncthreads();
-  if ((tid & 31) == 0 && mine_units) {
-    atomicAdd(&sh_total, mine); atomicAdd(&sh_units, mine_units); atomicMax(&sh_longest, mine_longest);
-  }
-  __syncthreads();
-  if (list == 0 && p.auto_split && !split_worth_estimating(sh_total, sh_units, sh_longest)) {
-    if (tid == 0) sh_rule = split_auto(sh_total, sh_units, max(sh_longest, 1), p.min_chunk_tiles);
-  } else if (list == 0 && p.auto_split) {
-    // every lane a candidate chunk length, the requests dealt to the warps; then the least
-    // (estimate, candidate) wins
-    const int lane = tid & 31, ct = max(split_candidate(lane, sh_longest), 1);
-    SplitStat st{};
-    for (int r = tid >> 5; r < p.max_requests; r += T / 32)
-      split_stat_add(st, one_pass ? geom_of(p, s_w[r], s_P[r], list) : req_geom(p, r, list), p.n_kv_heads, ct);
-    if (st.items) {
-      atomicAdd(&sh_stat[lane].work, st.work); atomicAdd(&sh_stat[lane].items, st.items);
-      atomicAdd(&sh_stat[lane].parts, st.parts); atomicMax(&sh_stat[lane].longest, st.longest);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const float inv_tps = inv_of(p.tiles_per_slot);
+
+  // Record of unit `ul` of a request of list 0.  Full pairs first, numbered h * nfull + pr: the pairs of one
+  // (request, KV head) are adjacent, are handed out back to back and so share their K/V through L2.  Then the
+  // leftover tile, one unit per two KV heads.
+  auto unit_record = [&](const ReqGeom& q, int req, int first, int ul) {
+    const bool full = ul < q.nfull * p.n_kv_heads;
+    const int hf = q.nfull > 1 ? quot(ul, q.nfull, inv_of(q.nfull)) : ul;
+    const int h = full ? hf : 2 * (ul - q.nfull * p.n_kv_heads);
+    const int qa = q.tile0 + (full ? 2 * (ul - hf * q.nfull) : q.ntq - 1);
+    const bool two = !full && h + 1 < p.n_kv_heads;
+    return make_unit(p, q, req, first, qa, full ? qa + 1 : two ? qa : -1, h, two ? h + 1 : h, inv_tps);
+  };
+  // the last k < n with base[k] <= i (requests without units share their successor's base and are skipped by "last")
+  auto owner = [](const int* base, int n, int i) {
+    int lo = 0, hi = n - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (base[mid] <= i) lo = mid; else hi = mid - 1;
     }
-    __syncthreads();
-    if (tid < 32) {
-      const float e = lane > 0 && ct < p.auto_min_chunk ? -1.f : split_estimate(sh_stat[lane], max_parts);
-      // (non-negative floats order like their bits; nothing to do at all: candidate 0)
-      unsigned best = e >= 0.f ? __float_as_uint(e) : 0xffffffffu;
-      int at = lane;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const unsigned b2 = __shfl_xor_sync(0xffffffffu, best, o);
-        const int a2 = __shfl_xor_sync(0xffffffffu, at, o);
-        if (b2 < best || (b2 == best && a2 < at)) { best = b2; at = a2; }
+    return lo;
+  };
+  // One request, no more items than SMs: its pieces are alike and each CTA gets one or none, so nothing is sorted.
+  // (Not for several requests: with the longest pieces first, the two SMs of a pair get a long and a short one;
+  // 8 requests with four layers 167 us a step sorted, 169 without.)  A unit's pieces side by side: with the same keys of
+  // all units side by side instead, one request of 3,000 tokens and four layers takes 1 % longer.
+  auto one_request = [&](const SplitRule& rule, int k, int n_items) {
+    const ReqGeom q = geom_of(p, s_w[k], s_P[k], list);
+    const int nc = req_split(rule, s_wb[k], q.nunits, q.nt).nch_c;
+    const float inv = inv_of(max(nc, 1));
+    for (int i = tid; i < n_items; i += T) {
+      const int u = quot(i, nc, inv), c = i - u * nc;
+      if (c == 0) {
+        AttnUnit un = unit_record(q, k, s_first[k], u);
+        un.n_chunks = nc;
+        un.part_base = nc > 1 ? i : -1;
+        units[u] = un;
       }
-      const int chosen = __shfl_sync(0xffffffffu, ct, at);
-      if (lane == 0) sh_rule = split_auto(sh_total, sh_units, chosen, p.min_chunk_tiles);
+      AttnItem it; it.unit = u; it.chunk = c; it.jb = quot(c * q.nt, nc, inv); it.je = quot((c + 1) * q.nt, nc, inv);
+      it.req = k; it.pad[0] = it.pad[1] = it.pad[2] = 0;
+      items[i] = it;
     }
-  } else if (tid == 0) {
-    sh_rule = split_rule(sh_total, sh_units, p.target_items[list], p.min_chunk_tiles);
-  }
-  __syncthreads();
-  const SplitRule rule = sh_rule;
-  // phase 2 + 3: per-request bases (scan over up to T requests at a time), then the units of
-  // these requests: unit record, cost histogram of its items.  A unit cut into many pieces is
-  // given to several threads.
-  int unit_run = 0, part_run = 0, slot_run = 0, work_run = 0, lanes = 1;
-  for (int r0 = 0; r0 < p.max_requests; r0 += T) {
-    const int r = r0 + tid;
-    ReqGeom g{};
-    if (one_pass) g = g0;
-    else if (r < p.max_requests) g = req_geom(p, r, list);
-    const int nunits = g.nt ? g.nunits : 0;
-    int pre[3], tot[3];
-    block_excl_scan<T, 3>({nunits * g.nt, nunits, g.w}, pre, tot, sh_scan);
-    const int wbase = work_run + pre[0];
-    const ReqSplit rs = req_split(rule, wbase, nunits, g.nt);
-    if (nunits) atomicMax(&sh_chunks, max(rs.ufine > 0 ? rs.nch_c : 0, rs.ufine < nunits ? rs.nch_f : 0));
-    int ppre[1], ptot[1];
-    block_excl_scan<T, 1>({rs.parts(nunits)}, ppre, ptot, sh_scan2);
-    const int tu = tot[1];
-    s_ub[tid] = pre[1]; s_pb[tid] = part_run + ppre[0]; s_first[tid] = slot_run + pre[2]; s_wb[tid] = wbase;
-    if (!one_pass) { s_w[tid] = g.w; s_P[tid] = g.P; }
-    if (tid == 0) s_ub[T] = tu;
-    __syncthreads();
-    lanes = 1;
-    while (lanes < 32 && lanes < sh_chunks && 2 * lanes * tu <= T) lanes *= 2;
-    for (int j = tid; j < tu * lanes; j += T) {
-      const int i = j / lanes, c0 = j % lanes;
-      // the request of unit i: the last k with s_ub[k] <= i (requests without units share
-      // their successor's base and are skipped by "last")
-      int lo = 0, hi = min(T, p.max_requests - r0) - 1;
-      while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (s_ub[mid] <= i) lo = mid; else hi = mid - 1;
-      }
-      const int k = lo, ul = i - s_ub[k];
+  };
+  auto write_header = [&](int n_items, int unit_total, int part_total, int total_tiles, int ct, int most) {
+    if (tid != 0) return;
+    hdr->n_items = min(n_items, max_items);
+    hdr->n_units = min(mult * unit_total, max_units);
+    hdr->chunk_tiles = ct;
+    hdr->n_parts = mult * part_total;
+    hdr->total_tiles = total_tiles;
+    hdr->ticket = 0; hdr->done = 0; hdr->max_chunks = most;
+    if (n_items > max_items || mult * unit_total > max_units || mult * part_total > max_parts)
+      atomicOr(p.status, FB_ST_BAD_STATE);
+  };
+  // The units of the `n` requests from r0 on, whose geometry and bases are in the tables: unit record, cost
+  // histogram of its items.  A unit cut into many pieces is given to several threads.
+  auto write_units = [&](const SplitRule& rule, int r0, int n, int tu, int unit_run, int most) {
+    int shift = 0;
+    while (shift < 5 && (1 << shift) < most && (tu << (shift + 1)) <= T) ++shift;
+    for (int j = tid; j < tu << shift; j += T) {
+      const int i = j >> shift, c0 = j & ((1 << shift) - 1);
+      const int k = owner(s_ub, n, i), ul = i - s_ub[k];
       const int u = unit_run + i;
       if (mult * (u + 1) > max_units) continue;
       const ReqGeom q = geom_of(p, s_w[k], s_P[k], list);
@@ -244,20 +230,12 @@ __device__ void build_sched(const PackParams& p, const int list) {
       const int first = s_first[k], nc = qs.chunks(ul);
       AttnUnit un[2];
       if (list == 0) {
-        // Full pairs first, numbered h * nfull + pr: the pairs of one (request, KV head) are
-        // adjacent, are handed out back to back and so share their K/V through L2.  Then the
-        // leftover tile, one unit per two KV heads.
-        const bool full = ul < q.nfull * p.n_kv_heads;
-        const int h = full ? ul / q.nfull : 2 * (ul - q.nfull * p.n_kv_heads);
-        const int qa = q.tile0 + (full ? 2 * (ul % q.nfull) : q.ntq - 1);
-        if (full) un[0] = make_unit(p, q, r0 + k, first, qa, qa + 1, h, h);
-        else if (h + 1 < p.n_kv_heads) un[0] = make_unit(p, q, r0 + k, first, qa, qa, h, h + 1);
-        else un[0] = make_unit(p, q, r0 + k, first, qa, -1, h, h);
+        un[0] = unit_record(q, r0 + k, first, ul);
       } else {
         // quad qd of KV head h: tiles 4 qd + r and 4 qd + 2 + r belong to CTA r of the pair
         const int h = ul / q.nquad, qd = ul % q.nquad;
-        un[0] = make_unit(p, q, r0 + k, first, 4 * qd, 4 * qd + 2, h, h);
-        un[1] = make_unit(p, q, r0 + k, first, 4 * qd + 1, 4 * qd + 3, h, h);
+        un[0] = make_unit(p, q, r0 + k, first, 4 * qd, 4 * qd + 2, h, h, inv_tps);
+        un[1] = make_unit(p, q, r0 + k, first, 4 * qd + 1, 4 * qd + 3, h, h, inv_tps);
       }
       int nch = nc;
       const int pb = nc > 1 ? mult * (s_pb[k] + qs.part_off(ul)) : -1;
@@ -272,18 +250,17 @@ __device__ void build_sched(const PackParams& p, const int list) {
         nvA = max(nvA, un[rr].nvisA); nvB = max(nvB, un[rr].nvisB);
       }
       if (c0 == 0 && u < kUnitInfo) { s_info[u] = make_int4(nvA, nvB, q.nt, nch); s_req[u] = r0 + k; }
-      for (int c = c0; c < nch; c += lanes) {
-        const int jb = c * q.nt / nc, je = (c + 1) * q.nt / nc;
-        int cost = item_cost(max(0, min(je, nvA) - jb), max(0, min(je, nvB) - jb));
+      const float inv = inv_of(nc);
+      for (int c = c0; c < nch; c += 1 << shift) {
+        const int jb = quot(c * q.nt, nc, inv), je = quot((c + 1) * q.nt, nc, inv);
+        const int cost = item_cost(max(0, min(je, nvA) - jb), max(0, min(je, nvB) - jb));
         atomicAdd(&bins[min(cost, kCostBins - 1)], 1);
       }
     }
-    unit_run += tu; part_run += ptot[0]; slot_run += tot[2]; work_run += tot[0];
-    __syncthreads();                      // the tables are overwritten next
-  }
-  // descending exclusive offsets over the cost bins: thread t owns the bins
-  // kCostBins-1-kBinsPer*t and below (largest cost first)
-  {
+  };
+  // Behind the units: descending exclusive offsets over the cost bins (thread t owns the bins
+  // kCostBins - 1 - kBinsPer * t and below: largest cost first), the header, the items, longest first.
+  auto write_items = [&](int unit_total, int part_total, int total_tiles, int ct, int most) {
     constexpr int kBinsPer = kCostBins / T;
     static_assert(kBinsPer * T == kCostBins && kBinsPer >= 1, "whole bins per thread");
     int c[kBinsPer], sum = 0;
@@ -295,45 +272,183 @@ __device__ void build_sched(const PackParams& p, const int list) {
     const int total_items = btot[0];
 #pragma unroll
     for (int j = 0; j < kBinsPer; ++j) { bins[kCostBins - 1 - (kBinsPer * tid + j)] = base; base += c[j]; }
-    if (tid == 0) {
-      hdr->n_items = min(total_items, max_items);
-      hdr->n_units = min(mult * unit_run, max_units);
-      hdr->chunk_tiles = rule.ct;
-      hdr->n_parts = mult * part_run;
-      hdr->total_tiles = sh_total;
-      hdr->ticket = 0; hdr->done = 0; hdr->max_chunks = sh_chunks;
-      if (total_items > max_items || mult * unit_run > max_units || mult * part_run > max_parts)
-        atomicOr(p.status, FB_ST_BAD_STATE);
-    }
-  }
-  __syncthreads();
-  // phase 4: scatter items, longest first
-  const int n_sched = min(unit_run, max_units / mult);
-  lanes = 1;
-  while (lanes < 32 && lanes < sh_chunks && 2 * lanes * n_sched <= T) lanes *= 2;
-  for (int j = tid; j < n_sched * lanes; j += T) {
-    const int u = j / lanes;
-    int nvA, nvB, nt, nch, req;
-    if (u < kUnitInfo) {
-      req = s_req[u];
-      const int4 f = s_info[u];
-      nvA = f.x; nvB = f.y; nt = f.z; nch = f.w;
-    } else {
-      const AttnUnit un = units[mult * u];
-      nvA = un.nvisA; nvB = un.nvisB; nt = un.n_tiles; nch = un.n_chunks; req = un.req;
-      if (mult == 2) { const AttnUnit u1 = units[2 * u + 1]; nvA = max(nvA, u1.nvisA); nvB = max(nvB, u1.nvisB); }
-    }
-    for (int c = j % lanes; c < nch; c += lanes) {
-      const int jb = c * nt / nch, je = (c + 1) * nt / nch;
-      int cost = item_cost(max(0, min(je, nvA) - jb), max(0, min(je, nvB) - jb));
-      const int at = atomicAdd(&bins[min(cost, kCostBins - 1)], 1);
-      if (at < max_items) {
-        AttnItem it; it.unit = mult * u; it.chunk = c; it.jb = jb; it.je = je;
-        it.req = req; it.pad[0] = it.pad[1] = it.pad[2] = 0;
-        items[at] = it;
+    write_header(total_items, unit_total, part_total, total_tiles, ct, most);
+    __syncthreads();
+    const int n_sched = min(unit_total, max_units / mult);
+    int shift = 0;
+    while (shift < 5 && (1 << shift) < most && (n_sched << (shift + 1)) <= T) ++shift;
+    for (int j = tid; j < n_sched << shift; j += T) {
+      const int u = j >> shift;
+      int nvA, nvB, nt, nch, req;
+      if (u < kUnitInfo) {
+        req = s_req[u];
+        const int4 f = s_info[u];
+        nvA = f.x; nvB = f.y; nt = f.z; nch = f.w;
+      } else {
+        const AttnUnit un = units[mult * u];
+        nvA = un.nvisA; nvB = un.nvisB; nt = un.n_tiles; nch = un.n_chunks; req = un.req;
+        if (mult == 2) { const AttnUnit u1 = units[2 * u + 1]; nvA = max(nvA, u1.nvisA); nvB = max(nvB, u1.nvisB); }
+      }
+      const float inv = inv_of(max(nch, 1));
+      for (int c = j & ((1 << shift) - 1); c < nch; c += 1 << shift) {
+        const int jb = quot(c * nt, nch, inv), je = quot((c + 1) * nt, nch, inv);
+        const int cost = item_cost(max(0, min(je, nvA) - jb), max(0, min(je, nvB) - jb));
+        const int at = atomicAdd(&bins[min(cost, kCostBins - 1)], 1);
+        if (at < max_items) {
+          AttnItem it; it.unit = mult * u; it.chunk = c; it.jb = jb; it.je = je;
+          it.req = req; it.pad[0] = it.pad[1] = it.pad[2] = 0;
+          items[at] = it;
+        }
       }
     }
+  };
+  auto most_chunks = [](const ReqSplit& sp, int nunits) {
+    return nunits ? max(sp.ufine > 0 ? sp.nch_c : 0, sp.ufine < nunits ? sp.nch_f : 0) : 0;
+  };
+  // the candidate of this lane, and the best of all: the least (estimate, candidate)
+  auto best_candidate = [&](const SplitStat& st, int ct) {
+    const float e = lane > 0 && ct < p.auto_min_chunk ? -1.f : split_estimate(st, max_parts);
+    // (non-negative floats order like their bits; nothing to do at all: candidate 0)
+    const unsigned mine = e >= 0.f ? __float_as_uint(e) : 0xffffffffu, least = __reduce_min_sync(kAll, mine);
+    return __shfl_sync(kAll, ct, __ffs(__ballot_sync(kAll, mine == least)) - 1);
+  };
+  auto add_request = [&](SplitStat& st, int nt, int pairs, int nunits, int ct, float inv_ct) {
+    const int nch = quot(nt + ct - 1, ct, inv_ct), len = quot(nt + nch - 1, nch, inv_of(nch));
+    split_stat_add_pieces(st, nt, pairs, nunits, nch, len);
+  };
+
+  for (int i = tid; i < kCostBins; i += T) bins[i] = 0;
+  if (p.max_requests <= kPackSmallRequests) {
+    // ---- every warp for itself: lane r is request r
+    const ReqGeom g = lane < p.max_requests ? req_geom(p, lane, list) : ReqGeom{};
+    const int nunits = g.nt ? g.nunits : 0, pairs = g.nfull * p.n_kv_heads;
+    const int total = __reduce_add_sync(kAll, nunits * g.nt), n_units = __reduce_add_sync(kAll, nunits);
+    const int longest = __reduce_max_sync(kAll, g.nt);
+    SplitRule rule;
+    if (list == 0 && p.auto_split) {
+      int chosen = max(longest, 1);
+      if (split_worth_estimating(total, n_units, longest)) {
+        const int ct = max(split_candidate(lane, longest), 1);
+        const float inv_ct = inv_of(ct);
+        SplitStat st{};
+        for (unsigned todo = __ballot_sync(kAll, nunits > 0); todo; todo &= todo - 1) {
+          const int r = __ffs(todo) - 1;
+          add_request(st, __shfl_sync(kAll, g.nt, r), __shfl_sync(kAll, pairs, r), __shfl_sync(kAll, nunits, r), ct, inv_ct);
+        }
+        chosen = best_candidate(st, ct);
+      }
+      rule = split_auto(total, n_units, chosen, p.min_chunk_tiles);
+    } else {
+      rule = split_rule(total, n_units, p.target_items[list], p.min_chunk_tiles);
+    }
+    int v[3] = {nunits * g.nt, nunits, g.w}, x[3] = {v[0], v[1], v[2]};
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1)
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        const int y = __shfl_up_sync(kAll, x[i], o);
+        if (lane >= o) x[i] += y;
+      }
+    const ReqSplit sp = req_split(rule, x[0] - v[0], nunits, g.nt);
+    const int parts = sp.parts(nunits), most = __reduce_max_sync(kAll, most_chunks(sp, nunits));
+    const int n_items = __reduce_add_sync(kAll, sp.items(nunits));
+    int xp = parts;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(kAll, xp, o);
+      if (lane >= o) xp += y;
+    }
+    if (warp == 0) {
+      s_ub[lane] = x[1] - v[1]; s_pb[lane] = xp - parts; s_first[lane] = x[2] - v[2];
+      s_wb[lane] = x[0] - v[0]; s_w[lane] = g.w; s_P[lane] = g.P;
+    }
+    const int part_total = __shfl_sync(kAll, xp, 31);
+    __syncthreads();                    // the tables are there, the bins are clear
+    const unsigned with_work = __ballot_sync(kAll, nunits > 0);
+    if (list == 0 && __popc(with_work) == 1 && rule.fine_from == 0x7fffffff && n_items <= min(kSms, max_items) &&
+        n_units <= max_units && part_total <= max_parts) {
+      write_header(n_items, n_units, part_total, total, rule.ct, most);
+      one_request(rule, __ffs(with_work) - 1, n_items);
+      return;
+    }
+    write_units(rule, 0, p.max_requests, n_units, 0, most);
+    __syncthreads();
+    write_items(n_units, part_total, total, rule.ct, most);
+    return;
   }
+  // ---- a thread per request, T at a time
+  if (tid == 0) { sh_total = 0; sh_units = 0; sh_chunks = 0; sh_longest = 0; }
+  if (tid < kSplitCandidates) sh_stat[tid] = SplitStat{};
+  // phase 1: total key-tile work, longest key range -> chunk length.  The requests' geometry is
+  // loaded once where one pass over the requests holds all of them.
+  const bool one_pass = p.max_requests <= T;
+  ReqGeom g0{};
+  int mine = 0, mine_units = 0, mine_longest = 0;
+  for (int r = tid; r < p.max_requests; r += T) {
+    const ReqGeom g = req_geom(p, r, list);
+    mine += g.nunits * g.nt;
+    mine_units += g.nt ? g.nunits : 0;
+    mine_longest = max(mine_longest, g.nt);
+    g0 = g;
+  }
+  s_w[tid] = g0.w; s_P[tid] = g0.P;
+  mine = __reduce_add_sync(kAll, mine); mine_units = __reduce_add_sync(kAll, mine_units);
+  mine_longest = __reduce_max_sync(kAll, mine_longest);
+  __syncthreads();
+  if (lane == 0 && mine_units) {
+    atomicAdd(&sh_total, mine); atomicAdd(&sh_units, mine_units); atomicMax(&sh_longest, mine_longest);
+  }
+  __syncthreads();
+  if (list == 0 && p.auto_split && !split_worth_estimating(sh_total, sh_units, sh_longest)) {
+    if (tid == 0) sh_rule = split_auto(sh_total, sh_units, max(sh_longest, 1), p.min_chunk_tiles);
+  } else if (list == 0 && p.auto_split) {
+    // every lane a candidate chunk length, the requests dealt to the warps
+    const int ct = max(split_candidate(lane, sh_longest), 1);
+    const float inv_ct = inv_of(ct);
+    SplitStat st{};
+    for (int r = warp; r < p.max_requests; r += NW) {
+      const ReqGeom g = one_pass ? geom_of(p, s_w[r], s_P[r], list) : req_geom(p, r, list);
+      if (g.nt > 0) add_request(st, g.nt, g.nfull * p.n_kv_heads, g.nunits, ct, inv_ct);
+    }
+    if (st.items) {
+      atomicAdd(&sh_stat[lane].work, st.work); atomicAdd(&sh_stat[lane].items, st.items);
+      atomicAdd(&sh_stat[lane].parts, st.parts); atomicMax(&sh_stat[lane].longest, st.longest);
+    }
+    __syncthreads();
+    if (tid < 32) {
+      const int chosen = best_candidate(sh_stat[lane], ct);
+      if (lane == 0) sh_rule = split_auto(sh_total, sh_units, chosen, p.min_chunk_tiles);
+    }
+  } else if (tid == 0) {
+    sh_rule = split_rule(sh_total, sh_units, p.target_items[list], p.min_chunk_tiles);
+  }
+  __syncthreads();
+  const SplitRule rule = sh_rule;
+  // phase 2 + 3: per-request bases (scan over up to T requests at a time), then the units of
+  // these requests
+  int unit_run = 0, part_run = 0, slot_run = 0, work_run = 0;
+  for (int r0 = 0; r0 < p.max_requests; r0 += T) {
+    const int r = r0 + tid;
+    ReqGeom g{};
+    if (one_pass) g = g0;
+    else if (r < p.max_requests) g = req_geom(p, r, list);
+    const int nunits = g.nt ? g.nunits : 0;
+    int pre[3], tot[3];
+    block_excl_scan<T, 3>({nunits * g.nt, nunits, g.w}, pre, tot, sh_scan);
+    const int wbase = work_run + pre[0];
+    const ReqSplit rs = req_split(rule, wbase, nunits, g.nt);
+    const int most = __reduce_max_sync(kAll, most_chunks(rs, nunits));
+    if (lane == 0) atomicMax(&sh_chunks, most);
+    int ppre[1], ptot[1];
+    block_excl_scan<T, 1>({rs.parts(nunits)}, ppre, ptot, sh_scan2);
+    s_ub[tid] = pre[1]; s_pb[tid] = part_run + ppre[0]; s_first[tid] = slot_run + pre[2]; s_wb[tid] = wbase;
+    if (!one_pass) { s_w[tid] = g.w; s_P[tid] = g.P; }
+    __syncthreads();
+    write_units(rule, r0, min(T, p.max_requests - r0), tot[1], unit_run, sh_chunks);
+    unit_run += tot[1]; part_run += ptot[0]; slot_run += tot[2]; work_run += tot[0];
+    __syncthreads();                      // the tables are overwritten next
+  }
+  write_items(unit_run, part_run, sh_total, rule.ct, sh_chunks);
 }
 
 template <int T>

@@ -147,3 +147,48 @@ def _plan_and_attention(wl, tunings, resident):
     # (2^-9 each) and the output once more
     err = float((outs[0] - outs[1]).norm() / outs[1].norm())
     assert err <= 4 * 2 ** -9, err
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n_requests,w,kv_heads,prefix", [
+    (1, 2, 8, 3001), (1, 3, 8, 28123), (8, 2, 4, 900), (9, 2, 4, 900), (37, 1, 4, 700), (37, 2, 4, 700), (38, 1, 8, 700),
+    (31, 3, 3, 2500), (33, 3, 3, 2500), (600, 1, 1, 300)])
+def test_list_holds_every_key_range_once(n_requests, w, kv_heads, prefix):
+    # one request (not sorted), few requests and many, 148 items and more, odd KV heads
+    tiles_per_slot, wmax, blocks = 1, 3, 8
+    ctx = B.Context(**_cfg(max_requests=n_requests, wmax=wmax, n_q_heads=4 * kv_heads, n_kv_heads=kv_heads, max_blocks=blocks,
+                           max_pages_per_req=450))
+    P = np.maximum(prefix - 64 * np.arange(n_requests), prefix // 2).astype(np.int32)
+    st = B.DeviceState.from_numpy(DEV, np.ones(n_requests, np.int32), P, np.zeros(n_requests, np.int32),
+                                  np.full(n_requests, w, np.int32), np.zeros((n_requests, blocks * 32), np.int32),
+                                  np.zeros((n_requests, wmax), np.uint8), np.zeros((n_requests, 450), np.int32))
+    pk, sb = B.PackBuffers.alloc(ctx, DEV), B.StepBuffers(ctx, DEV)
+    B.fb_pack_wavefronts(ctx, st, pk, sb.ws, sb.status)
+    torch.cuda.synchronize()
+    assert int(sb.status.item()) == 0
+    plan, ws = ctx.attn_plan(P, np.full(n_requests, w)), sb.ws.cpu().numpy()
+    n_items, n_units, _, n_parts, _, ticket, done, most = ws[:32].view(np.int32)
+    assert (n_units, n_items, n_parts) == (plan["units"], plan["items"], plan["parts"]) and ticket == done == 0
+    at = 256 + -(-plan["max_items"] * 32 // 256) * 256
+    items = ws[256:256 + 32 * n_items].view(np.int32).reshape(-1, 8)
+    units = ws[at:at + 64 * n_units].view(np.int32).reshape(-1, 16)
+    chunks, n_tiles, part_base = units[:, 7], units[:, 6], units[:, 10]
+    assert most == chunks.max() and (units[items[:, 0], 0] == items[:, 4]).all()
+    # every unit's key tiles once, in its pieces' order
+    order = np.lexsort((items[:, 1], items[:, 0]))
+    it, k = items[order], 0
+    for u in range(n_units):
+        own = it[k:k + chunks[u]]
+        k += chunks[u]
+        assert (own[:, 0] == u).all() and (own[:, 1] == np.arange(chunks[u])).all()
+        assert own[0, 2] == 0 and own[-1, 3] == n_tiles[u] and (own[1:, 2] == own[:-1, 3]).all() and (own[:, 3] > own[:, 2]).all()
+    assert k == n_items
+    # split units have places of their own for their pieces
+    assert (part_base[chunks <= 1] == -1).all()
+    split = np.argsort(part_base)[(chunks <= 1).sum():]
+    assert (part_base[split][1:] >= (part_base + chunks)[split][:-1]).all()
+    # every (slot, KV head) once, as tile A or B
+    tiles = [(u[2], u[1] & 0xffff, u[4]) for u in units] + [(u[3], u[1] >> 16, u[5]) for u in units if u[3] >= 0]
+    assert len(set(tiles)) == len(tiles) == n_requests * w * kv_heads * tiles_per_slot
+    if n_requests > 1:          # longest first
+        assert (np.diff(items[:, 3] - items[:, 2]) <= 1).all()
