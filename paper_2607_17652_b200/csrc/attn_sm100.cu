@@ -475,6 +475,8 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
             ++cntPA;
             tc_fence_after();
             issue_pv(0, sv, nks, j > 0);
+            // (its epilogue does not wait for tile B: from the last P to O 2,400 -> 1,000 cycles an item)
+            if (j + 1 == nA) commit(&o_full[0]);
           }
           if (j + 1 < nA) {
             tc_fence_after();
@@ -487,6 +489,7 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
             ++cntPB;
             tc_fence_after();
             issue_pv(1, sv, nks, j > 0);
+            if (j + 1 == nB) commit(&o_full[1]);
           }
           commit(&v_empty[sv]);
           if (j + 1 < nB) {
@@ -520,6 +523,7 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
             if (X) ++cntPB; else ++cntPA;
             tc_fence_after();
             issue_pv(X, X, pv_steps(g.limit(j, g.winA, p.resident)), j > 0);
+            if (j + 1 == n) commit(&o_full[X]);
             commit(&v_empty[X]);
             if (j + 1 < n) {
               // this stream's next K tile could only be requested when its last Q K^T had
@@ -533,9 +537,6 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
           }
         }
       }
-      if (!ok) break;
-      if (nA > 0) commit(&o_full[0]);
-      if (nB > 0) commit(&o_full[1]);
     }
   }
   } else {
@@ -688,7 +689,9 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
         const int y = kvh * p.group + row0 % p.group, z = rec[kRecSlot + X] * p.bl + rec[kRecT0 + X] + row0 / p.group;
         uint8_t* stage = sOut + (warp - 4) * kStageBytes;
         const float inv = out_scale / l;
-#pragma unroll
+        // (a loop: straight code that runs once an item is bound by fetching its instructions.  With O handed over
+        // tile by tile, steps in us: a toy request 21.5 -> 20.7, a 28,000-token one 81.7 -> 81.2, larger ones alike.)
+#pragma unroll 1
         for (int h = 0; h < NH; ++h) {
           uint32_t o[64];
           tmem_ld32(tO + h * 64, o);
@@ -713,7 +716,7 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
         // the reference the exponentials were taken against, and the sum (the merge divides by
         // it: the V scale goes in here)
         reinterpret_cast<float2*>(p.part_ml)[tile * kTileM + row] = make_float2(m_ref * sl2 - kShift, l / out_scale);
-#pragma unroll
+#pragma unroll 1
         for (int c = 0; c < D / 32; ++c) {
           uint32_t o[32];
           tmem_ld32(tO + c * 32, o);
