@@ -228,26 +228,30 @@ __device__ void build_sched(const PackParams& p, const int list) {
       const ReqGeom q = geom_of(p, s_w[k], s_P[k], list);
       const ReqSplit qs = req_split(rule, s_wb[k], q.nunits, q.nt);
       const int first = s_first[k], nc = qs.chunks(ul);
-      AttnUnit un[2];
+      // (records in registers: an array of them indexed in a loop lives in local memory)
+      AttnUnit un, un1;
       if (list == 0) {
-        un[0] = unit_record(q, r0 + k, first, ul);
+        un = unit_record(q, r0 + k, first, ul);
       } else {
         // quad qd of KV head h: tiles 4 qd + r and 4 qd + 2 + r belong to CTA r of the pair
         const int h = ul / q.nquad, qd = ul % q.nquad;
-        un[0] = make_unit(p, q, r0 + k, first, 4 * qd, 4 * qd + 2, h, h, inv_tps);
-        un[1] = make_unit(p, q, r0 + k, first, 4 * qd + 1, 4 * qd + 3, h, h, inv_tps);
+        un = make_unit(p, q, r0 + k, first, 4 * qd, 4 * qd + 2, h, h, inv_tps);
+        un1 = make_unit(p, q, r0 + k, first, 4 * qd + 1, 4 * qd + 3, h, h, inv_tps);
       }
       int nch = nc;
       const int pb = nc > 1 ? mult * (s_pb[k] + qs.part_off(ul)) : -1;
       // the workspace is sized for the bound on the split pieces (split_rule); a unit that
       // would still fall outside it is dropped and FB_ST_BAD_STATE is raised below
       if (nc > 1 && pb + mult * nc > max_parts) nch = 0;
-      int nvA = 0, nvB = 0;
-      for (int rr = 0; rr < mult; ++rr) {
-        un[rr].n_chunks = nch;
-        un[rr].part_base = nc > 1 ? pb + rr * nc : -1;
-        if (c0 == 0) units[mult * u + rr] = un[rr];
-        nvA = max(nvA, un[rr].nvisA); nvB = max(nvB, un[rr].nvisB);
+      int nvA = un.nvisA, nvB = un.nvisB;
+      un.n_chunks = nch;
+      un.part_base = nc > 1 ? pb : -1;
+      if (c0 == 0) units[mult * u] = un;
+      if (list == 1) {
+        un1.n_chunks = nch;
+        un1.part_base = nc > 1 ? pb + nc : -1;
+        if (c0 == 0) units[2 * u + 1] = un1;
+        nvA = max(nvA, un1.nvisA); nvB = max(nvB, un1.nvisB);
       }
       if (c0 == 0 && u < kUnitInfo) { s_info[u] = make_int4(nvA, nvB, q.nt, nch); s_req[u] = r0 + k; }
       const float inv = inv_of(nc);
