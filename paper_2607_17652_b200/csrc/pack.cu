@@ -15,6 +15,7 @@ namespace fb {
 // 6.6 / 7.6, 24 requests 8.6 / 8.0 / 8.9, 128 requests 19.0 / 16.9 / 17.2 (measured before build_sched got shorter).
 constexpr int kPackThreads = 512, kPackThreadsSmall = 256, kPackSmallRequests = 8;
 constexpr int kSlotsPerBlock = 32;
+constexpr int kPackLongPages = 1 << 20;   // (kLong: with two pages a key tile, ranges stay below 2^20 key tiles here)
 constexpr int kCostBins = 1024;
 constexpr int kUnitInfo = 1024;       // units whose geometry stays in shared memory between the two passes over items
 
@@ -99,9 +100,14 @@ __device__ __forceinline__ ReqGeom req_geom(const PackParams& p, int r, int list
 
 // a / d for 0 <= a, 0 < d with a quotient below 2^20: a reciprocal (inv_of(d)) off by a few units in the last
 // place puts the product within one of the quotient, the remainder says which way.  The list is built by
-// chains of such quotients; a hardware-less integer division is four times as long.
+// chains of such quotients; a hardware-less integer division is four times as long.  Quotients that count key
+// tiles may be larger where a page table reaches that far: there the estimate is off by several (up to four at
+// 2^24), and kLong divides.  (Divided in here whenever the estimate is large, the code of the division alone
+// costs ordinary lists 0.3 to 0.7 us; as a kernel of its own, nothing.)
 __device__ __forceinline__ float inv_of(int d) { return __fdividef(1.0f, (float)d); }
+template <bool kLong = false>
 __device__ __forceinline__ int quot(int a, int d, float inv) {
+  if (kLong) return a / d;
   const int q = (int)((float)a * inv), r = a - q * d;
   return q + (r >= d) - (r < 0);
 }
@@ -142,7 +148,7 @@ __device__ __forceinline__ AttnUnit make_unit(const PackParams& p, const ReqGeom
 // this and the quotients by reciprocal: one request of 3,000 tokens 5.7 / 4.2, 8 requests 6.1 / 5.4, 24 requests
 // 8.2 / 7.7, 64 requests 9.7 to 11 / 8.2 to 9.4, in 8 bits 10 to 13 / 8.8, 128 requests 14 to 18 / 12.4 to 16.
 // Steps: a toy request 23.3 / 21.3, one request with four layers 110.1 / 107.5, a 28,000-token one 83.2 / 82.2.
-template <int T>
+template <int T, bool kLong>
 __device__ void build_sched(const PackParams& p, const int list) {
   constexpr unsigned kAll = 0xffffffffu;
   constexpr int NW = T / 32;
@@ -199,7 +205,7 @@ __device__ void build_sched(const PackParams& p, const int list) {
         un.part_base = nc > 1 ? i : -1;
         units[u] = un;
       }
-      AttnItem it; it.unit = u; it.chunk = c; it.jb = quot(c * q.nt, nc, inv); it.je = quot((c + 1) * q.nt, nc, inv);
+      AttnItem it; it.unit = u; it.chunk = c; it.jb = quot<kLong>(c * q.nt, nc, inv); it.je = quot<kLong>((c + 1) * q.nt, nc, inv);
       it.req = k; it.pad[0] = it.pad[1] = it.pad[2] = 0;
       items[i] = it;
     }
@@ -256,7 +262,7 @@ __device__ void build_sched(const PackParams& p, const int list) {
       if (c0 == 0 && u < kUnitInfo) { s_info[u] = make_int4(nvA, nvB, q.nt, nch); s_req[u] = r0 + k; }
       const float inv = inv_of(nc);
       for (int c = c0; c < nch; c += 1 << shift) {
-        const int jb = quot(c * q.nt, nc, inv), je = quot((c + 1) * q.nt, nc, inv);
+        const int jb = quot<kLong>(c * q.nt, nc, inv), je = quot<kLong>((c + 1) * q.nt, nc, inv);
         const int cost = item_cost(max(0, min(je, nvA) - jb), max(0, min(je, nvB) - jb));
         atomicAdd(&bins[min(cost, kCostBins - 1)], 1);
       }
@@ -295,7 +301,7 @@ __device__ void build_sched(const PackParams& p, const int list) {
       }
       const float inv = inv_of(max(nch, 1));
       for (int c = j & ((1 << shift) - 1); c < nch; c += 1 << shift) {
-        const int jb = quot(c * nt, nch, inv), je = quot((c + 1) * nt, nch, inv);
+        const int jb = quot<kLong>(c * nt, nch, inv), je = quot<kLong>((c + 1) * nt, nch, inv);
         const int cost = item_cost(max(0, min(je, nvA) - jb), max(0, min(je, nvB) - jb));
         const int at = atomicAdd(&bins[min(cost, kCostBins - 1)], 1);
         if (at < max_items) {
@@ -317,7 +323,7 @@ __device__ void build_sched(const PackParams& p, const int list) {
     return __shfl_sync(kAll, ct, __ffs(__ballot_sync(kAll, mine == least)) - 1);
   };
   auto add_request = [&](SplitStat& st, int nt, int pairs, int nunits, int ct, float inv_ct) {
-    const int nch = quot(nt + ct - 1, ct, inv_ct), len = quot(nt + nch - 1, nch, inv_of(nch));
+    const int nch = quot(nt + ct - 1, ct, inv_ct), len = quot<kLong>(nt + nch - 1, nch, inv_of(nch));
     split_stat_add_pieces(st, nt, pairs, nunits, nch, len);
   };
 
@@ -455,13 +461,13 @@ __device__ void build_sched(const PackParams& p, const int list) {
   write_items(unit_run, part_run, sh_total, rule.ct, sh_chunks);
 }
 
-template <int T>
+template <int T, bool kLong>
 __global__ void __launch_bounds__(T) pack_kernel(const PackParams p) {
   // Not followed early: the attention's CTAs, which take an SM each, would move in while the list is
   // still being built.  Steps with and without that, in us: one request with four layers 105 -> 102,
   // 28,000 tokens 83 -> 81, 8 requests 79 -> 77.5, 24 requests 311.5 -> 308.5.
   pdl_wait_only();
-  if ((int)blockIdx.x >= p.n_gather_blocks) { build_sched<T>(p, (int)blockIdx.x - p.n_gather_blocks); return; }
+  if ((int)blockIdx.x >= p.n_gather_blocks) { build_sched<T, kLong>(p, (int)blockIdx.x - p.n_gather_blocks); return; }
   __shared__ int sh_scan[T / 32];
   __shared__ int s_req[kSlotsPerBlock], s_idx[kSlotsPerBlock], s_w[kSlotsPerBlock];
   const int tid = threadIdx.x;
@@ -545,10 +551,12 @@ int launch_pack(fb_ctx* ctx, const fb_state* st, const fb_pack* out, void* ws, i
   p.n_gather_blocks = (p.max_slots + kSlotsPerBlock - 1) / kSlotsPerBlock;
   // one more block per work list in use (the CTA-pair kernel's list only when that kernel is on)
   const int grid = p.n_gather_blocks + 1 + (p.pair_on ? 1 : 0);
-  return cuda_err(ctx, p.max_requests <= kPackSmallRequests
-                           ? launch_pdl(pack_kernel<kPackThreadsSmall>, grid, kPackThreadsSmall, 0, stream, p)
-                           : launch_pdl(pack_kernel<kPackThreads>, grid, kPackThreads, 0, stream, p),
-                  "pack_kernel launch");
+  // (a prefix that its row of the page table does not hold is a bad state, reported by the attention)
+  const bool small = p.max_requests <= kPackSmallRequests, far = c.max_pages_per_req >= kPackLongPages;
+  const int threads = small ? kPackThreadsSmall : kPackThreads;
+  auto* const kernel = small ? (far ? pack_kernel<kPackThreadsSmall, true> : pack_kernel<kPackThreadsSmall, false>)
+                             : (far ? pack_kernel<kPackThreads, true> : pack_kernel<kPackThreads, false>);
+  return cuda_err(ctx, launch_pdl(kernel, grid, threads, 0, stream, p), "pack_kernel launch");
 }
 
 }  // namespace fb

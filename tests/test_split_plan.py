@@ -192,3 +192,31 @@ def test_list_holds_every_key_range_once(n_requests, w, kv_heads, prefix):
     assert len(set(tiles)) == len(tiles) == n_requests * w * kv_heads * tiles_per_slot
     if n_requests > 1:          # longest first
         assert (np.diff(items[:, 3] - items[:, 2]) <= 1).all()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("max_requests", [1, 2, 9])
+@pytest.mark.parametrize("tiles", [(1 << 19) - 2, (1 << 19) - 1, (1 << 20) + 5, 11423809, 13823826, 16777000])
+def test_cuts_of_a_very_long_range(max_requests, tiles):
+    # quotients on both sides of the 2^20 up to which they are taken by reciprocal, and near the largest prefix
+    # (the call reads neither the pages nor the page table)
+    ctx = B.Context(**_cfg(max_requests=max_requests, wmax=1, block_len=64, n_q_heads=2, n_kv_heads=1, head_dim=64, max_blocks=2,
+                           max_pages_per_req=2 * tiles + 2))
+    P = np.zeros(max_requests, np.int32)
+    w = np.zeros(max_requests, np.int32)
+    P[-1], w[-1] = 128 * tiles, 1
+    st = B.DeviceState.from_numpy(DEV, np.ones(max_requests, np.int32), P, np.zeros(max_requests, np.int32), w,
+                                  np.zeros((max_requests, 2 * 64), np.int32), np.zeros((max_requests, 1), np.uint8),
+                                  np.zeros((max_requests, 4), np.int32))
+    pk, sb = B.PackBuffers.alloc(ctx, DEV), B.StepBuffers(ctx, DEV)
+    B.fb_pack_wavefronts(ctx, st, pk, sb.ws, sb.status)
+    torch.cuda.synchronize()
+    assert int(sb.status.item()) == 0
+    plan, ws = ctx.attn_plan(P, w), sb.ws.cpu().numpy()
+    n_items, n_units, _, n_parts = ws[:16].view(np.int32)
+    assert (n_units, n_items, n_parts) == (plan["units"], plan["items"], plan["parts"]) and n_items > 1
+    items = ws[256:256 + 32 * n_items].view(np.int32).reshape(-1, 8)
+    items = items[np.argsort(items[:, 1])]
+    edges = np.arange(n_items + 1, dtype=np.int64) * (tiles + 1) // n_items
+    assert (items[:, 1] == np.arange(n_items)).all()
+    assert (items[:, 2] == edges[:-1]).all() and (items[:, 3] == edges[1:]).all()
