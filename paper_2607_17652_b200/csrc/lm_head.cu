@@ -21,18 +21,19 @@
 // operations as 48 KB before, six stages fit, and a CTA reads 8 KB instead of 12 KB of shared memory
 // per MMA.  What bounds the product is the board's power limit, which is where the saved traffic shows:
 // a step of 64 requests (5,120 rows, V = 151,552, hidden 2048), back to back, 2832 -> 2657 us.
-// Where which one runs: see lm_pairs (on the device, by live rows) and launch_lm_head.
+// Where which one runs: see lm_pairs in lm_forms.h (on the device, by live rows) and launch_lm_head.
 #include <cudaTypedefs.h>
 
 #include <cfloat>
 
 #include "fb_common.cuh"
+#include "lm_forms.h"
 #include "ptx_sm100.cuh"
 
 namespace fb {
 
 constexpr int kLmThreads = 256;
-constexpr int kLmBM = 128, kLmBN = 256, kLmBK = 64, kLmStages = 4;
+constexpr int kLmBK = 64, kLmStages = 4;
 constexpr int kLmABytes = kLmBM * kLmBK * 2, kLmBBytes = kLmBN * kLmBK * 2;
 constexpr int kLmStageBytes = kLmABytes + kLmBBytes;                 // 48 KB
 constexpr int kLmPairStages = 6, kLmPairStageBytes = kLmABytes + kLmBBytes / 2;   // 32 KB a CTA
@@ -44,7 +45,7 @@ struct LmParams {
   const int32_t* n_live;
   float4* part;          // [n_tiles_n][rows_pad] (max, sum exp, first index of the max as bits, -)
   int32_t* status;
-  int32_t bl, vocab, hidden, n_tiles_n, rows_pad;
+  int32_t bl, vocab, hidden, n_tiles_n, rows_pad, sms;
   int32_t pair;          // both forms are launched, lm_pairs says which one works
   long long wait_cycles;
 };
@@ -84,16 +85,6 @@ __device__ __forceinline__ void absorb32(const uint32_t* v, int col, float& mx, 
   sum += t.x + t.y;
 }
 
-// Row tiles two by two?  An odd one out leaves half of a pair idle for a whole tile.  Call in us at V = 151,552,
-// one CTA a tile / pairs, an even number of row tiles:
-//   hidden 1024:  4 tiles 136 / 122    8 234 / 207   14 400 / 361   20 570 / 537
-//   hidden 2048:  4 tiles 235 / 209    8 421 / 387   14 772 / 715   20 1128 / 1086
-//   hidden 4096:  4 tiles 484 / 442    8 968 / 865
-// 13 tiles, the last pair half empty: 364 / 347 (hidden 1024), 735 / 694 (2048), 1491 / 1477 (4096); at 7 tiles a
-// pair form that takes as long as for 8 would lose.
-constexpr int kLmPairOddTiles = 13;
-__device__ __forceinline__ bool lm_pairs(int m_tiles) { return m_tiles >= 2 && ((m_tiles & 1) == 0 || m_tiles >= kLmPairOddTiles); }
-
 template <bool kPair>
 __global__ void __launch_bounds__(kLmThreads, 1)
 lm_head_stats_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW,
@@ -102,7 +93,7 @@ lm_head_stats_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
   pdl_wait_only();
   const int live_rows = *p.n_live * p.bl;
   const int m_tiles = (live_rows + kLmBM - 1) / kLmBM;          // row tiles that hold live rows
-  if (p.pair && lm_pairs(m_tiles) != kPair) return;             // (the whole grid)
+  if (p.pair && lm_pairs(m_tiles, p.n_tiles_n, p.hidden, p.sms) != kPair) return;             // (the whole grid)
   extern __shared__ uint8_t smem_raw[];
   // (a pair's CTAs lay their shared memory out alike: the MMA's descriptors are offsets in both)
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -378,6 +369,7 @@ int launch_lm_head(fb_ctx* ctx, const fb_pack* pk, const void* x, const void* w,
   p.bl = c.block_len; p.vocab = c.vocab; p.hidden = hidden;
   p.n_tiles_n = (c.vocab + kLmBN - 1) / kLmBN;
   p.rows_pad = lm_rows_pad(c);
+  p.sms = ctx->num_sms;
   p.wait_cycles = ctx->wait_cycles;
   // Both forms are launched, since the live rows are only known on the device; the one that is not wanted costs
   // 2 us.  So not for small calls (three row tiles: 112 us + 2), and not below 768 hidden elements, where the

@@ -1,0 +1,33 @@
+"""Which form of the LM head's product runs: the rules of csrc/lm_forms.h, compiled on their own."""
+import ctypes
+import os
+import subprocess
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2607_17652_b200", "csrc")
+SMS = 148
+
+
+@pytest.fixture(scope="module")
+def rules(tmp_path_factory):
+    d = tmp_path_factory.mktemp("lm_forms")
+    (d / "r.cc").write_text('#include "lm_forms.h"\n'
+                            'extern "C" int pairs(int m, int n, int hidden, int sms) { return fb::lm_pairs(m, n, hidden, sms); }\n')
+    subprocess.run(["g++", "-std=c++17", "-shared", "-fPIC", "-I", CSRC, str(d / "r.cc"), "-o", str(d / "r.so")], check=True)
+    return ctypes.CDLL(str(d / "r.so"))
+
+
+# (row tiles, vocabulary tiles, hidden): measured faster that way
+@pytest.mark.parametrize("m,n,hidden,form", [
+    (0, 592, 2048, 0), (1, 592, 2048, 0), (2, 592, 2048, 1), (3, 592, 2048, 0), (5, 592, 1024, 0), (7, 592, 4096, 0), (11, 592, 1024, 1),
+    (13, 592, 2048, 1), (16, 592, 1024, 1), (40, 592, 2048, 1), (41, 592, 2048, 1), (16, 592, 768, 1), (11, 592, 768, 0), (13, 592, 768, 0),
+    (13, 91, 4096, 0), (11, 91, 4096, 0), (5, 91, 4096, 1), (1, 64, 2048, 0), (3, 64, 2048, 1), (7, 64, 2048, 1), (9, 64, 2048, 0),
+    (131072, 1 << 23, 4096, 1)])
+def test_form_by_rounds(rules, m, n, hidden, form):
+    assert rules.pairs(m, n, hidden, SMS) == form
+
+
+# the live row tiles that test_gpu_lm_pair.py runs at 297 vocabulary tiles
+def test_forms_of_the_gpu_test(rules):
+    assert [rules.pairs(m, 297, 768, SMS) for m in (1, 2, 3, 4, 13, 16)] == [0, 1, 0, 1, 0, 1]
