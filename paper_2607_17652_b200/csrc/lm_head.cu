@@ -21,7 +21,7 @@
 // operations as 48 KB before, six stages fit, and a CTA reads 8 KB instead of 12 KB of shared memory
 // per MMA.  What bounds the product is the board's power limit, which is where the saved traffic shows:
 // a step of 64 requests (5,120 rows, V = 151,552, hidden 2048), back to back, 2832 -> 2657 us.
-// Where which one runs: see lm_pairs in lm_forms.h (on the device, by live rows) and launch_lm_head.
+// Where which one runs: lm_forms.h, by what the context can hold on the host and by the live rows on the device.
 #include <cudaTypedefs.h>
 
 #include <cfloat>
@@ -45,8 +45,9 @@ struct LmParams {
   const int32_t* n_live;
   float4* part;          // [n_tiles_n][rows_pad] (max, sum exp, first index of the max as bits, -)
   int32_t* status;
-  int32_t bl, vocab, hidden, n_tiles_n, rows_pad, sms;
-  int32_t pair;          // both forms are launched, lm_pairs says which one works
+  int32_t bl, vocab, hidden, n_tiles_n, rows_pad;
+  int32_t both;          // both forms are launched ...
+  unsigned long long pairs_mask;   // ... and lm_pairs_of says which one works
   long long wait_cycles;
 };
 
@@ -90,10 +91,19 @@ __global__ void __launch_bounds__(kLmThreads, 1)
 lm_head_stats_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW,
                      const LmParams p) {
   constexpr int kStages = kPair ? kLmPairStages : kLmStages, kStageBytes = kPair ? kLmPairStageBytes : kLmStageBytes;
-  pdl_wait_only();
-  const int live_rows = *p.n_live * p.bl;
+  // Where both forms are launched, the pairs' grid comes second.  It is started when the first one is through (turned
+  // down), or from its first moment on (at work: the CTAs find room as the first one's leave, and what is turned down is
+  // gone when that ends).  Either way the first has waited for everything older, so the pairs may read n_live (past the
+  // L1) ahead of their own wait.  Turned down, they let the merge start, and one CTA waits for the first grid all the
+  // same: the merge waits for this grid alone.
+  const bool second = p.both && kPair;
+  if (!second) pdl_wait_only();
+  const int live_rows = __ldcg(p.n_live) * p.bl;
   const int m_tiles = (live_rows + kLmBM - 1) / kLmBM;          // row tiles that hold live rows
-  if (p.pair && lm_pairs(m_tiles, p.n_tiles_n, p.hidden, p.sms) != kPair) return;             // (the whole grid)
+  const bool wanted = !p.both || lm_pairs_of(p.pairs_mask, m_tiles) == kPair;
+  if (p.both && wanted != kPair) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (second && (wanted || blockIdx.x == 0)) pdl_wait_only();
+  if (!wanted) return;                                          // (the whole grid)
   extern __shared__ uint8_t smem_raw[];
   // (a pair's CTAs lay their shared memory out alike: the MMA's descriptors are offsets in both)
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -339,7 +349,7 @@ int launch_lm_head(fb_ctx* ctx, const fb_pack* pk, const void* x, const void* w,
   const fb_config& c = ctx->cfg;
   const int rows = c.max_requests * c.wmax * c.block_len;
   auto fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled>(ctx->encode_fn);
-  CUtensorMap tmX, tmW, tmWHalf;
+  CUtensorMap tmX, tmW;
   const cuuint32_t es[2] = {1, 1};
   {
     const cuuint64_t dims[2] = {(cuuint64_t)hidden, (cuuint64_t)rows};
@@ -350,18 +360,17 @@ int launch_lm_head(fb_ctx* ctx, const fb_pack* pk, const void* x, const void* w,
            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
       return set_err(ctx, FB_ERR_CUDA, "cuTensorMapEncodeTiled failed for x");
   }
-  {
+  auto encode_w = [&](CUtensorMap& map, cuuint32_t box_rows) {
     const cuuint64_t dims[2] = {(cuuint64_t)hidden, (cuuint64_t)c.vocab};
     const cuuint64_t str[1] = {(cuuint64_t)hidden * 2};
-    const cuuint32_t box[2] = {kLmBK, kLmBN}, half[2] = {kLmBK, kLmBN / 2};
-    if (fn(&tmW, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(w), dims, str, box, es,
-           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS ||
-        fn(&tmWHalf, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(w), dims, str, half, es,
+    const cuuint32_t box[2] = {kLmBK, box_rows};
+    if (fn(&map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(w), dims, str, box, es,
            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
       return set_err(ctx, FB_ERR_CUDA, "cuTensorMapEncodeTiled failed for w");
-  }
+    return (int)FB_OK;
+  };
+  if (int e = encode_w(tmW, kLmBN)) return e;
   LmParams p;
   p.n_live = pk->n_live;
   p.part = static_cast<float4*>(ws);
@@ -369,20 +378,20 @@ int launch_lm_head(fb_ctx* ctx, const fb_pack* pk, const void* x, const void* w,
   p.bl = c.block_len; p.vocab = c.vocab; p.hidden = hidden;
   p.n_tiles_n = (c.vocab + kLmBN - 1) / kLmBN;
   p.rows_pad = lm_rows_pad(c);
-  p.sms = ctx->num_sms;
   p.wait_cycles = ctx->wait_cycles;
-  // Both forms are launched, since the live rows are only known on the device; the one that is not wanted costs
-  // 2 us.  So not for small calls (three row tiles: 112 us + 2), and not below 768 hidden elements, where the
-  // epilogue bounds a tile and pairs gain nothing (hidden 512: 4 tiles 91 / 96, 20 tiles 355 / 357).
-  const int most_tiles = (rows + kLmBM - 1) / kLmBM;
-  p.pair = most_tiles >= 4 && hidden >= 768 && (long long)most_tiles * p.n_tiles_n >= 8ll * ctx->num_sms;
-  if (p.pair)
-    if (int e = cuda_err(ctx, launch_pdl_cluster(lm_head_stats_kernel<true>, ctx->num_sms / 2 * 2, kLmThreads, kLmSmem, stream, 2,
-                                                 tmX, tmWHalf, p), "lm_head_stats_kernel (pairs) launch"))
-      return e;
+  // (both forms, since the live rows are only known on the device)
+  p.both = lm_both_forms((rows + kLmBM - 1) / kLmBM, p.n_tiles_n, hidden, ctx->num_sms);
+  p.pairs_mask = lm_pairs_mask(p.n_tiles_n, hidden, ctx->num_sms);
   if (int e = cuda_err(ctx, launch_pdl(lm_head_stats_kernel<false>, ctx->num_sms, kLmThreads, kLmSmem, stream, tmX, tmW, p),
                        "lm_head_stats_kernel launch"))
     return e;
+  if (p.both) {
+    CUtensorMap tmWHalf;
+    if (int e = encode_w(tmWHalf, kLmBN / 2)) return e;
+    if (int e = cuda_err(ctx, launch_pdl_cluster(lm_head_stats_kernel<true>, ctx->num_sms / 2 * 2, kLmThreads, kLmSmem, stream, 2,
+                                                 tmX, tmWHalf, p), "lm_head_stats_kernel (pairs) launch"))
+      return e;
+  }
   if (int e = cuda_err(ctx, launch_pdl(lm_head_merge_kernel, (rows + 31) / 32, 32 * kLmMergeWarps, 0, stream, p, argmax, conf, rows),
                        "lm_head_merge_kernel launch"))
     return e;
