@@ -68,3 +68,104 @@ def test_lm_head_row_tiles_in_pairs(head, blocks):
     am, cf = sb.argmax.cpu().numpy(), sb.conf.cpu().numpy()
     assert ((am[:rows] >= 0) & (am[:rows] < V)).all() and ((cf[:rows] > 0) & (cf[:rows] <= 1)).all()
     assert (am[rows:] == -1).all() and not cf[rows:].any()
+
+
+# ---- all rows, bit for bit, against the one-CTA form (which form runs where: test_lm_forms.py)
+class Head:
+    def __init__(self, requests, vocab):
+        self.ctx = B.Context(max_requests=requests, wmax=WMAX, block_len=BL, n_q_heads=4, n_kv_heads=1, head_dim=64, page_size=64,
+                             num_pages=8, max_pages_per_req=4, vocab=vocab, mask_id=vocab - 1, eos_id=vocab - 2, max_blocks=8, s_pe=1,
+                             tau_mask=0.9, tau_edit=0.95, theta_spawn=0.5, sm_scale=0.0)
+        self.requests, self.rows = requests, requests * WMAX * BL
+        self.ws = torch.zeros(B.lib().fb_lm_head_workspace_bytes(self.ctx.handle), dtype=torch.uint8, device=DEV)
+
+    def run(self, x, w, blocks):
+        """`x`: as many rows as the context holds.  (argmax, conf, status, action, state)"""
+        live = np.array([min(WMAX, max(0, blocks - WMAX * r)) for r in range(self.requests)], np.int32)
+        n, z = self.requests, np.zeros
+        tokens = np.full((n, 8 * BL), self.ctx.cfg.mask_id, np.int32)
+        st = B.DeviceState.from_numpy(DEV, np.ones(n, np.int32), z(n, np.int32), z(n, np.int32), live, tokens,
+                                      z((n, WMAX), np.uint8), z((n, 4), np.int32))
+        pk, sb = B.PackBuffers.alloc(self.ctx, DEV), B.StepBuffers(self.ctx, DEV)
+        B.fb_pack_wavefronts(self.ctx, st, pk, sb.ws, sb.status)
+        B.fb_lm_head_t2t(self.ctx, pk, x, w, st, sb.argmax, sb.conf, sb.action, sb.slot_stats, self.ws, sb.status)
+        torch.cuda.synchronize()
+        return sb.argmax, sb.conf, int(sb.status.item()), sb.action, st
+
+
+def one_cta(x, w, blocks):
+    """The same rows three row tiles at a time: contexts of that size launch the one-CTA form alone."""
+    h, out = Head(3, w.shape[0]), []
+    for r0 in range(0, blocks * BL, h.rows):
+        part = torch.zeros((h.rows, x.shape[1]), dtype=x.dtype, device=DEV)
+        own = x[r0:min(r0 + h.rows, blocks * BL)]
+        part[:len(own)] = own
+        a, c, status, action, _ = h.run(part, w, len(own) // BL)
+        assert status == 0
+        out.append((a[:len(own)], c[:len(own)], action[:len(own)]))
+    return [torch.cat(t) for t in zip(*out)]
+
+
+def draw(hidden, vocab, rows, seed):
+    g = torch.Generator(device=DEV)
+    g.manual_seed(seed)
+    w = torch.randn((vocab, hidden), device=DEV, dtype=torch.bfloat16, generator=g).mul_(hidden ** -0.5)
+    x = torch.randn((rows, hidden), device=DEV, dtype=torch.bfloat16, generator=g)
+    x[::2] += 4 * w[torch.randint(0, vocab - 2, (rows // 2,), device=DEV, generator=g)]     # (half of the rows with a winner)
+    return x, w
+
+
+# live blocks (row tiles, form): 8 (2, pairs), 13 (4, pairs, ragged), 20 (5, one CTA a tile), 49 (13, pairs, half of the last one idle,
+# ragged; hidden 768: one CTA a tile), 64 (16, pairs)
+@pytest.mark.parametrize("hidden", [768, 1088, 2048])
+def test_pairs_give_the_one_cta_forms_bits(hidden):
+    x, w = draw(hidden, V, REQUESTS * WMAX * BL, hidden)
+    h = Head(REQUESTS, V)
+    for blocks in (8, 13, 20, 49, 64):
+        rows = blocks * BL
+        a, c, status, action, _ = h.run(x, w, blocks)
+        a1, c1, action1 = one_cta(x, w, blocks)
+        assert status == 0 and bool((a[rows:] == -1).all()) and not bool(c[rows:].any())
+        assert torch.equal(a[:rows], a1) and torch.equal(c[:rows], c1) and torch.equal(action[:rows], action1), blocks
+
+
+# rows of W that are NaN: single ones, in either half of a pair's slice, a whole slice, the last columns; behind -inf
+@pytest.mark.parametrize("first,last,minus_inf", [(0, 1, 0), (127, 129, 0), (200, 201, 0), (256, 512, 0), (V - 8, V, 0), (160, 161, 160)])
+def test_pairs_report_nan(first, last, minus_inf):
+    x, w = draw(HIDDEN, V, REQUESTS * WMAX * BL, 3)
+    x = x.abs() + 0.5                       # (a weight of -inf gives a logit of -inf)
+    w[:minus_inf] = -float("inf")
+    w[first:last] = float("nan")
+    a, c, status, action, st = Head(REQUESTS, V).run(x, w, 64)
+    assert status & B.FB_ST_NAN_LOGIT
+    assert float(c.abs().max()) == 0.0 and int(action.max()) == 0 and bool((st.tokens == V - 1).all())
+
+
+def test_pairs_certain_rows():
+    """One logit far above the rest, up to where nothing else shows in 32 bits: every row revealed, its confidence within
+    4e-6 of 1 / (1 + (V - 1) e^-d) (at most 60 additions of 2^-24 behind the term 1)."""
+    rows, top = REQUESTS * WMAX * BL, V // 2 + 200
+    d = torch.tensor([20.0, 26.5, 30.0, 38.0, 43.0, 50.0, 71.0, 1000.0], dtype=torch.float64)
+    x, w = torch.zeros(rows, HIDDEN, dtype=torch.bfloat16), torch.zeros(V, HIDDEN, dtype=torch.bfloat16)
+    x[:, 0], x[:, 1] = 1.0, d.to(torch.bfloat16).repeat(rows // 8)
+    w[:, 0], w[top, 1] = -10.0, 1.0
+    a, c, status, action, st = Head(REQUESTS, V).run(x.to(DEV), w.to(DEV), 64)
+    want = (1 / (1 + (V - 1) * torch.exp(-d))).repeat(rows // 8)
+    assert status == 0 and bool((a == top).all()) and bool((action == O.ACT_M2T).all())
+    assert float((c.cpu().double() - want).abs().max()) <= 4e-6 and float(c.max()) <= 1.0
+
+
+def test_pairs_give_up_report_and_recover():
+    """Every wait gives up at once (no spinning), as in test_gpu_giveup.py: the launch ends by itself, says so, and the
+    same context computes the same bits as before afterwards."""
+    x, w = draw(HIDDEN, V, REQUESTS * WMAX * BL, 4)
+    h = Head(REQUESTS, V)
+    h.ctx.set_tuning(wait_cycles=-1)
+    for blocks in (8, 64):
+        assert h.run(x, w, blocks)[2] & B.FB_ST_DEV_TIMEOUT
+    h.ctx.set_tuning()
+    for blocks in (8, 64):
+        a, c, status, action, _ = h.run(x, w, blocks)
+        a1, c1, action1 = one_cta(x, w, blocks)
+        rows = blocks * BL
+        assert status == 0 and torch.equal(a[:rows], a1) and torch.equal(c[:rows], c1) and torch.equal(action[:rows], action1)

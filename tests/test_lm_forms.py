@@ -48,6 +48,10 @@ def test_both_forms_only_where_pairs_can_pay(rules, most, n, hidden, both):
     assert rules.both(most, n, hidden, SMS) == both
 
 
-# the live row tiles that test_gpu_lm_pair.py runs at 297 vocabulary tiles
+# the live row tiles that test_gpu_lm_pair.py runs at 297 vocabulary tiles and 16 row tiles of capacity, and the contexts that it
+# takes for the one-CTA form
 def test_forms_of_the_gpu_test(rules):
-    assert rules.both(16, 297, 768, SMS) and [rules.masked(m, 297, 768, SMS) for m in (1, 2, 3, 4, 13, 16)] == [0, 1, 0, 1, 0, 1]
+    tiles = (1, 2, 3, 4, 5, 13, 16)
+    assert rules.both(16, 297, 768, SMS) and not rules.both(3, 297, 2048, SMS)
+    assert [rules.masked(m, 297, 768, SMS) for m in tiles] == [0, 1, 0, 1, 0, 0, 1]
+    assert all([rules.masked(m, 297, h, SMS) for m in tiles] == [0, 1, 0, 1, 0, 1, 1] for h in (1088, 2048))
