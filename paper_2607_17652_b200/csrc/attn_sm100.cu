@@ -475,12 +475,14 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
             ++cntPA;
             tc_fence_after();
             issue_pv(0, sv, nks, j > 0);
-            // (its epilogue does not wait for tile B: from the last P to O 2,400 -> 1,000 cycles an item)
-            if (j + 1 == nA) commit(&o_full[0]);
           }
           if (j + 1 < nA) {
             tc_fence_after();
             issue_qk(0, st1, round16(g.limit(j + 1, g.winA, p.resident)));
+          } else if (j + 1 == nA) {
+            // its epilogue does not wait for tile B.  (In the branch that only the last key tile takes: a test of its
+            // own between P V and the next Q K^T costs 8-bit pages 1 % of long items.)
+            commit(&o_full[0]);
           }
           // tile B
           if (j < nB) {
@@ -489,12 +491,13 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
             ++cntPB;
             tc_fence_after();
             issue_pv(1, sv, nks, j > 0);
-            if (j + 1 == nB) commit(&o_full[1]);
           }
           commit(&v_empty[sv]);
           if (j + 1 < nB) {
             tc_fence_after();
             issue_qk(1, st1, round16(g.limit(j + 1, g.winB, p.resident)));
+          } else if (j + 1 == nB) {
+            commit(&o_full[1]);
           }
           if (j + 1 < n) {
             commit(&k_empty[st1]);
@@ -523,7 +526,6 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
             if (X) ++cntPB; else ++cntPA;
             tc_fence_after();
             issue_pv(X, X, pv_steps(g.limit(j, g.winA, p.resident)), j > 0);
-            if (j + 1 == n) commit(&o_full[X]);
             commit(&v_empty[X]);
             if (j + 1 < n) {
               // this stream's next K tile could only be requested when its last Q K^T had
@@ -533,6 +535,8 @@ wavefront_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
               issue_qk(X, X, round16(g.limit(j + 1, g.winA, p.resident)));
               commit(&k_empty[X]);
               if (j + 2 == n && X == 1) commit(q_empty);
+            } else {
+              commit(&o_full[X]);
             }
           }
         }
