@@ -194,6 +194,68 @@ def test_list_holds_every_key_range_once(n_requests, w, kv_heads, prefix):
         assert (np.diff(items[:, 3] - items[:, 2]) <= 1).all()
 
 
+
+# windows and whether a request is decoding; one request with work among many rows, few and many, odd KV heads, requests without
+# units between others, blocks of one and two Q tiles, the window beside the pages and in them
+@pytest.mark.gpu
+@pytest.mark.parametrize("resident", [0, 1])
+@pytest.mark.parametrize("block_len,kv_heads,windows,prefix", [
+    (32, 8, [0, 0, 0, 0, 0, 2, 0, 0], 3001), (64, 3, [-3, 0, 0, 1], 9000), (32, 4, [0, 3, 0, 0, -2, 0, 1, 0], 5000),
+    (64, 8, [1, 0, 3, 2, 0, 0, 3, 1], 1500), (32, 1, [0] * 7 + [3], 300), (32, 3, [0] * 20 + [2], 4000),
+    (64, 3, [0, 1, 2, 3, -1] * 6, 2500), (32, 5, [3, 0, 0, 1] * 150, 700), (32, 8, [0] * 8, 500), (32, 8, [0] * 9, 500)])
+def test_list_of_a_mixed_batch(resident, block_len, kv_heads, windows, prefix):
+    n, wmax, blocks, G = len(windows), 3, 8, 4
+    ctx = B.Context(**_cfg(max_requests=n, wmax=wmax, block_len=block_len, n_q_heads=G * kv_heads, n_kv_heads=kv_heads,
+                           max_blocks=blocks, max_pages_per_req=160, window_in_pages=resident))
+    rg = np.random.default_rng(n * block_len + kv_heads)
+    P, w = rg.integers(prefix // 3, prefix + 1, n).astype(np.int32), np.abs(windows).astype(np.int32)
+    st = B.DeviceState.from_numpy(DEV, np.array([x >= 0 for x in windows], np.int32), P, np.zeros(n, np.int32), w,
+                                  np.zeros((n, blocks * block_len), np.int32), np.zeros((n, wmax), np.uint8),
+                                  np.zeros((n, 160), np.int32))
+    w = np.maximum(windows, 0)                       # (a request that is not decoding has no window)
+    pk, sb = B.PackBuffers.alloc(ctx, DEV), B.StepBuffers(ctx, DEV)
+    B.fb_pack_wavefronts(ctx, st, pk, sb.ws, sb.status)
+    torch.cuda.synchronize()
+    assert int(sb.status.item()) == 0 and int(pk.n_live.item()) == w.sum()
+    plan, ws = ctx.attn_plan(P, w), sb.ws.cpu().numpy()
+    n_items, n_units, _, n_parts, total, _, _, most = ws[:32].view(np.int32)
+    assert (n_units, n_items, n_parts) == (plan["units"], plan["items"], plan["parts"])
+    at = 256 + -(-plan["max_items"] * 32 // 256) * 256
+    items = ws[256:256 + 32 * n_items].view(np.int32).reshape(-1, 8)
+    units = ws[at:at + 64 * n_units].view(np.int32).reshape(-1, 16)
+    slot_req, slot_s = pk.slot_req.cpu().numpy(), pk.slot_s.cpu().numpy()
+    up = lambda a, b: -(-a // b)
+    tiles, per = [], block_len * G // 128
+    for u, (req, kvh, slot_a, slot_b, t0_a, t0_b, n_tiles, chunks, nvis_a, nvis_b, part, pre, npt, _, win_a, win_b) in enumerate(units):
+        window = w[req] * block_len
+        assert w[req] > 0 and pre == P[req]
+        assert n_tiles == (up(P[req] + window, 128) if resident else up(P[req], 128) + up(window, 128))
+        assert npt == (n_tiles if resident else up(P[req], 128))
+        for slot, t0, nvis, win, kv in ((slot_a, t0_a, nvis_a, win_a, kvh & 0xffff), (slot_b, t0_b, nvis_b, win_b, kvh >> 16)):
+            if slot < 0:
+                assert slot == slot_b and nvis == 0
+                continue
+            assert slot_req[slot] == req and win == (slot_s[slot] + 1) * block_len and t0 in range(0, block_len, 128 // G)
+            assert nvis == (up(P[req] + win, 128) if resident else npt + up(win, 128))
+            tiles.append((slot, t0, kv))
+        own = items[items[:, 0] == u]
+        own = own[np.argsort(own[:, 1])]
+        edges = np.arange(chunks + 1) * n_tiles // chunks
+        assert len(own) == chunks and (own[:, 2] == edges[:-1]).all() and (own[:, 3] == edges[1:]).all() and (own[:, 4] == req).all()
+        assert part == -1 if chunks <= 1 else 0 <= part <= n_parts - chunks
+    assert len(items) == units[:, 7].sum() and len(set(tiles)) == len(tiles) == w.sum() * kv_heads * per
+    assert total == (units[:, 6]).sum() and (most == units[:, 7].max() if n_units else most == 0)
+    # the most costly first, but for one request's few, which come unit by unit
+    if n_units:
+        nv = units[items[:, 0]][:, 8:10]
+        n_ab = np.clip(np.minimum(items[:, 3:4], nv) - items[:, 2:3], 0, None)
+        cost = (6 * n_ab.max(1) + n_ab.min(1) + 1) >> 1
+        if n <= 8 and (w > 0).sum() == 1 and n_items <= 148:
+            assert (np.diff(items[:, 0]) >= 0).all() and (items[:, 1] == np.concatenate([np.arange(c) for c in units[:, 7]])).all()
+        else:
+            assert (np.diff(cost) <= 0).all()
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("max_requests", [1, 2, 9])
 @pytest.mark.parametrize("tiles", [(1 << 19) - 2, (1 << 19) - 1, (1 << 20) + 5, 11423809, 13823826, 16777000])
