@@ -48,7 +48,7 @@ FB_HOST_DEVICE inline bool lm_pairs_of(unsigned long long mask, int m_tiles) { r
 //   hidden 2048, V = 151,552 (14,208 tiles):  +1 -55  -78 -136
 FB_HOST_DEVICE inline bool lm_both_forms(int most_tiles, int n_tiles, int hidden, int sms) {
   const long long tiles = (long long)most_tiles * n_tiles;
-  return most_tiles >= 4 && hidden >= 768 && tiles >= 8ll * sms && tiles * (hidden - 512) >= 1 << 20;
+  return sms >= 2 && most_tiles >= 4 && hidden >= 768 && tiles >= 8ll * sms && tiles * (hidden - 512) >= 1 << 20;
 }
 
 }  // namespace fb

@@ -381,7 +381,7 @@ int launch_lm_head(fb_ctx* ctx, const fb_pack* pk, const void* x, const void* w,
   p.wait_cycles = ctx->wait_cycles;
   // (both forms, since the live rows are only known on the device)
   p.both = lm_both_forms((rows + kLmBM - 1) / kLmBM, p.n_tiles_n, hidden, ctx->num_sms);
-  p.pairs_mask = lm_pairs_mask(p.n_tiles_n, hidden, ctx->num_sms);
+  p.pairs_mask = p.both ? lm_pairs_mask(p.n_tiles_n, hidden, ctx->num_sms) : 0;
   if (int e = cuda_err(ctx, launch_pdl(lm_head_stats_kernel<false>, ctx->num_sms, kLmThreads, kLmSmem, stream, tmX, tmW, p),
                        "lm_head_stats_kernel launch"))
     return e;

@@ -45,7 +45,7 @@ def test_mask_holds_the_rule(rules):
     (3, 592, 4096, 0), (4, 592, 2048, 1), (24, 592, 704, 0), (24, 592, 768, 1), (24, 125, 768, 0), (24, 125, 1024, 1), (8, 250, 1024, 0),
     (8, 250, 2048, 1), (8, 125, 4096, 0), (64, 592, 768, 1), (16, 297, 768, 1), (131072, 1 << 23, 4096, 1)])
 def test_both_forms_only_where_pairs_can_pay(rules, most, n, hidden, both):
-    assert rules.both(most, n, hidden, SMS) == both
+    assert rules.both(most, n, hidden, SMS) == both and not rules.both(most, n, hidden, 1)
 
 
 # the live row tiles that test_gpu_lm_pair.py runs at 297 vocabulary tiles and 16 row tiles of capacity, and the contexts that it
