@@ -139,7 +139,7 @@ __host__ __device__ inline SplitRule split_rule(int total, int units, int target
 // one in full; from three waves on handing out longest first fills half of that in.  The costs (in
 // units of 100 ns; the merge per piece in ns) are a key tile of a pair, of two K/V streams; what an
 // item costs beside its tiles, whole or as a piece; the merge.  They were measured at head_dim 128 when
-// the estimate was written, before the key loop, the epilogue and the start of an item got shorter, and
+// the estimate was written, before the key loop, the start of an item and its end got shorter, and
 // head_dim 64, whose tiles and partials are half the size, uses the same: they rank the candidates, they do
 // not predict a time.  Against always aiming at two items an SM, with the kernel of then: 28,000-token
 // request 72 -> 64 us, 24 requests of 700 to 5,000 tokens 161 -> 151 (not split at all), 8 requests 24.6

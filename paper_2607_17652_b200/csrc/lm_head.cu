@@ -20,7 +20,7 @@
 // accumulator is its own 128 rows again, so the epilogue is the same.  A stage is 32 KB for as many
 // operations as 48 KB before, six stages fit, and a CTA reads 8 KB instead of 12 KB of shared memory
 // per MMA.  What bounds the product is the board's power limit, which is where the saved traffic shows:
-// a step of 64 requests (5,120 rows, V = 151,552, hidden 2048), back to back, 2832 -> 2657 us.
+// a step of 64 requests (5,120 rows, V = 151,552, hidden 2048), back to back, 2781 -> 2616 us.
 // Where which one runs: lm_forms.h, by what the context can hold on the host and by the live rows on the device.
 #include <cudaTypedefs.h>
 

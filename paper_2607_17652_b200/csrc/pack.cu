@@ -2,7 +2,7 @@
 //
 // One launch.  Blocks 0..nb-1 compact the live blocks of all decoding
 // requests into slots and gather tokens / position ids; the last two blocks
-// build the two attention work lists (units, key-axis chunks, longest first)
+// build the two attention work lists (units, key-axis chunks, longest first but for one request's few)
 // from the same per-request state: list 0 for the one-CTA kernel, list 1 (four
 // Q tiles of one request and KV head at a time) for the CTA-pair kernel.
 // Everything is integer work on a few KB.
@@ -10,9 +10,14 @@
 
 namespace fb {
 
-// Threads per block: bound by latency (dependent loads, block barriers), so small batches take
-// small blocks: call in us with 256 / 512 / 1024 threads, 1 request 5.5 / 6.0 / 7.0, 8 requests 5.9 /
-// 6.6 / 7.6, 24 requests 8.6 / 8.0 / 8.9, 128 requests 19.0 / 16.9 / 17.2 (measured before build_sched got shorter).
+// Threads per block: bound by latency (dependent loads, block barriers), so small batches take small blocks
+// (1024 threads do not fit their tables into static shared memory).  Call in us, back to back:
+//   requests        1    2    4    8    9   16   24   32   64  128
+//   128 threads   4.4  4.8  5.0  5.8
+//   256           4.4  4.7  5.1  5.7  5.5  5.9  6.2  8.0  7.6 10.7
+//   512           4.4  5.2  5.6  6.3  6.0  6.4  6.6  7.4  7.7 10.8
+// The line lies at 8 because build_sched changes its way there: every warp for itself up to 8 requests, a thread a
+// request above (16 requests 6.9 the first way, 6.4 the other; 24: 7.8, 6.6; 32: 10.6, 7.4).
 constexpr int kPackThreads = 512, kPackThreadsSmall = 256, kPackSmallRequests = 8;
 constexpr int kSlotsPerBlock = 32;
 constexpr int kPackLongPages = 1 << 20;   // (kLong: with two pages a key tile, ranges stay below 2^20 key tiles here)
@@ -143,11 +148,11 @@ __device__ __forceinline__ AttnUnit make_unit(const PackParams& p, const ReqGeom
 // cut into the same chunks; an item names record 2u.
 //
 // Bound by the chain of dependent steps in one block.  Up to kPackSmallRequests every warp holds all of them, a
-// lane each, and forms sums, split and bases for itself, without a barrier; above, a thread holds a request
-// (a lane each up to 32 requests: 24 requests 9.8 us, a thread each 7.7).  Call in us, back to back, before and with
-// this and the quotients by reciprocal: one request of 3,000 tokens 5.7 / 4.2, 8 requests 6.1 / 5.4, 24 requests
-// 8.2 / 7.7, 64 requests 9.7 to 11 / 8.2 to 9.4, in 8 bits 10 to 13 / 8.8, 128 requests 14 to 18 / 12.4 to 16.
-// Steps: a toy request 23.3 / 21.3, one request with four layers 110.1 / 107.5, a 28,000-token one 83.2 / 82.2.
+// lane each, and forms sums, split and bases for itself, without a barrier; above, a thread holds a request.
+// Call in us, back to back, before and with this, the quotients by reciprocal and the unit records in registers: one
+// request of 3,000 tokens 5.7 / 4.0, 8 requests 6.0 / 5.2, 24 requests 7.4 / 6.4, 64 requests 9.3 / 7.6, in 8 bits
+// 9.6 / 7.8, 128 requests 13.3 / 10.6, 600 requests 46 / 37.  Steps with the first two: a toy request 23.5 / 21.8, one
+// request with four layers 105.8 / 102.4, a 28,000-token one 83.1 / 80.2.
 template <int T, bool kLong>
 __device__ void build_sched(const PackParams& p, const int list) {
   constexpr unsigned kAll = 0xffffffffu;

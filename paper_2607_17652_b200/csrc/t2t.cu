@@ -246,8 +246,9 @@ __global__ void __launch_bounds__(128) t2t_update_kernel(const UpdParams p) {
   const int lane = threadIdx.x & 31;
   // The kernel before is the row pass or the merge of the LM head, of the same call, and releases this one when it
   // has waited itself: slots and state are older and read ahead of the wait, the first 32 tokens of the block too.
-  // What is left behind it is one round of loads.  Steps in us, before / with it: a toy request 23.7 / 23.4, one
-  // request with four layers 113.6 / 110.0, a 28,000-token one 84.3 / 83.4, 8 requests 85.8 / 85.4.
+  // What is left behind it is one round of loads.  Both kernels in us, back to back, before / with it: V = 1024: 24
+  // requests 8.5 / 7.8, 64 requests 12.7 / 11.9, 128 requests 21.5 / 20.5; V = 8,000: 64 requests 23.0 / 21.7; V = 151,552:
+  // one request 10.4 / 9.9, 64 requests 246.0 / 245.7.
   int n_live = 0, r = 0, s0 = 0, g = 0, x0 = 0;
   int32_t* tok = p.tokens;
   if (slot < p.max_slots) {
