@@ -169,3 +169,31 @@ def test_pairs_give_up_report_and_recover():
         a1, c1, action1 = one_cta(x, w, blocks)
         rows = blocks * BL
         assert status == 0 and torch.equal(a[:rows], a1) and torch.equal(c[:rows], c1) and torch.equal(action[:rows], action1)
+
+
+def test_form_follows_the_live_rows_under_a_graph():
+    """One captured pack and head call, replayed while the live rows change: either form, the same bits as direct calls."""
+    x, w = draw(1088, V, REQUESTS * WMAX * BL, 6)
+    h = Head(REQUESTS, V)
+    direct = {blocks: h.run(x, w, blocks) for blocks in (8, 20, 49, 4)}
+    st = B.DeviceState.from_numpy(DEV, np.ones(REQUESTS, np.int32), *(np.zeros(REQUESTS, np.int32) for _ in range(3)),
+                                  np.full((REQUESTS, 8 * BL), V - 1, np.int32), np.zeros((REQUESTS, WMAX), np.uint8),
+                                  np.zeros((REQUESTS, 4), np.int32))
+    pk, sb = B.PackBuffers.alloc(h.ctx, DEV), B.StepBuffers(h.ctx, DEV)
+
+    def step(stream):
+        B.fb_pack_wavefronts(h.ctx, st, pk, sb.ws, sb.status, stream)
+        B.fb_lm_head_t2t(h.ctx, pk, x, w, st, sb.argmax, sb.conf, sb.action, sb.slot_stats, h.ws, sb.status, stream)
+
+    side = torch.cuda.Stream()
+    graph = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, stream=side):
+        step(side.cuda_stream)
+    for blocks, (a, c, _, action, _) in direct.items():
+        live = np.array([min(WMAX, max(0, blocks - WMAX * r)) for r in range(REQUESTS)], np.int32)
+        st.R.copy_(torch.from_numpy(live))
+        st.tokens.fill_(V - 1)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert int(sb.status.item()) == 0 and torch.equal(sb.argmax, a) and torch.equal(sb.conf, c) and torch.equal(sb.action, action)
